@@ -17,6 +17,7 @@
 #include "gpp_internal.h"
 #include "gpp_terms_f32.cuh"
 #include "gpp_terms_f64.cuh"
+#include "gpp_terms_fix.cuh"
 
 namespace gpp {
 
@@ -97,8 +98,96 @@ __device__ __noinline__ void f32_general_pair(int B, int64_t G, int nocc,
 #ifndef GPP_F32_MAXNREG
 #define GPP_F32_MAXNREG 72
 #endif
-template <int W, bool F32>
-__device__ __forceinline__ void batched_body(const BatchInst* __restrict__ inst, int ninst,
+// One (igp, ig) pair of the FP64 sum in FP64 arithmetic, by the fast or the general form, for
+// the warps outside the split-integer form's range. Not inlined, so that its registers do
+// not count against the split-integer band loop.
+template <int W, bool FAST>
+__device__ __noinline__ void f64_pair(int B, int64_t G, int nocc, const double2* __restrict__ aqsn,
+                                      const double2* __restrict__ am,
+                                      const BandEntry* __restrict__ bt, bool live, double2 w,
+                                      double2 I, double sx2, double* tacc) {
+  double a[4 * W];
+#pragma unroll
+  for (int k = 0; k < 4 * W; ++k) a[k] = tacc[k];
+  band_loop<W, FAST>(B, G, nocc, aqsn, am, bt, live, w.x, w.y, fma(I.x, w.x, -I.y * w.y),
+                     fma(I.x, w.y, I.y * w.x), sx2, a);
+#pragma unroll
+  for (int k = 0; k < 4 * W; ++k) tacc[k] = a[k];
+}
+
+// The FP64 sum's tiles: every warp of a pass takes the split-integer form where its inputs
+// allow (gpp_terms_fix.cuh), else the FP64 fast or general form. smem: fix_smem_bytes.
+template <int W>
+__device__ __forceinline__ void f64_body(const BatchInst* __restrict__ inst, int ninst,
+                                         int64_t t_begin, int64_t ntiles, int igpt,
+                                         unsigned long long* counter,
+                                         double* __restrict__ partials) {
+  __shared__ double red[(256 / 32) * 4 * kMaxNw];
+  __shared__ long long s_t;
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  double acc[4 * W];   // the thread's tile sums, in local memory (touched once per pair)
+  for (;;) {
+    if (threadIdx.x == 0) s_t = t_begin + static_cast<long long>(atomicAdd(counter, 1ULL));
+    __syncthreads();
+    const int64_t t = s_t;
+    __syncthreads();
+    if (t >= ntiles) break;
+    int ilo = 0, ihi = ninst - 1;  // instance holding tile t (tile ranges are sorted)
+    while (ilo < ihi) {
+      const int mid = (ilo + ihi) >> 1;
+      if (__ldg(&inst[mid].tile_end) > t)
+        ihi = mid;
+      else
+        ilo = mid + 1;
+    }
+    const BatchInst& d = inst[ilo];
+    const int B = d.B, nocc = d.nocc;
+    const int64_t G = d.G;
+    const int64_t local = t - d.tile0;
+    const int64_t igt = local / d.P;
+    const int64_t p = local - igt * d.P;
+    const bool col_ok = d.colg[p] >= 0;
+    const bool x_fast = d.flags[0] == 0;
+    const FixInfo fix = *reinterpret_cast<const FixInfo*>(d.flags + kFlagFix);
+    const double* xrange = reinterpret_cast<const double*>(d.flags + kFlagRange);
+    const double2* am = d.am + p * B;
+#pragma unroll
+    for (int k = 0; k < 4 * W; ++k) acc[k] = 0.0;
+    for (int j = 0; j < igpt; ++j) {
+      const int64_t ig = (igt * igpt + j) * blockDim.x + threadIdx.x;
+      const bool live = ig < G && col_ok;
+      if (!__any_sync(0xffffffffu, live)) continue;   // a dead column, or past G
+      double2 w = make_double2(1.0, 0.5);  // inert lane: in every range, finite terms, zero weight
+      double2 I = make_double2(0.0, 0.0);
+      if (live) {
+        w = ldg2(d.wt + p * G + ig);
+        I = ldg2(d.eps + p * G + ig);
+      }
+      const double2* an = d.aqsn + (live ? ig : 0);
+      const double wabs2 = fma(w.x, w.x, w.y * w.y);
+      if (fix.ok) {
+        double xmax = xrange[kMaxNw];
+        for (int k = 1; k < W; ++k) xmax = fmax(xmax, xrange[kMaxNw + k]);
+        if (__all_sync(0xffffffffu, fix_lane(w, wabs2, fix.E, xmax) || !live) &&
+            fix_band_loop<W>(B, G, nocc, an, am, d.bt, live, w, live ? d.wt + p * G + ig : d.wt, I,
+                             fix.E, xrange, dyn_smem, acc))
+          continue;
+      }
+      // the FP64 fast form's conditions, with the partial fractions' bound on x / |w|
+      const bool fast_lane = w.x >= 0.0 && gt_nonneg(wabs2, kFastWabs2Lo) &&
+                             lt_nonneg(wabs2, kFastWabs2Hi) &&
+                             !lt_nonneg(wabs2, pf_wabs2_min(d.flags));
+      if (__all_sync(0xffffffffu, fast_lane || !live) && x_fast)
+        f64_pair<W, true>(B, G, nocc, an, am, d.bt, live, w, I, 0.0, acc);
+      else
+        f64_pair<W, false>(B, G, nocc, an, am, d.bt, live, w, I, d.sx2, acc);
+    }
+    block_partials<4 * W>(acc, red, partials + t * 4 * W);
+  }
+}
+
+template <int W>
+__device__ __forceinline__ void f32_body(const BatchInst* __restrict__ inst, int ninst,
                                              int64_t t_begin, int64_t ntiles, int igpt,
                                              unsigned long long* counter,
                                              double* __restrict__ partials) {
@@ -113,7 +202,7 @@ __device__ __forceinline__ void batched_body(const BatchInst* __restrict__ inst,
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   float* const s_slots = reinterpret_cast<float*>(dyn_smem);
   const int tile_n = blockDim.x * igpt;
-  const int sort_n = F32 ? pow2_ceil(tile_n) : 0;
+  const int sort_n = pow2_ceil(tile_n);
   float* const s_key = s_slots;
   int* const s_pos = reinterpret_cast<int*>(
       s_slots + max(F32Slots<W>::kFloats * static_cast<int>(blockDim.x), sort_n));
@@ -142,13 +231,8 @@ __device__ __forceinline__ void batched_body(const BatchInst* __restrict__ inst,
     const int64_t igt = local / d.P;
     const int64_t p = local - igt * d.P;
     const bool col_ok = d.colg[p] >= 0;
-    const bool x_fast = d.flags[0] == 0 && (!F32 || d.flags[2] == 0);
-    // FP64: the partial fractions' bound on x / |w| (gpp_device.cuh)
-    const double wabs2_pf = F32 ? 0.0 : pf_wabs2_min(d.flags);
-    double acc[4 * W];                 // FP64 sums (GPP_FP64)
-#pragma unroll
-    for (int k = 0; k < 4 * W; ++k) acc[k] = 0.0;
-    if (F32) {
+    const bool x_fast = d.flags[0] == 0 && d.flags[2] == 0;
+    {
       if (threadIdx.x == 0) s_bt64 = d.bt;
       // With at least kSortBands bands, the G-vectors of each pass over the tile (blockDim.x
       // of them, when that is a power of two; else the whole tile) are taken in order of
@@ -179,18 +263,18 @@ __device__ __forceinline__ void batched_body(const BatchInst* __restrict__ inst,
       for (int k = 0; k < 2 * W; ++k) tpair[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     for (int j = 0; j < igpt; ++j) {
-      // F32: a padding position (>= tile_n, key +inf like an inert one) can sort into the
+      // a padding position (>= tile_n, key +inf like an inert one) can sort into the
       // first tile_n slots when the whole tile is sorted; it is inert
-      const int q = F32 ? s_pos[j * blockDim.x + threadIdx.x] : 0;
-      const int64_t ig = F32 ? igt * tile_n + q : (igt * igpt + j) * blockDim.x + threadIdx.x;
-      const bool live = (!F32 || q < tile_n) && ig < G && col_ok;
+      const int q = s_pos[j * blockDim.x + threadIdx.x];
+      const int64_t ig = igt * tile_n + q;
+      const bool live = q < tile_n && ig < G && col_ok;
       double2 w = make_double2(0.5, 1.0);  // inert lane: finite terms, zero weight
       if (live) w = ldg2(d.wt + p * G + ig);
       const double wabs2 = fma(w.x, w.x, w.y * w.y);
       const bool fast_lane = w.x >= 0.0 && gt_nonneg(wabs2, kFastWabs2Lo) &&
-                             lt_nonneg(wabs2, kFastWabs2Hi) && !lt_nonneg(wabs2, wabs2_pf);
+                             lt_nonneg(wabs2, kFastWabs2Hi);
       const bool fast = __all_sync(0xffffffffu, fast_lane) && x_fast;
-      if (F32 && fast) {
+      if (fast) {
         band_loop_f32<W>(B, G, nocc, d.aqsn32 + (live ? ig : 0), d.am32 + p * B, d.bt32,
                          &s_bt64, w, live, s_slots);
         // I w in FP64 once per pair (w re-read from the thread's slot, I from memory, so
@@ -207,45 +291,40 @@ __device__ __forceinline__ void batched_body(const BatchInst* __restrict__ inst,
       if (live) I = ldg2(d.eps + p * G + ig);
       const double Iwr = fma(I.x, w.x, -I.y * w.y);
       const double Iwi = fma(I.x, w.y, I.y * w.x);
-      if (F32) {  // the general path in FP64, folded into the tile pairs
-        f32_general_pair<W>(B, G, nocc, d.aqsn + (live ? ig : 0), d.am + p * B, d.bt, live,
-                            w.x, w.y, Iwr, Iwi, d.sx2, tpair);
-      } else if (fast) {
-        band_loop<W, true>(B, G, nocc, d.aqsn + (live ? ig : 0), d.am + p * B, d.bt, live,
-                           w.x, w.y, Iwr, Iwi, 0.0, acc);
-      } else {
-        band_loop<W, false>(B, G, nocc, d.aqsn + (live ? ig : 0), d.am + p * B, d.bt, live,
-                            w.x, w.y, Iwr, Iwi, d.sx2, acc);
+      // the general path in FP64, folded into the tile pairs
+      f32_general_pair<W>(B, G, nocc, d.aqsn + (live ? ig : 0), d.am + p * B, d.bt, live, w.x, w.y,
+                          Iwr, Iwi, d.sx2, tpair);
+    }
+    float hi[4 * W], lo[4 * W];
+#pragma unroll
+    for (int qd = 0; qd < W; ++qd) {
+      float4 th = tpair[qd], tl = tpair[W + qd];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        hi[4 * qd + i] = quad_elem(th, i);
+        lo[4 * qd + i] = quad_elem(tl, i);
       }
     }
-    if (F32) {
-      float hi[4 * W], lo[4 * W];
-#pragma unroll
-      for (int qd = 0; qd < W; ++qd) {
-        float4 th = tpair[qd], tl = tpair[W + qd];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          hi[4 * qd + i] = quad_elem(th, i);
-          lo[4 * qd + i] = quad_elem(tl, i);
-        }
-      }
-      block_pairs<4 * W>(hi, lo, reinterpret_cast<float2*>(red),
-                         reinterpret_cast<float2*>(partials) + t * 4 * W);
-    }
-    else
-      block_partials<4 * W>(acc, red, partials + t * 4 * W);
+    block_pairs<4 * W>(hi, lo, reinterpret_cast<float2*>(red),
+                       reinterpret_cast<float2*>(partials) + t * 4 * W);
   }
 }
 
-// The two instantiations of the main kernel. FP64: one 256-thread CTA's worth of registers
-// per SM at most (the FP64 band loop takes ~160 registers). FP32-bulk: held to
+// The two instantiations of the main kernel. FP64: two 256-thread CTAs' worth of registers per
+// SM (128 per thread), which the split-integer band loop fits without spilling; the FP64 band
+// loop runs as fast at 128 registers as at its unconstrained 166. FP32-bulk: held to
 // GPP_F32_MAXNREG registers (80 for nw > 5, whose band loop would spill at fewer).
+//
+// Measured (GB300, main sum with the split-integer form against the FP64 form alone):
+// B = 512, P = 819, G = 16384, nw = 3: 174.1 against 692.8 ms; B = 128, P = 410, G = 8192:
+// 11.68 against 44.43 ms; B = 32, P = 64, G = 512: 0.216 against 0.330 ms. Bound now: the
+// instruction issue of the integer and FP32 pipes (FP64 pipe 60% busy).
 template <int W>
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(256, 2)
     gpp_batched_kernel_f64(const BatchInst* __restrict__ inst, int ninst, int64_t t_begin,
                            int64_t ntiles, int igpt, unsigned long long* counter,
                            double* __restrict__ partials) {
-  batched_body<W, false>(inst, ninst, t_begin, ntiles, igpt, counter, partials);
+  f64_body<W>(inst, ninst, t_begin, ntiles, igpt, counter, partials);
 }
 
 template <int W>
@@ -253,7 +332,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(W <= 5 ? GPP_F32_MAXNREG : 80
     gpp_batched_kernel_f32(const BatchInst* __restrict__ inst, int ninst, int64_t t_begin,
                            int64_t ntiles, int igpt, unsigned long long* counter,
                            double* __restrict__ partials) {
-  batched_body<W, true>(inst, ninst, t_begin, ntiles, igpt, counter, partials);
+  f32_body<W>(inst, ninst, t_begin, ntiles, igpt, counter, partials);
 }
 
 // One CTA per instance: the instance's tile partials summed in tile order, then a tree.
@@ -316,7 +395,7 @@ const void* batched_kernel_ptr(int nw, bool f32) {
 size_t batched_smem_bytes(int threads, int nw, bool f32, int igpt) {
   // F32Slots<nw>::kFloats floats per thread (at least as many as the sort keys, which alias
   // them), then the sorted positions
-  if (!f32) return 0;
+  if (!f32) return fix_smem_bytes(threads, nw < kFixMaxGroup ? nw : kFixMaxGroup);
   const size_t sort_n = static_cast<size_t>(pow2_ceil(threads * igpt));
   const size_t slots = static_cast<size_t>(threads) * (8 * nw + 4);
   return (slots > sort_n ? slots : sort_n) * sizeof(float) + sort_n * sizeof(int);
@@ -357,7 +436,7 @@ cudaError_t launch_batched_main(const BatchInst* inst, int ninst, int64_t ntiles
     gpp_batched_kernel_f32<WV><<<grid, threads, smem, s>>>(inst, ninst, t_begin, ntiles, igpt,    \
                                                            counter, partials);                    \
   else                                                                                            \
-    gpp_batched_kernel_f64<WV><<<grid, threads, 0, s>>>(inst, ninst, t_begin, ntiles, igpt,       \
+    gpp_batched_kernel_f64<WV><<<grid, threads, smem, s>>>(inst, ninst, t_begin, ntiles, igpt,       \
                                                         counter, partials)
   switch (nw) {
     case 1: GPP_BATCHED_LAUNCH(1); break;

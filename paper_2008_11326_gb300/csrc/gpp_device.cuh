@@ -24,11 +24,23 @@ constexpr double kFastWabs2Hi = 62499.0;
 
 constexpr int kMaxNw = 8;
 
-// One (band, iw) entry of the FP64 band table: x = wx_array[b][iw], x^2 and -x/2 (hi.x pads
-// the entry to 32 bytes).
+// One (band, iw) entry of the FP64 band table: x = wx_array[b][iw], x^2, and x split into
+// integers and floats for the split-integer form (fix_x in gpp_terms_fix.cuh; zeros when the
+// instance's frequencies are outside its range).
 struct alignas(32) BandEntry {
   double2 lo;  // x, x^2
-  double2 hi;  // 0, -x/2
+  int4 fx;
+};
+
+// What the gather kernel tells the main kernel about an instance's frequencies, beside the
+// flags (at kFlagFix): whether they fit the split-integer form, and with which binary scale.
+struct FixInfo {
+  int ok, E;
+};
+
+template <int V>
+struct IntTag {
+  static constexpr int value = V;
 };
 
 // The FP32 band table: per band, f32_band_quads(W) float4: x_hi[0..W-1] (each frequency
@@ -41,10 +53,17 @@ __host__ __device__ constexpr int f32_band_quads(int W) { return 2 * f32_half_qu
 
 // Flags written by the gather kernel: [0] some wx < 0 or NaN, [1] bad index count,
 // [2] some |wx| >= kFp32MaxX or NaN (the FP32 decision margin assumes smaller x); from int
-// kFlagXmax on, the bits of max |wx| as a 64-bit integer. kFlagBytes in all.
+// kFlagXmax on, the bits of max |wx| as a 64-bit integer (kFlagBytes so far, cleared before
+// the gather); then, written whole by the gather, a FixInfo at int kFlagFix and, as doubles
+// from int kFlagRange on, min wx of every frequency and max wx of every frequency (kMaxNw
+// each). kFlagAllBytes in all.
 constexpr double kFp32MaxX = 1.0e4;
 constexpr int kFlagXmax = 4;
 constexpr size_t kFlagBytes = 4 * sizeof(int) + sizeof(unsigned long long);
+constexpr int kFlagFix = 8;
+constexpr int kFlagRange = 16;
+constexpr size_t kFlagAllBytes = kFlagRange * sizeof(int) + 2 * kMaxNw * sizeof(double);
+static_assert(kFlagAllBytes <= 256, "the flags fill one aligned workspace segment");
 
 // The FP64 fast paths (forward and adjoint) take the asxtemp terms in partial fractions,
 // M w / (A S) = (M/A - M/S) / 2, whose subtraction loses about log2(1 + x / |w|) bits where

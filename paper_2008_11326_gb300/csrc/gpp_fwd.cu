@@ -32,11 +32,15 @@
 #include "gpp_device.cuh"
 #include "gpp_internal.h"
 #include "gpp_terms_f64.cuh"
+#include "gpp_terms_fix.cuh"
 
 namespace gpp {
 
 namespace {
 
+// Band count up to which the gather offers the split-integer form (each of its blocks reads
+// all the frequencies).
+constexpr int64_t kFixMaxBands = 16384;
 
 // Global column of local column p, or -1 if it contributes nothing. Counts indices that
 // are outside their arrays (the sentinel indinv[k] == G is legitimate).
@@ -66,7 +70,7 @@ __global__ void gpp_prep_kernel(int64_t B, int64_t G, int64_t P, int W,
                                 const int32_t* __restrict__ indinv,
                                 const double* __restrict__ wx, int* flags, int* colg,
                                 BandEntry* bt, double2* am, float4* bt32, float2* am32,
-                                BatchInst* desc_out, const BatchInst desc) {
+                                bool want_fix, BatchInst* desc_out, const BatchInst desc) {
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const int64_t tid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (desc_out && tid == 0) *desc_out = desc;
@@ -83,9 +87,54 @@ __global__ void gpp_prep_kernel(int64_t B, int64_t G, int64_t P, int W,
     am[i] = v;
     if (am32) am32[i] = make_float2(static_cast<float>(v.x), static_cast<float>(v.y));
   }
+  // For the FP64 sum's split-integer form, every block that writes band-table entries forms
+  // the ranges of the frequencies itself (a few KB from L2; 8 / W warps share a frequency), so
+  // that the table's split form and the flags need no second launch.
+  FixInfo fix{0, 0};
+  if (want_fix && static_cast<int64_t>(blockIdx.x) * blockDim.x < B * W) {
+    __shared__ double s_lo[8], s_hi[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;   // 8 warps, W <= 8
+    const int iw = warp % W, part = warp / W, parts = 8 / W;
+    if (part < parts) {
+      double lo = INFINITY, hi = -INFINITY;
+#pragma unroll 4
+      for (int64_t b = part * 32 + lane; b < B; b += parts * 32) {
+        const double x = wx[b * W + iw];
+        lo = x >= 0.0 ? fmin(lo, x) : -INFINITY;   // a negative or NaN frequency: out of range
+        hi = fmax(hi, x);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      }
+      if (lane == 0) {
+        s_lo[warp] = lo;
+        s_hi[warp] = hi;
+      }
+    }
+    __syncthreads();
+    double lo = s_lo[0], hi = s_hi[0];
+    for (int k = 1; k < parts * W; ++k) {
+      lo = fmin(lo, s_lo[k]);
+      hi = fmax(hi, s_hi[k]);
+    }
+    fix = fix_info(lo, hi);
+    if (blockIdx.x == 0 && threadIdx.x < W) {
+      double* range = reinterpret_cast<double*>(flags + kFlagRange);
+      double l = s_lo[threadIdx.x], h = s_hi[threadIdx.x];
+      for (int k = 1; k < parts; ++k) {
+        l = fmin(l, s_lo[k * W + threadIdx.x]);
+        h = fmax(h, s_hi[k * W + threadIdx.x]);
+      }
+      range[threadIdx.x] = l;
+      range[kMaxNw + threadIdx.x] = h;
+    }
+  }
+  if (tid == 0) *reinterpret_cast<FixInfo*>(flags + kFlagFix) = fix;
   for (int64_t i = tid; i < B * W; i += stride) {
     double x = wx[i];
-    bt[i] = BandEntry{make_double2(x, x * x), make_double2(0.0, -0.5 * x)};
+    bt[i] = BandEntry{make_double2(x, x * x), fix.ok ? fix_x(x, fix.E) : make_int4(0, 0, 0, 0)};
     if (!(x >= 0.0)) flags[0] = 1;
     if (!(fabs(x) < kFp32MaxX)) flags[2] = 1;
     // max |wx|: non-negative doubles order as their bit patterns
@@ -156,6 +205,7 @@ cudaError_t launch_prep(const gpp_problem& p, const FwdPlan& plan, char* ws, boo
                            p.ncouls, p.number_bands, 0, p.ncouls, s);
     if (e != cudaSuccess) return e;
   }
+  const bool want_fix = !fp32 && p.number_bands <= kFixMaxBands;
   const int64_t work = p.ngpown * p.number_bands + p.number_bands * p.nw + p.ngpown;
   int64_t blocks = (work + 255) / 256;
   if (blocks < 1) blocks = 1;
@@ -167,7 +217,7 @@ cudaError_t launch_prep(const gpp_problem& p, const FwdPlan& plan, char* ws, boo
       reinterpret_cast<BandEntry*>(ws + plan.off_bt), reinterpret_cast<double2*>(ws + plan.off_am),
       fp32 ? reinterpret_cast<float4*>(ws + plan.off_bt32) : nullptr,
       fp32 ? reinterpret_cast<float2*>(ws + plan.off_am32) : nullptr,
-      desc ? reinterpret_cast<BatchInst*>(ws + plan.off_desc) : nullptr, desc ? *desc : BatchInst());
+      want_fix, desc ? reinterpret_cast<BatchInst*>(ws + plan.off_desc) : nullptr, desc ? *desc : BatchInst());
   return cudaGetLastError();
 }
 

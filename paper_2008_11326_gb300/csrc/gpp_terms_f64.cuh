@@ -54,7 +54,7 @@ __device__ __forceinline__ void band_terms_fast(double Kr, double Ki, double Kwr
 //   Mw = (-Im M Im w, Re M Im w)     so that M conj(A) = (Re M Ar + Mw.re, Im M Ar + Mw.im)
 //   P1 = (-Im M2 Im w^2, Re M2 Im w^2)  so that M2 conj(C) = (Re M2 Yr + P1.re, Im M2 Yr + P1.im)
 //   P2 = Mw / 2 (halved on the integer pipe) so that M (-conj(S)/2) = (Re M Yr + P2.re, Im M Yr + P2.im)
-// with Yr = x^2 - Re w^2 (branch 1) or -(x + Re w)/2 (branch 2); one reciprocal
+// with Yr = Re C = Ar Sr + (Im w)^2 (branch 1) or -(x + Re w)/2 (branch 2); one reciprocal
 // r = 1/(|A|^2 |S|^2) serves the three denominators (gpp_fwd.cu).
 struct BandK {
   double Kr, Ki, K2r, K2i, Kwr, Kwi, P1r, P1i, P2r, P2i;  // M, M2, Mw, P1, P2
@@ -67,12 +67,11 @@ template <int W, bool OCC>
 __device__ __forceinline__ void band_terms_general(const BandK& k,
                                                    const BandEntry* __restrict__ btb,
                                                    double wr, double wi2, double wabs2,
-                                                   double mw2r, double wrh, double sx2,
+                                                   double sx2,
                                                    double (&acc)[4 * W]) {
 #pragma unroll
   for (int iw = 0; iw < W; ++iw) {
-    const double2 xlo = __ldg(&btb[iw].lo);
-    const double x = xlo.x, x2 = xlo.y, xh = __ldg(&btb[iw].hi.y);
+    const double x = __ldg(&btb[iw].lo.x);
     const double Ar = x - wr;                 // A = x - w = (Ar, -Im w)
     const double A2 = fma(Ar, Ar, wi2);       // |wdiff|^2
     const double Sr = x + wr;
@@ -95,7 +94,7 @@ __device__ __forceinline__ void band_terms_general(const BandK& k,
                        (c1 ? gt_nonneg(wabs2 * wabs2 * r, sx2)
                            : gt_nonneg(wabs2, 4.0 * sx2 * S2));
       coef = cut ? 0.0 : coef;
-      const double Yr = (c1 ? x2 : xh) + (c1 ? mw2r : wrh);
+      const double Yr = fma(c1 ? Ar : -0.5, Sr, c1 ? wi2 : 0.0);
       const double ur = fma(c1 ? k.K2r : k.Kr, Yr, c1 ? k.P1r : k.P2r);
       const double ui = fma(c1 ? k.K2i : k.Ki, Yr, c1 ? k.P1i : k.P2i);
       acc[4 * iw + 2] = fma(ur, coef, acc[4 * iw + 2]);
@@ -113,8 +112,8 @@ __device__ __forceinline__ void band_range(int b0, int b1, int64_t G,
                                            const double2* __restrict__ an_ptr,
                                            const double2* __restrict__ am_ptr,
                                            const BandEntry* __restrict__ bt, bool live, double wr,
-                                           double wi, double wi2, double wabs2, double mw2r,
-                                           double w2i, double wrh, double sx2,
+                                           double wi, double wi2, double wabs2, double w2i,
+                                           double sx2,
                                            double (&acc)[4 * W]) {
 #pragma unroll 1
   for (int b = b0; b < b1; ++b) {
@@ -139,8 +138,8 @@ __device__ __forceinline__ void band_range(int b0, int b1, int64_t G,
     k.P1i = k.K2r * w2i;
     k.P2r = half_alu(Kwr);
     k.P2i = half_alu(Kwi);
-    band_terms_general<W, OCC>(k, bt + static_cast<int64_t>(b) * W, wr, wi2, wabs2, mw2r, wrh,
-                               sx2, acc);
+    band_terms_general<W, OCC>(k, bt + static_cast<int64_t>(b) * W, wr, wi2, wabs2, sx2,
+                               acc);
   }
 }
 
@@ -156,14 +155,12 @@ __device__ __forceinline__ void band_loop(int B, int64_t G, int nocc,
                                           double sx2, double (&acc)[4 * W]) {
   const double wi2 = wi * wi;
   const double wabs2 = fma(wr, wr, wi2);
-  const double mw2r = -fma(wr, wr, -wi2);   // -Re w^2
   const double w2i = 2.0 * wr * wi;         // Im w^2
-  const double wrh = -0.5 * wr;
   double t[4 * W];
 #pragma unroll
   for (int k = 0; k < 4 * W; ++k) t[k] = 0.0;
-  band_range<W, FAST, true>(0, nocc, G, an_ptr, am_ptr, bt, live, wr, wi, wi2, wabs2, mw2r, w2i,
-                            wrh, sx2, t);
+  band_range<W, FAST, true>(0, nocc, G, an_ptr, am_ptr, bt, live, wr, wi, wi2, wabs2, w2i, sx2,
+                            t);
   if (FAST) {   // the occupied bands' asxtemp: (their achtemp - sum M/S) / 2
 #pragma unroll
     for (int iw = 0; iw < W; ++iw) {
@@ -172,8 +169,8 @@ __device__ __forceinline__ void band_loop(int B, int64_t G, int nocc,
     }
   }
   if (nocc < B)
-    band_range<W, FAST, false>(nocc, B, G, an_ptr, am_ptr, bt, live, wr, wi, wi2, wabs2, mw2r,
-                               w2i, wrh, sx2, t);
+    band_range<W, FAST, false>(nocc, B, G, an_ptr, am_ptr, bt, live, wr, wi, wi2, wabs2, w2i,
+                               sx2, t);
 #pragma unroll
   for (int k = 0; k < 2 * W; ++k) {   // acc += Iw t, per complex value
     const double tr = t[2 * k], ti = t[2 * k + 1];

@@ -1,0 +1,101 @@
+"""GPU parity of the FP64 sum's split-integer form (gpp_terms_fix.cuh) at the edges of its
+range and of its loops, against the CPU oracle.
+
+Tolerance, derived before the first run: a pair's sum carries at most about 2^-51 of its root
+mean square, pairs are independent, and the final FP64 additions add a few 2^-53; so every
+output lies within 2^-48 (3.6e-15) of the root mean square of its kind, whatever cancels.
+"""
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2008_11326_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+TOL = 2.0 ** -48
+
+
+@pytest.fixture(scope="module")
+def gpp():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2008_11326_gb300 import gpp as g
+    return g
+
+
+def check(gpp, prob, occ="all", **opts):
+    import torch
+    dp = gpp.DeviceProblem.from_host(prob, device="cuda")
+    got = gpp.sigma(dp, occ_mode=occ, **opts)
+    torch.cuda.synchronize()
+    ref = oracle.sigma(prob, occ_mode=0 if occ == "all" else 1)
+    for g, r in zip(got, ref):
+        rms = np.sqrt(np.mean(np.abs(r) ** 2))
+        err = np.max(np.abs(g.cpu().numpy() - r))
+        assert err <= TOL * rms, (err / rms, prob.shape)
+
+
+# bands: one, around the FP32 low sums (16), the staged weights (64), the modular sums (1024);
+# G-vectors around a warp and a tile; every frequency group (1, 2, 3, 2+2, 3+2, 3+3, 3+2+2, 3+3+2)
+@pytest.mark.parametrize("shape", [(1, 1, 1, 1), (2, 33, 3, 2), (15, 127, 5, 3), (16, 128, 4, 4),
+                                   (17, 129, 4, 5), (63, 511, 3, 6), (64, 513, 3, 7),
+                                   (65, 130, 3, 8), (1023, 40, 2, 3), (1025, 40, 2, 3),
+                                   (2049, 33, 1, 1)])
+def test_loop_edges(gpp, shape):
+    B, G, P, W = shape
+    prob = inputs.make_problem(B, 2, G, P, W, seed=B + G)
+    check(gpp, prob)
+    check(gpp, prob.replace(nvband=B // 2), occ="occupied")
+
+
+# largest frequency at the edge of each binary scale (0.75 2^E) and past the last one; |w| from
+# below 2^(E-7) to above 1.375 2^E - max x
+@pytest.mark.parametrize("xmax", [0.4, 3.0, 3.0001, 6.0, 12.0, 23.9, 47.999, 48.0, 48.001, 90.0])
+def test_frequency_and_pole_range(gpp, xmax):
+    rng = np.random.Generator(np.random.PCG64(int(xmax * 1000)))
+    prob = inputs.make_problem(20, 2, 320, 4, 3, seed=7)
+    wx = rng.uniform(0.0, xmax, size=prob.wx_array.shape)
+    wx[3, 1] = xmax
+    wx[4, 0] = 0.0
+    E = 2
+    while E < 6 and xmax > 0.75 * 2 ** E:
+        E += 1
+    wt = prob.wtilde_array.copy()
+    lo, hi = 2.0 ** (E - 7), 1.375 * 2 ** E - xmax
+    for p in range(4):   # segments of one warp each, just inside and just outside the bounds
+        for k, mod in enumerate((lo * 1.0001, lo * 0.9999, 3 * lo, hi * 0.9999, hi * 1.0001)):
+            if mod > 0:
+                ph = rng.uniform(-1.5, 1.5, size=32)
+                wt[p, 64 * k:64 * k + 32] = mod * np.exp(1j * ph)
+    check(gpp, prob.replace(wx_array=wx, wtilde_array=wt))
+
+
+@pytest.mark.parametrize("spread", [0.5, 2.0, 6.0])
+def test_weight_range(gpp, spread):
+    """Weights spread over e^(+-2 spread) per band and column (the widest leaves most pairs to
+    the FP64 form), zero rows, zero columns, very large and very small scales."""
+    rng = np.random.Generator(np.random.PCG64(int(10 * spread)))
+    prob = inputs.make_problem(24, 2, 256, 6, 3, seed=3)
+    am = prob.aqsmtemp * np.exp(spread * rng.standard_normal((24, 256)))
+    an = prob.aqsntemp * np.exp(spread * rng.standard_normal((24, 256)))
+    an[:, 5] = 0.0
+    an[:, 64:96] *= 1e-90
+    an[:, 100] *= 1e-250           # below the integer scaling's range: FP64
+    am[7] = 0.0
+    check(gpp, prob.replace(aqsmtemp=am, aqsntemp=an))
+    check(gpp, prob.replace(aqsmtemp=am * 1e30, aqsntemp=an * 1e-20))
+
+
+def test_one_column_of_each_extreme(gpp):
+    """A column whose largest weight and largest aqsntemp fall in different bands (their
+    product is far below the product of the maxima), beside ordinary ones."""
+    prob = inputs.make_problem(8, 2, 96, 3, 2, seed=21)
+    g = prob.indinv[prob.inv_igp_index]
+    am, an = prob.aqsmtemp.copy(), prob.aqsntemp.copy()
+    am[:, g[1]] *= 1e-4
+    am[2, g[1]] = 1.0
+    an[2, 40:60] *= 1e-5
+    check(gpp, prob.replace(aqsmtemp=am, aqsntemp=an))
