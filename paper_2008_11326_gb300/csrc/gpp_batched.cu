@@ -165,14 +165,10 @@ __device__ __forceinline__ void f64_body(const BatchInst* __restrict__ inst, int
       }
       const double2* an = d.aqsn + (live ? ig : 0);
       const double wabs2 = fma(w.x, w.x, w.y * w.y);
-      if (fix.ok) {
-        double xmax = xrange[kMaxNw];
-        for (int k = 1; k < W; ++k) xmax = fmax(xmax, xrange[kMaxNw + k]);
-        if (__all_sync(0xffffffffu, fix_lane(w, wabs2, fix.E, xmax) || !live) &&
-            fix_band_loop<W>(B, G, nocc, an, am, d.bt, live, w, live ? d.wt + p * G + ig : d.wt, I,
-                             fix.E, xrange, dyn_smem, acc))
-          continue;
-      }
+      if (fix.ok && __all_sync(0xffffffffu, fix_lane(w, wabs2, fix) || !live) &&
+          fix_band_loop<W>(B, G, nocc, an, am, d.bt, live, w, live ? d.wt + p * G + ig : d.wt, I,
+                           fix.E, xrange, dyn_smem, acc))
+        continue;
       // the FP64 fast form's conditions, with the partial fractions' bound on x / |w|
       const bool fast_lane = w.x >= 0.0 && gt_nonneg(wabs2, kFastWabs2Lo) &&
                              lt_nonneg(wabs2, kFastWabs2Hi) &&
@@ -316,9 +312,9 @@ __device__ __forceinline__ void f32_body(const BatchInst* __restrict__ inst, int
 // GPP_F32_MAXNREG registers (80 for nw > 5, whose band loop would spill at fewer).
 //
 // Measured (GB300, main sum with the split-integer form against the FP64 form alone):
-// B = 512, P = 819, G = 16384, nw = 3: 174.1 against 692.8 ms; B = 128, P = 410, G = 8192:
-// 11.68 against 44.43 ms; B = 32, P = 64, G = 512: 0.216 against 0.330 ms. Bound now: the
-// instruction issue of the integer and FP32 pipes (FP64 pipe 60% busy).
+// B = 512, P = 819, G = 16384, nw = 3: 163.7 against 692.8 ms; B = 128, P = 410, G = 8192:
+// 10.80 against 44.43 ms; B = 32, P = 64, G = 512: 0.188 against 0.330 ms. Bound now: the
+// instruction issue of the integer and FP32 pipes.
 template <int W>
 __global__ void __launch_bounds__(256, 2)
     gpp_batched_kernel_f64(const BatchInst* __restrict__ inst, int ninst, int64_t t_begin,

@@ -36,6 +36,7 @@ struct alignas(32) BandEntry {
 // flags (at kFlagFix): whether they fit the split-integer form, and with which binary scale.
 struct FixInfo {
   int ok, E;
+  double wlo2, whi2;   // its bounds on |w|^2
 };
 
 template <int V>
@@ -151,18 +152,43 @@ __device__ __forceinline__ float warp_sumf(float v) {
   return v;
 }
 
-// Per-CTA partial of NV doubles: warp butterflies, then warp partials summed in warp
-// order by the first NV threads. `red` is shared memory of at least (blockDim/32) * NV.
+// Sums of N values over the warp, each left in acc[0] of one lane (idx: which value, past the
+// last for none; the lane returns true): at every step of a fixed xor butterfly a lane hands
+// over half of its values and adds its partner's other half, so that 12 values take 13 FP64
+// additions per lane instead of 60 (they are once per tile and FP64 is narrow: a tile of few
+// bands spent a tenth of its time in them).
+template <int N, int OFF>
+__device__ __forceinline__ bool warp_scatter_sum(double* v, int lane, int& idx) {
+  if constexpr (OFF == 0) {
+    return true;
+  } else if constexpr (N == 1) {
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], OFF);
+    return warp_scatter_sum<1, OFF / 2>(v, lane, idx) && (lane & OFF) == 0;
+  } else {
+    constexpr int H = (N + 1) / 2;   // values [0, H) stay below, [H, N) go above
+    const bool up = (lane & OFF) != 0;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      const double lo = v[i], hi = i + H < N ? v[i + H] : 0.0;
+      v[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, OFF);
+    }
+    int sub = 0;
+    const bool mine = warp_scatter_sum<H, OFF / 2>(v, lane, sub);
+    idx = up ? (sub < N - H ? sub + H : N) : (sub < H ? sub : N);
+    return mine;
+  }
+}
+
+// Per-CTA partial of NV doubles: warp sums, then warp partials summed in warp order by the
+// first NV threads. `red` is shared memory of at least (blockDim/32) * NV.
 template <int NV>
 __device__ __forceinline__ void block_partials(double (&acc)[NV], double* red, double* out) {
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    double v = warp_sum(acc[k]);
-    if (lane == 0) red[warp * NV + k] = v;
-  }
+  int idx = 0;
+  const bool mine = warp_scatter_sum<NV, 16>(acc, lane, idx);
+  if (mine && idx < NV) red[warp * NV + idx] = acc[0];
   __syncthreads();
   if (threadIdx.x < NV) {
     double s = 0.0;

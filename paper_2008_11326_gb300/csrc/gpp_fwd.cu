@@ -90,7 +90,7 @@ __global__ void gpp_prep_kernel(int64_t B, int64_t G, int64_t P, int W,
   // For the FP64 sum's split-integer form, every block that writes band-table entries forms
   // the ranges of the frequencies itself (a few KB from L2; 8 / W warps share a frequency), so
   // that the table's split form and the flags need no second launch.
-  FixInfo fix{0, 0};
+  FixInfo fix{0, 0, 0.0, 0.0};
   if (want_fix && static_cast<int64_t>(blockIdx.x) * blockDim.x < B * W) {
     __shared__ double s_lo[8], s_hi[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;   // 8 warps, W <= 8

@@ -25,11 +25,12 @@
 //
 // Accumulation. The 64-bit sums of M1 U are taken modulo 2^64 (a product alone reaches 2^62)
 // beside an FP32 sum of the same products, which tells the multiple of 2^64 at the end
-// (kFlushBands bounds its error). The small parts are summed in FP32 over kLowBands bands,
-// then in FP64. Integer sums do not round, so the error does not grow with the number of
-// bands as a running FP64 sum's does. Against 128-bit arithmetic, per (p, ig) sum relative to
-// its root mean square: 2^-53.1 / -52.7 / -52.0 / -51.6 for 1 / 5 / 64 / 512 bands, the FP64
-// form's 2^-52.9 / -52.7 / -51.7 / -50.3.
+// (kFlushBands bounds its error). The small parts are summed in FP32 over kLowBands bands and
+// then moved to the integer sums. Integer sums do not round, so the error does not grow with
+// the number of bands as a running FP64 sum's does. Against 128-bit arithmetic on the drawn
+// workloads, over the root of the sum of the terms' squares (achtemp, asxtemp): 1.7e-16,
+// 1.9e-16 / 2.0, 2.1 / 2.1, 2.2 / 2.4, 2.5 for 1 / 5 / 64 / 200 bands; the FP64 form: 1.8,
+// 2.8 / 2.1, 2.4 / 3.1, 3.6 / 4.4, 5.0.
 //
 // Range (fix_lane, FixInfo): 0 <= x <= 48, Re w >= 0, 2^(E-7) <= |w| <= 1.375 2^E - max x with
 // the binary scale E of the instance's frequencies; weights whose row and column maxima over
@@ -43,7 +44,7 @@
 namespace gpp {
 
 constexpr int kStageBands = 64;    // bands of one warp's staged weights in shared memory
-constexpr int kLowBands = 16;      // bands of the FP32 low sums between FP64 flushes
+constexpr int kLowBands = 8;       // bands between moves of the FP32 low sums to the integers
 constexpr int kFlushBands = 1024;  // bands of the modular sums between flushes
 constexpr float kFixKappa = 1.0f - 0x1p-12f;
 constexpr float kFixNear = 0x1p-20f;  // |(|wdiff|^2 - 1/4)| below which FP64 decides
@@ -90,65 +91,74 @@ __device__ __forceinline__ int mad_lo(int a, int b, int c) {
   return d;
 }
 
-// The instance's frequencies fit the split-integer range with binary scale E.
+// What the split-integer form needs to know of an instance's frequencies, which lie in
+// [xmin, xmax]: whether they are in its range, the binary scale E, and the bounds on |w|^2.
 __device__ __forceinline__ FixInfo fix_info(double xmin, double xmax) {
   FixInfo f;
   f.ok = xmin >= 0.0 && xmax <= 48.0;
   int E = 2;
   while (E < 6 && xmax > 0.75 * static_cast<double>(1 << E)) ++E;
+  const double lim = 1.375 * static_cast<double>(1 << E) - xmax;
   f.E = E;
+  f.wlo2 = exp2i(2 * E - 14);
+  f.whi2 = lim * lim;
   return f;
 }
 
-// v = hi 2^-h + lo 2^-(h+32) for |v| < 2^(31-h), to 2^-(h+33).
-__device__ __forceinline__ void fix_split(double v, int h, int& hi, int& lo) {
-  const double s = v * exp2i(h);
-  double r = rint(s), l = rint((s - r) * 4294967296.0);
-  if (l >= 2147483648.0) {
-    r += 1.0;
-    l -= 4294967296.0;
-  }
-  hi = static_cast<int>(r);
-  lo = static_cast<int>(l);
+// Whether a lane's w lies in the split-integer range.
+__device__ __forceinline__ bool fix_lane(double2 w, double wabs2, const FixInfo& f) {
+  return w.x >= 0.0 && !lt_nonneg(wabs2, f.wlo2) && !gt_nonneg(wabs2, f.whi2);
 }
-// v = a + b with a a multiple of 2^ge (v / 2^ge below 2^24) and b its FP32-rounded remainder.
-__device__ __forceinline__ void fix_fsplit(double v, int ge, float& a, float& b) {
-  const double r = rint(v * exp2i(-ge)) * exp2i(ge);
-  a = static_cast<float>(r);
-  b = static_cast<float>(v - r);
+
+// v 2^k = n1 + n0 2^-32 (|n0| <= 2^31), for |v| 2^k < 2^31 - 1; khi = (k + 32) 2^20. The
+// scaling is an addition to the exponent field (k >= 0; a zero or subnormal v gives a value
+// far below the last unit), the rest one FP64 -> 64-bit integer conversion (as slow as an FP64
+// multiply-add, but the only FP64 instruction here).
+__device__ __forceinline__ void fix_value(double v, int khi, int& n1, int& n0) {
+  const double s = __hiloint2double(__double2hiint(v) + khi, __double2loint(v));
+  const long long i = __double2ll_rn(s);   // v 2^(k + 32)
+  n1 = static_cast<int>((i + 0x80000000LL) >> 32);
+  n0 = static_cast<int>(i);
+}
+
+// The FP32 form of hi 2^-h + lo 2^-(h+32), h = 30 - E: a, a multiple of 2^(E-23), plus b.
+__device__ __forceinline__ void fix_floats(int hi, int lo, int E, float& a, float& b) {
+  const int q = (hi + 64) >> 7;
+  a = static_cast<float>(q) * exp2if(E - 23);
+  b = fmaf(static_cast<float>(lo), exp2if(E - 62), static_cast<float>(hi - (q << 7)) * exp2if(E - 30));
 }
 
 // One band-table entry's split frequency.
 __device__ __forceinline__ int4 fix_x(double x, int E) {
   int hi, lo;
   float a, b;
-  fix_split(x, 30 - E, hi, lo);
-  fix_fsplit(x, E - 23, a, b);
+  fix_value(x, (62 - E) << 20, hi, lo);
+  fix_floats(hi, lo, E, a, b);
   return make_int4(hi, lo, __float_as_int(a), __float_as_int(b));
 }
 
 __device__ __forceinline__ FixPair fix_pair(double2 w, int E) {
   FixPair q;
-  fix_split(w.x, 30 - E, q.wh, q.wl);
-  fix_split(w.y, 30 - E, q.ih, q.il);
-  fix_fsplit(w.x, E - 23, q.w1, q.w2);
-  q.i1 = static_cast<float>(w.y);
-  q.i2 = static_cast<float>(w.y - static_cast<double>(q.i1));
-  fix_fsplit(w.y * w.y, 2 * E - 21, q.n1, q.n2);
+  fix_value(w.x, (62 - E) << 20, q.wh, q.wl);
+  fix_value(w.y, (62 - E) << 20, q.ih, q.il);
+  fix_floats(q.wh, q.wl, E, q.w1, q.w2);
+  // Im w = i1 + i2: the leading 24 bits of the high part, and the rest
+  const float r = static_cast<float>(q.ih);
+  q.i1 = r * exp2if(E - 30);
+  q.i2 = fmaf(static_cast<float>(q.il), exp2if(E - 62),
+              static_cast<float>(q.ih - __float2int_rn(r)) * exp2if(E - 30));
+  // (Im w)^2 = n1 + n2, n1 a multiple of 2^(2E-21)
+  const float p = q.i1 * q.i1, g = exp2if(2 * E - 21);
+  q.n1 = rintf(p * exp2if(21 - 2 * E)) * g;
+  q.n2 = (p - q.n1) + fmaf(q.i1 + q.i1, q.i2, fmaf(q.i1, q.i1, -p));
   return q;
-}
-
-// Whether a lane's w lies in the split-integer range (see the top of this file).
-__device__ __forceinline__ bool fix_lane(double2 w, double wabs2, int E, double xmax) {
-  const double lim = 1.375 * exp2i(E) - xmax;
-  return w.x >= 0.0 && wabs2 >= exp2i(2 * E - 14) && wabs2 <= lim * lim;
 }
 
 // The scales of u (or v) of one frequency: with |u| <= 1/d, ks = 31 + floor(log2 d) (U stays
 // below 2^31; from d^2, whose exponent halves), s = 2^ks and c = -1/(kappa 2^(h+ks)), minus
 // the unit of the residual e.
-__device__ __forceinline__ int fix_ks(double d2) {
-  return 31 + ((((__double2hiint(d2) >> 20) & 0x7ff) - 1023) >> 1);
+__device__ __forceinline__ int fix_ks(float d2) {
+  return 31 + (((__float_as_int(d2) >> 23) - 127) >> 1);
 }
 __device__ __forceinline__ float2 fix_scale(int ks, int E) {
   return make_float2(exp2if(ks), (-1.0f / kFixKappa) * exp2if(-(30 - E + ks)));
@@ -230,17 +240,6 @@ __host__ __device__ constexpr size_t fix_smem_bytes(int threads, int wg) {
 // Largest frequency group: more accumulators than 16 x 3 would not fit the register budget.
 constexpr int kFixMaxGroup = 3;
 
-// v 2^k = n1 + n0 2^-32 (|n0| <= 2^31), for |v| 2^k < 2^30. The scaling is an addition to the
-// exponent field (k >= 0; a zero or subnormal v gives a value far below the last unit), the
-// rest one FP64 -> 64-bit integer conversion (as slow as an FP64 multiply-add, but the only
-// FP64 instruction here).
-__device__ __forceinline__ void fix_value(double v, int khi, int& n1, int& n0) {
-  const double s = __hiloint2double(__double2hiint(v) + khi, __double2loint(v));
-  const long long i = __double2ll_rn(s);   // v 2^(k + 32)
-  n1 = static_cast<int>((i + 0x80000000LL) >> 32);
-  n0 = static_cast<int>(i);
-}
-
 // The weight M = am an of a band, times 2^(ka + kn - sh): M1 + M0.
 struct FixM {
   int r1, i1, nr1, ni1;   // M1 and -M1
@@ -272,17 +271,26 @@ __device__ __forceinline__ FixM fix_weight(const FixAm& a, double2 an, int nkhi,
   return m;
 }
 
-// Bands [b0, b1) of the thread's pair, WG frequencies from iw0 of W, added to the thread's
-// FP64 sums st[k blockDim.x] (units of kappa 2^ks M; values 4 iw + {0, 1}: sum M u, + {2, 3},
-// with OCC: sum M v).
+// What a pair's band loops share.
+struct FixCtx {
+  int64_t G;
+  const double2* an;   // the pair's column of aqsntemp (stride G)
+  const double2* am;   // the row of weights
+  const double2* w64;  // the FP64 w, for exact branch decisions
+  const BandEntry* bt;
+  int W, nkhi, akhi, sh;
+  FixAm* stage;
+};
+
+// Bands [b0, b1) of the thread's pair, WG frequencies from iw0, into the thread's FP64 sums
+// st[k blockDim.x] (units of kappa 2^ks M with the ks of u; values 4 iw + {0, 1}: sum M u, and
+// with OCC + {2, 3}: sum M u - sum M v), added to them, or with `fresh` replacing them.
 template <int WG, bool OCC>
-__device__ __forceinline__ void fix_range(int b0, int b1, int64_t G, int W, int iw0,
-                                           const double2* __restrict__ an_ptr, int nkhi,
-                                           const double2* __restrict__ am_ptr, int akhi,
-                                           const BandEntry* __restrict__ bt, const FixPair& w,
-                                           const double2* __restrict__ w_ptr, int sh, double* st,
-                                          const float2* sc, FixAm* stage) {
+__device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixCtx& ctx, int iw0,
+                                          const FixPair& w, double* st, const float2* sc) {
   const int nt = blockDim.x, lane = threadIdx.x & 31;
+  const int64_t G = ctx.G;
+  FixAm* const stage = ctx.stage;
 #pragma unroll 1
   for (int f0 = b0; f0 < b1; f0 += kFlushBands) {
     const int f1 = min(f0 + kFlushBands, b1);
@@ -294,16 +302,16 @@ __device__ __forceinline__ void fix_range(int b0, int b1, int64_t G, int W, int 
       aH[k] = 0.0f;
       aL[k] = 0.0f;
     }
-    double2 an_next = ldg2(an_ptr + static_cast<int64_t>(f0) * G);
+    double2 an_next = ldg2(ctx.an + static_cast<int64_t>(f0) * G);
 #pragma unroll 1
     for (int s0 = f0; s0 < f1; s0 += kStageBands) {
       const int s1 = min(s0 + kStageBands, f1);
       __syncwarp();
       for (int b = s0 + lane; b < s1; b += 32) {   // this warp's weights of the next bands
-        const double2 a = ldg2(am_ptr + b);
+        const double2 a = ldg2(ctx.am + b);
         FixAm e;
-        fix_value(a.x, akhi, e.r1, e.r0);
-        fix_value(a.y, akhi, e.i1, e.i0);
+        fix_value(a.x, ctx.akhi, e.r1, e.r0);
+        fix_value(a.y, ctx.akhi, e.i1, e.i0);
         stage[b - s0] = e;
       }
       __syncwarp();
@@ -313,9 +321,9 @@ __device__ __forceinline__ void fix_range(int b0, int b1, int64_t G, int W, int 
 #pragma unroll 1
         for (int b = l0; b < l1; ++b) {
           const double2 an = an_next;
-          if (b + 1 < b1) an_next = ldg2(an_ptr + static_cast<int64_t>(b + 1) * G);
-          const FixM m = fix_weight(stage[b - s0], an, nkhi, sh);
-          const BandEntry* btb = bt + static_cast<int64_t>(b) * W + iw0;
+          if (b + 1 < b1) an_next = ldg2(ctx.an + static_cast<int64_t>(b + 1) * G);
+          const FixM m = fix_weight(stage[b - s0], an, ctx.nkhi, ctx.sh);
+          const BandEntry* btb = ctx.bt + static_cast<int64_t>(b) * ctx.W + iw0;
           int4 xv[WG];
           FixN na[WG];
           float d[WG];   // |wdiff|^2 - 1/4: its sign decides branch 1
@@ -328,7 +336,7 @@ __device__ __forceinline__ void fix_range(int b0, int b1, int64_t G, int W, int 
             dmin = fminf(dmin, fabsf(d[k]));
           }
           if (__any_sync(0xffffffffu, dmin <= kFixNear)) {   // rare: the FP64 form's decisions
-            const double2 wv = ldg2(w_ptr);
+            const double2 wv = ldg2(ctx.w64);
 #pragma unroll
             for (int k = 0; k < WG; ++k) {
               const double a = __ldg(&btb[k].lo.x) - wv.x;
@@ -358,22 +366,57 @@ __device__ __forceinline__ void fix_range(int b0, int b1, int64_t G, int W, int 
             }
           }
         }
+        // the low sums (below 2^36) into the integer sums in units of 2^6; the rest stays
 #pragma unroll
         for (int k = 0; k < 4 * WG; ++k)
           if (OCC || (k & 2) == 0) {
-            st[k * nt] += static_cast<double>(aL[k]);
-            aL[k] = 0.0f;
+            const int r = __float2int_rn(aL[k] * 0x1p-6f);
+            acc[k] = mad_wide(r, 64, acc[k]);
+            aL[k] = fmaf(-64.0f, static_cast<float>(r), aL[k]);
           }
       }
     }
 #pragma unroll
-    for (int k = 0; k < 4 * WG; ++k)
-      if (OCC || (k & 2) == 0) {
-        // the sum is acc + j 2^64 with j from the FP32 sum
-        const float top = static_cast<float>(static_cast<int>(acc[k] >> 32)) * 0x1p-32f;
-        const int j = __float2int_rn(fmaf(aH[k], 0x1p-64f, -top));
-        st[k * nt] += fma(static_cast<double>(j), 18446744073709551616.0, static_cast<double>(acc[k]));
+    for (int k = 0; k < 4 * WG; ++k) acc[k] += __float2int_rn(aL[k]);
+    // the sums are acc + j 2^64, with j from the FP32 sums (mostly zero)
+    int j[4 * WG], any = 0;
+#pragma unroll
+    for (int k = 0; k < 4 * WG; ++k) {
+      const float top = static_cast<float>(static_cast<int>(acc[k] >> 32)) * 0x1p-32f;
+      j[k] = __float2int_rn(fmaf(aH[k], 0x1p-64f, -top));
+      any |= j[k];
+    }
+    const bool carry = __any_sync(0xffffffffu, any != 0);
+    auto sum = [&](int k) {
+      const double v = static_cast<double>(acc[k]);
+      return carry ? fma(static_cast<double>(j[k]), 18446744073709551616.0, v) : v;
+    };
+    auto put = [&](int k, double v) { st[k * nt] = (!fresh || f0 > b0) ? st[k * nt] + v : v; };
+#pragma unroll
+    for (int k = 0; k < WG; ++k) {
+      if (!OCC) {
+        put(4 * k, sum(4 * k));
+        put(4 * k + 1, sum(4 * k + 1));
+        continue;
       }
+      const double r = -exp2i((__float_as_int(sc[2 * k * nt].x) - __float_as_int(sc[(2 * k + 1) * nt].x)) >> 23);
+#pragma unroll
+      for (int c = 4 * k; c < 4 * k + 2; ++c) {
+        double a, d;
+        if (carry) {
+          a = sum(c);
+          d = fma(r, sum(c + 2), a);
+        } else {   // by halves: the difference (which may cancel) is rounded once
+          constexpr double k32 = 4294967296.0;
+          const double ah = static_cast<int>(acc[c] >> 32), al = static_cast<unsigned>(acc[c]);
+          const double sh = static_cast<int>(acc[c + 2] >> 32), sl = static_cast<unsigned>(acc[c + 2]);
+          a = fma(ah, k32, al);
+          d = fma(fma(r, sh, ah), k32, fma(r, sl, al));
+        }
+        put(c, a);
+        put(c + 2, d);
+      }
+    }
   }
 }
 
@@ -393,7 +436,7 @@ __device__ __forceinline__ bool fix_exponent(unsigned m, int& k) {
 }
 
 // All bands of the thread's pair by the split-integer form, multiplied by Iw = I w and added
-// to tacc[4 W]. Returns false (nothing added) if any lane of the warp is out of range.
+// to tacc[4 W]. Returns false (nothing added) if any lane of the warp is out of range. B >= 1.
 template <int W>
 __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
                                            const double2* __restrict__ an_ptr,
@@ -406,8 +449,6 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
   const int nt = blockDim.x, warp = threadIdx.x >> 5;
   double* st = reinterpret_cast<double*>(smem) + threadIdx.x;
   float2* sc = reinterpret_cast<float2*>(smem + static_cast<size_t>(nt) * 4 * WG * 8) + threadIdx.x;
-  FixAm* stage = reinterpret_cast<FixAm*>(smem + static_cast<size_t>(nt) * 6 * WG * 8) +
-                 warp * kStageBands;
   // the magnitudes of the column of aqsntemp, of the row of weights and of their products
   unsigned mn = 0, ma = 0, mp = 0;
   int kn, ka;
@@ -419,50 +460,58 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
     ma = max(ma, ha);
     mp = max(mp, hn + ha);
   }
-  const bool exp_ok = fix_exponent(mn, kn) && fix_exponent(ma, ka);
+  const bool n_ok = fix_exponent(mn, kn), a_ok = fix_exponent(ma, ka);
+  if (!live) kn = 0;   // whatever its column holds: the values stay finite and I is zero
   // every |M| comp 2^(ka + kn) < 2^top: twice (complex) the largest product, 0.18 for its
   // logarithm; sh takes the largest to 31 bits
   const int top = static_cast<int>((mp + (1u << 20) + 188744u) >> 20) + 1 - 2046 + ka + kn;
-  const bool m_ok = exp_ok && (mn == 0 || ma == 0 || top >= kFixMinTop);
-  if (!__all_sync(0xffffffffu, m_ok || !live)) return false;
+  const bool m_ok = n_ok && (mn == 0 || ma == 0 || top >= kFixMinTop);
+  if (!a_ok || !__all_sync(0xffffffffu, m_ok || !live)) return false;
   const int sh = max(min(top - 31, 30), 1);
-  const int nkhi = (kn + 32) << 20, akhi = (ka + 32) << 20;   // for fix_value
+  const FixCtx ctx{G, an_ptr, am_ptr, w_ptr, bt, W, (kn + 32) << 20, (ka + 32) << 20, sh,
+                   reinterpret_cast<FixAm*>(smem + static_cast<size_t>(nt) * 6 * WG * 8) +
+                       warp * kStageBands};
   const FixPair w = fix_pair(wv, E);
   const double Iwr = fma(I.x, wv.x, -I.y * wv.y), Iwi = fma(I.x, wv.y, I.y * wv.x);
-  double add[4 * W];
-  auto group = [&](auto tag, int iw0, double* out) {
+  auto group = [&](auto tag, int iw0) {
     constexpr int N = decltype(tag)::value;
     int ks[2 * N];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-      const double lo = xrange[iw0 + k], hi = xrange[kMaxNw + iw0 + k];
-      const double dA = fmax(0.5, fmax(lo - wv.x, wv.x - hi));
-      const double sr = lo + wv.x;
+      // the distance of the frequencies from w and -w, less its FP32 rounding
+      const float lo = static_cast<float>(xrange[iw0 + k]);
+      const float hi = static_cast<float>(xrange[kMaxNw + iw0 + k]);
+      const float dA = fmaxf(0.5f, fmaxf(lo - w.w1, w.w1 - hi) * (1.0f - 0x1p-17f));
+      const float sr = lo + w.w1;
       ks[2 * k] = fix_ks(dA * dA);
-      ks[2 * k + 1] = fix_ks(fma(sr, sr, wv.y * wv.y));
+      ks[2 * k + 1] = fix_ks(fmaf(sr, sr, w.i1 * w.i1) * (1.0f - 0x1p-17f));
       sc[2 * k * nt] = fix_scale(ks[2 * k], E);
       sc[(2 * k + 1) * nt] = fix_scale(ks[2 * k + 1], E);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) st[(4 * k + i) * nt] = 0.0;
     }
-    fix_range<N, true>(0, nocc, G, W, iw0, an_ptr, nkhi, am_ptr, akhi, bt, w, w_ptr, sh,
-                       st, sc, stage);
+    // units: M1 = M 2^(ka + kn - sh), U = u kappa 2^ks
+    const int ex = sh - ka - kn;
+    double ax[2 * N];   // asxtemp: (its bands' achtemp - sum M v) / 2
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
-      // units: M1 = M 2^(ka + kn - sh), U = u kappa 2^ks
-      const double fa = exp2i(sh - ka - kn - ks[2 * k]) * (1.0 / kFixKappa);
-      const double fs = exp2i(sh - ka - kn - ks[2 * k + 1]) * (1.0 / kFixKappa);
-      out[4 * k + 2] = 0.5 * fma(fa, st[4 * k * nt], -fs * st[(4 * k + 2) * nt]);
-      out[4 * k + 3] = 0.5 * fma(fa, st[(4 * k + 1) * nt], -fs * st[(4 * k + 3) * nt]);
+    for (int k = 0; k < 2 * N; ++k) ax[k] = 0.0;
+    if (nocc > 0) {
+      fix_range<N, true>(0, nocc, true, ctx, iw0, w, st, sc);
+#pragma unroll
+      for (int k = 0; k < N; ++k) {
+        const double fa = exp2i(ex - ks[2 * k] - 1) * (1.0 / kFixKappa);
+        ax[2 * k] = fa * st[(4 * k + 2) * nt];
+        ax[2 * k + 1] = fa * st[(4 * k + 3) * nt];
+      }
     }
-    if (nocc < B)
-      fix_range<N, false>(nocc, B, G, W, iw0, an_ptr, nkhi, am_ptr, akhi, bt, w, w_ptr, sh,
-                         st, sc, stage);
+    if (nocc < B) fix_range<N, false>(nocc, B, nocc == 0, ctx, iw0, w, st, sc);
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
-      const double fa = exp2i(sh - ka - kn - ks[2 * k]) * (1.0 / kFixKappa);
-      out[4 * k] = fa * st[4 * k * nt];
-      out[4 * k + 1] = fa * st[(4 * k + 1) * nt];
+    for (int k = 0; k < N; ++k) {   // tacc += I w times the pair's sums
+      const double fa = exp2i(ex - ks[2 * k]) * (1.0 / kFixKappa);
+      const double ar = fa * st[4 * k * nt], ai = fa * st[(4 * k + 1) * nt];
+      double* o = tacc + 4 * (iw0 + k);
+      o[0] = fma(Iwr, ar, fma(-Iwi, ai, o[0]));
+      o[1] = fma(Iwr, ai, fma(Iwi, ar, o[1]));
+      o[2] = fma(Iwr, ax[2 * k], fma(-Iwi, ax[2 * k + 1], o[2]));
+      o[3] = fma(Iwr, ax[2 * k + 1], fma(Iwi, ax[2 * k], o[3]));
     }
   };
   // frequency groups of at most three; the weights are formed again for each
@@ -472,15 +521,9 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
   for (int g = 0; g < NG; ++g) {
     const int iw0 = g * LO + (g < NHI ? g : NHI);
     if (g < NHI)
-      group(IntTag<LO + 1>(), iw0, add + 4 * iw0);
+      group(IntTag<LO + 1>(), iw0);
     else
-      group(IntTag<LO>(), iw0, add + 4 * iw0);
-  }
-#pragma unroll
-  for (int k = 0; k < 2 * W; ++k) {   // tacc += Iw add, per complex value
-    const double tr = add[2 * k], ti = add[2 * k + 1];
-    tacc[2 * k] = fma(Iwr, tr, fma(-Iwi, ti, tacc[2 * k]));
-    tacc[2 * k + 1] = fma(Iwr, ti, fma(Iwi, tr, tacc[2 * k + 1]));
+      group(IntTag<LO>(), iw0);
   }
   return true;
 }
