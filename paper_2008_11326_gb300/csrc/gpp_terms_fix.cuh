@@ -141,6 +141,7 @@ __device__ __forceinline__ FixPair fix_pair(double2 w, int E) {
   FixPair q;
   fix_value(w.x, (62 - E) << 20, q.wh, q.wl);
   fix_value(w.y, (62 - E) << 20, q.ih, q.il);
+  q.il = max(q.il, -0x7fffffff);   // its negative is taken (2^-32 of the unit is below rounding)
   fix_floats(q.wh, q.wl, E, q.w1, q.w2);
   // Im w = i1 + i2: the leading 24 bits of the high part, and the rest
   const float r = static_cast<float>(q.ih);

@@ -99,3 +99,28 @@ def test_one_column_of_each_extreme(gpp):
     am[2, g[1]] = 1.0
     an[2, 40:60] *= 1e-5
     check(gpp, prob.replace(aqsmtemp=am, aqsntemp=an))
+
+
+def test_limb_edges(gpp):
+    """Poles, frequencies and weights whose low 32-bit limbs are exactly the most negative
+    integer, or whose values are exact in few bits (halves and multiples of the high limb's
+    unit, 2^-26 for frequencies up to 12; powers of two; equal magnitudes)."""
+    rng = np.random.Generator(np.random.PCG64(11))
+    prob = inputs.make_problem(19, 2, 256, 8, 3, seed=13)
+    u = 2.0 ** -26
+    wt = prob.wtilde_array.copy()
+    half = lambda a: (np.floor(a / u) + 0.5) * u  # noqa: E731
+    wt[0:2] = half(wt[0:2].real) + 1j * half(wt[0:2].imag)
+    wt[2:4] = half(wt[2:4].real) + 1j * np.round(wt[2:4].imag / u) * u
+    wt[4:6] = wt[4:6].real + 1j * half(wt[4:6].imag)
+    wt[6] = wt[6].real                              # real poles
+    wt[7] = rng.choice([0.25, 0.5, 1.0, 2.0], size=256) + 0.5j * rng.choice([-1, 0, 1], size=256)
+    wx = prob.wx_array.copy()
+    wx[:6] = half(wx[:6])
+    wx[6] = [0.0, 4.0, 12.0]
+    am, an = prob.aqsmtemp.copy(), prob.aqsntemp.copy()
+    an[3:6] = rng.choice([-1.0, 1.0], size=(3, 256)) + 1j * rng.choice([-1.0, 1.0], size=(3, 256))
+    an[7:9] = half(an[7:9].real) + 1j * half(an[7:9].imag)
+    am[4] = 1.0 - 2.0 ** -53
+    am[5] = -1.0 + 2.0 ** -53
+    check(gpp, prob.replace(wtilde_array=wt, wx_array=wx, aqsmtemp=am, aqsntemp=an))
