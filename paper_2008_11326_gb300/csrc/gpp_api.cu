@@ -121,9 +121,21 @@ int check_pointers(const gpp_problem& p, int precision, bool outputs = true) {
   return GPP_OK;
 }
 
-// Default G-vectors per thread of a tile. On GB300 (benchmark instance, 128 threads) the
-// FP32-bulk main kernel ran 93.6 / 92.6 / 95.3 / 94.2 / 94.9 ms at 1 / 2 / 3 / 4 / 8.
-int default_igpt(int precision) { return precision == GPP_FP32_BULK ? 2 : 4; }
+// Default G-vectors per thread of a tile, where `columns` is the number of tiles' worth of
+// blocks of `threads` G-vectors (over all instances). Deeper tiles share a tile's overhead
+// (FP64: block reduction; FP32-bulk: sort and reduction); shallower ones balance the SMs.
+// FP64 (128 threads, 4 CTAs per SM): 4 from 64 tiles per SM on, 2 from 16, else 1. Measured,
+// us at 1 / 2 / 4: B=128 P=410 G=8192 (43 tiles per SM at 4) 10650 / 10590 / 10790; B=64 P=200
+// G=3000 (16 at 2) 1068 / 1063 / 1102; B=32 P=64 G=512 (0.8 at 2) 88 / 115 / 190.
+// FP32-bulk: 2 from 2 tiles per SM on, else 1: benchmark instance 93.6 / 92.6 / 94.2 ms at
+// 1 / 2 / 4; B=37 P=95 G=1901 (5 at 2) 85 / 77 / 92 us; B=32 P=64 G=512 (0.8 at 2) 55 / 64 / 83.
+int default_igpt(int precision, double columns, int sms) {
+  if (precision == GPP_FP32_BULK) return columns >= 2.0 * 2 * sms ? 2 : 1;
+  return columns >= 4.0 * 64 * sms ? 4 : columns >= 2.0 * 16 * sms ? 2 : 1;
+}
+double tile_columns(const gpp_problem& p, int threads) {
+  return static_cast<double>(p.ngpown) * static_cast<double>((p.ncouls + threads - 1) / threads);
+}
 
 // Workspace layout of one instance. The gather segments come first; unless `gather_only`
 // (instances of a batched plan, the adjoint), the descriptor, tile counter and per-tile
@@ -134,7 +146,7 @@ int make_plan(const gpp_problem& p, const gpp_options& o, gpp::FwdPlan* plan,
   pl.nw = static_cast<int>(p.nw);
   const bool f32 = o.precision == GPP_FP32_BULK;
   pl.threads = o.block_threads ? o.block_threads : 128;
-  pl.igpt = o.ig_per_thread ? o.ig_per_thread : default_igpt(o.precision);
+  pl.igpt = o.ig_per_thread ? o.ig_per_thread : 1;
   if (degenerate(p)) {
     *plan = pl;
     return GPP_OK;
@@ -165,6 +177,7 @@ int make_plan(const gpp_problem& p, const gpp_options& o, gpp::FwdPlan* plan,
     int dev = 0, sms = 0;
     cudaError_t e = checked(cudaGetDevice(&dev));
     if (e == cudaSuccess) e = checked(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (!o.ig_per_thread) pl.igpt = default_igpt(o.precision, tile_columns(p, pl.threads), sms);
     if (e == cudaSuccess) e = gpp::batched_prepare(pl.threads, pl.nw, f32, pl.igpt);
     if (e != cudaSuccess) return cuda_fail(e, "querying the device");
     int bps = o.blocks_per_sm ? o.blocks_per_sm
@@ -375,7 +388,7 @@ int gpp_sigma(const gpp_problem* prob, const gpp_options* opt, void* workspace,
   desc.tile_end = plan.ntiles;
   cudaError_t e = checked(mark(0));
   if (e != cudaSuccess) return cuda_fail(e, "recording stage event 0");
-  e = checked(gpp::launch_prep(p, plan, ws, f32, &desc, s));
+  e = checked(gpp::launch_prep(p, plan, ws, f32, o.debug_checks != 0, &desc, s));
   if (e != cudaSuccess) return cuda_fail(e, "launching the column gather");
   if (o.debug_checks) {
     int flags[4];
@@ -391,7 +404,7 @@ int gpp_sigma(const gpp_problem* prob, const gpp_options* opt, void* workspace,
   double* partials = reinterpret_cast<double*>(ws + plan.off_partials);
   e = checked(gpp::launch_batched_main(dptr, 1, plan.ntiles, plan.nw, f32, plan.grid, plan.threads,
                                plan.igpt, reinterpret_cast<unsigned long long*>(ws + plan.off_counter),
-                               partials, s));
+                               true, partials, s));
   if (e != cudaSuccess) return cuda_fail(e, "launching the main sum");
   if ((e = checked(mark(2))) != cudaSuccess) return cuda_fail(e, "recording stage event 2");
   e = checked(gpp::launch_batched_reduce(dptr, 1, plan.nw, f32, partials, s));
@@ -449,7 +462,7 @@ int gpp_sigma_backward(const gpp_problem* prob, const gpp_options* opt,
     return fail(GPP_ERR_WORKSPACE, "adjoint workspace must be 256-byte aligned with %zu bytes",
                 plan.total);
   char* ws = static_cast<char*>(workspace);
-  cudaError_t e = checked(gpp::launch_prep(p, plan.fwd, ws, false, nullptr, s));
+  cudaError_t e = checked(gpp::launch_prep(p, plan.fwd, ws, false, o.debug_checks != 0, nullptr, s));
   if (e != cudaSuccess) return cuda_fail(e, "launching the column gather");
   if (o.debug_checks) {
     int flags[4];
@@ -476,8 +489,9 @@ struct gpp_batched_plan {
   gpp_options opt;  // the validated options (shared by every instance)
   int64_t ntiles = 0;
   char* ws = nullptr;
-  size_t total = 0, off_inst = 0, off_counter = 0, off_partials = 0;
+  size_t total = 0, off_inst = 0, off_prep = 0, off_counter = 0, off_partials = 0;
   std::vector<gpp_problem> probs;
+  std::vector<gpp::PrepArgs> prep;   // the instances' gathers, in the caller's order
   std::vector<gpp::FwdPlan> iplan;
   std::vector<size_t> ioff;
   std::vector<gpp::BatchInst> inst;  // in tile order
@@ -498,10 +512,12 @@ int batched_layout(const gpp_problem* probs, int n, const gpp_options* opt, bool
   bp->nw = static_cast<int>(probs[0].nw);
   bp->f32 = o.precision == GPP_FP32_BULK;
   bp->threads = o.block_threads ? o.block_threads : 128;
-  bp->igpt = o.ig_per_thread ? o.ig_per_thread : default_igpt(o.precision);
   int dev = 0, sms = 0;
   cudaError_t e = checked(cudaGetDevice(&dev));
   if (e == cudaSuccess) e = checked(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  double columns = 0.0;
+  for (int i = 0; i < n; ++i) columns += tile_columns(probs[i], bp->threads);
+  bp->igpt = o.ig_per_thread ? o.ig_per_thread : default_igpt(o.precision, columns, sms);
   if (e == cudaSuccess) e = gpp::batched_prepare(bp->threads, bp->nw, bp->f32, bp->igpt);
   if (e != cudaSuccess) return cuda_fail(e, "querying the device");
   int bps = o.blocks_per_sm ? o.blocks_per_sm
@@ -545,6 +561,8 @@ int batched_layout(const gpp_problem* probs, int n, const gpp_options* opt, bool
   bp->ntiles = t0;
   bp->off_inst = off;
   off = gpp::align_up(off + static_cast<size_t>(n) * sizeof(gpp::BatchInst));
+  bp->off_prep = off;
+  off = gpp::align_up(off + static_cast<size_t>(n) * sizeof(gpp::PrepArgs));
   bp->off_counter = off;
   off = gpp::align_up(off + sizeof(unsigned long long));
   bp->off_partials = off;
@@ -569,21 +587,31 @@ int batched_bind(gpp_batched_plan* bp, void* workspace, size_t bytes) {
     full.tile_end = d.tile_end;
     d = full;
   }
+  bp->prep.clear();
+  for (int i = 0; i < bp->n; ++i)
+    bp->prep.push_back(gpp::prep_args(bp->probs[i], bp->iplan[i], bp->ws + bp->ioff[i], bp->f32, false));
   return GPP_OK;
 }
 
 cudaError_t batched_enqueue(gpp_batched_plan* bp, cudaStream_t s) {
   for (int i = 0; i < bp->n; ++i) {
-    cudaError_t e = checked(gpp::launch_prep(bp->probs[i], bp->iplan[i], bp->ws + bp->ioff[i], bp->f32,
-                                     nullptr, s));
+    if (!bp->f32 || !bp->iplan[i].convert_c64) continue;
+    const gpp_problem& p = bp->probs[i];
+    cudaError_t e = checked(gpp::launch_convert_c64(
+        p.aqsntemp, p.ncouls,
+        reinterpret_cast<gpp_c64*>(bp->ws + bp->ioff[i] + bp->iplan[i].off_aqsn32), p.ncouls,
+        p.number_bands, 0, p.ncouls, s));
     if (e != cudaSuccess) return e;
   }
+  cudaError_t e = checked(gpp::launch_prep_batch(
+      bp->prep.data(), reinterpret_cast<const gpp::PrepArgs*>(bp->ws + bp->off_prep), bp->n, s));
+  if (e != cudaSuccess) return e;
   const auto* inst = reinterpret_cast<const gpp::BatchInst*>(bp->ws + bp->off_inst);
   double* partials = reinterpret_cast<double*>(bp->ws + bp->off_partials);
-  cudaError_t e = checked(gpp::launch_batched_main(inst, bp->n, bp->ntiles, bp->nw, bp->f32, bp->grid,
-                                           bp->threads, bp->igpt,
-                                           reinterpret_cast<unsigned long long*>(bp->ws + bp->off_counter),
-                                           partials, s));
+  e = checked(gpp::launch_batched_main(inst, bp->n, bp->ntiles, bp->nw, bp->f32, bp->grid, bp->threads,
+                                       bp->igpt,
+                                       reinterpret_cast<unsigned long long*>(bp->ws + bp->off_counter),
+                                       false, partials, s));
   if (e != cudaSuccess) return e;
   return gpp::launch_batched_reduce(inst, bp->n, bp->nw, bp->f32, partials, s);
 }
@@ -612,6 +640,9 @@ int gpp_batched_plan_create(gpp_batched_plan** plan, const gpp_problem* probs, i
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = checked(cudaMemcpyAsync(bp->ws + bp->off_inst, bp->inst.data(),
                                   bp->inst.size() * sizeof(gpp::BatchInst), cudaMemcpyHostToDevice, s));
+  if (e == cudaSuccess)
+    e = checked(cudaMemcpyAsync(bp->ws + bp->off_prep, bp->prep.data(),
+                                bp->prep.size() * sizeof(gpp::PrepArgs), cudaMemcpyHostToDevice, s));
   if (e == cudaSuccess) e = checked(cudaStreamSynchronize(s));
   if (e != cudaSuccess) {
     delete bp;
@@ -909,7 +940,7 @@ int gpp_sigma_host(const gpp_problem* prob, const gpp_options* opt, void* worksp
   desc.tile_end = plan.ntiles;
   e = checked(cudaStreamWaitEvent(s, ev.ev[1], 0));
   if (e == cudaSuccess) e = checked(mark(0));
-  if (e == cudaSuccess) e = checked(gpp::launch_prep(d, plan, sws, f32, &desc, s));
+  if (e == cudaSuccess) e = checked(gpp::launch_prep(d, plan, sws, f32, o.debug_checks != 0, &desc, s));
   if (e != cudaSuccess) return drain_fail(e, "launching the column gather");
   if (o.debug_checks) {
     int flags[4];
@@ -937,7 +968,7 @@ int gpp_sigma_host(const gpp_problem* prob, const gpp_options* opt, void* worksp
     e = checked(cudaStreamWaitEvent(sk, ev.ev[3 + k], 0));
     if (e == cudaSuccess)
       e = checked(gpp::launch_batched_main(dptr, 1, t1, plan.nw, f32, grid, plan.threads, plan.igpt,
-                                   counters + k, partials, sk, t0));
+                                   counters + k, false, partials, sk, t0));
     second_used = second_used || (k & 1);
   }
   if (e == cudaSuccess && second_used) {

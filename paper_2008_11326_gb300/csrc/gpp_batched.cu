@@ -11,6 +11,7 @@
 // tile. A per-instance kernel then sums the instance's tile partials in tile order. The
 // per-tile arithmetic is the single-instance kernels' (gpp_terms_f64.cuh / gpp_terms_f32.cuh).
 
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "gpp_device.cuh"
@@ -312,9 +313,9 @@ __device__ __forceinline__ void f32_body(const BatchInst* __restrict__ inst, int
 // GPP_F32_MAXNREG registers (80 for nw > 5, whose band loop would spill at fewer).
 //
 // Measured (GB300, main sum with the split-integer form against the FP64 form alone):
-// B = 512, P = 819, G = 16384, nw = 3: 163.7 against 692.8 ms; B = 128, P = 410, G = 8192:
-// 10.80 against 44.43 ms; B = 32, P = 64, G = 512: 0.188 against 0.330 ms. Bound now: the
-// instruction issue of the integer and FP32 pipes.
+// B = 512, P = 819, G = 16384, nw = 3: 163.6 against 692.8 ms; B = 128, P = 410, G = 8192:
+// 10.5 against 44.4 ms; B = 32, P = 64, G = 512: 0.057 against 0.30 ms (with shallower tiles
+// and the cheaper reduction). Bound now: the instruction issue of the integer and FP32 pipes.
 template <int W>
 __global__ void __launch_bounds__(256, 2)
     gpp_batched_kernel_f64(const BatchInst* __restrict__ inst, int ninst, int64_t t_begin,
@@ -331,38 +332,60 @@ __global__ void __launch_bounds__(256) __maxnreg__(W <= 5 ? GPP_F32_MAXNREG : 80
   f32_body<W>(inst, ninst, t_begin, ntiles, igpt, counter, partials);
 }
 
-// One CTA per instance: the instance's tile partials summed in tile order, then a tree.
+// A cluster of kReduceCtas CTAs per instance sums the instance's tile partials in a fixed
+// order: CTA r takes the r-th share of the tiles; its thread t takes value t % nv of every
+// (T / nv)-th tile of the share from tile t / nv on (so that the CTA reads the partials in
+// order); warp k then sums value k's threads and hands the sum to the first CTA's shared
+// memory, which adds the CTAs' in order. Bound by the latency of the loads (12 values, ncu):
+// 64 tiles 4.9 us, 13120 tiles 18 us; one CTA of 256 threads taking a value at a time was 20 and
+// 57 us (6560 tiles) between events.
+constexpr int kReduceThreads = 512, kReduceCtas = 8;
 template <bool F32>
-__global__ void __launch_bounds__(256) gpp_batched_reduce_kernel(const BatchInst* __restrict__ inst,
-                                                                 int nv,
-                                                                 const double* __restrict__ part) {
-  __shared__ double s[256];
-  const BatchInst& d = inst[blockIdx.x];
-  const int64_t n = d.tile_end - d.tile0;
-  for (int k = 0; k < nv; ++k) {
+__global__ void __launch_bounds__(kReduceThreads) __cluster_dims__(kReduceCtas, 1, 1)
+    gpp_batched_reduce_kernel(const BatchInst* __restrict__ inst, int nv,
+                              const double* __restrict__ part) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ double s[kReduceThreads];
+  __shared__ double total[kReduceCtas][4 * kMaxNw];
+  const int rank = static_cast<int>(cluster.block_rank());
+  const BatchInst& d = inst[blockIdx.x / kReduceCtas];
+  const int per = kReduceThreads / nv, j0 = threadIdx.x / nv, k = threadIdx.x - j0 * nv;
+  if (j0 < per) {
+    const int64_t n = d.tile_end - d.tile0;
+    const int64_t share = (n + kReduceCtas - 1) / kReduceCtas;
+    const int64_t first = rank * share, last = min(first + share, n);
     double v = 0.0;
-    for (int64_t j = threadIdx.x; j < n; j += 256) {
+#pragma unroll 8
+    for (int64_t j = first + j0; j < last; j += per) {
+      const int64_t at = (d.tile0 + j) * nv + k;
       if (F32) {
-        const float2 q = reinterpret_cast<const float2*>(part)[(d.tile0 + j) * nv + k];
+        const float2 q = reinterpret_cast<const float2*>(part)[at];
         v += static_cast<double>(q.x) + static_cast<double>(q.y);
       } else {
-        v += part[(d.tile0 + j) * nv + k];
+        v += part[at];
       }
     }
     s[threadIdx.x] = v;
-    __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-      if (threadIdx.x < h) s[threadIdx.x] += s[threadIdx.x + h];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-      const int iw = k / 4, c = k % 4;
-      if (c < 2)
-        reinterpret_cast<double*>(d.ach)[2 * iw + c] = s[0] * d.ach_scale;
-      else
-        reinterpret_cast<double*>(d.asx)[2 * iw + c - 2] = s[0];
-    }
-    __syncthreads();
+  }
+  cluster.sync();   // s is complete; every CTA of the cluster runs (its shared memory exists)
+  const int lane = threadIdx.x & 31;
+  double* const dst = cluster.map_shared_rank(&total[rank][0], 0);
+  for (int q = threadIdx.x >> 5; q < nv; q += kReduceThreads / 32) {
+    double v = 0.0;
+    for (int j = lane; j < per; j += 32) v += s[j * nv + q];
+    v = warp_sum(v);
+    if (lane == 0) dst[q] = v;
+  }
+  cluster.sync();   // after it no CTA reads another's shared memory
+  if (rank == 0 && threadIdx.x < nv) {
+    double v = 0.0;
+    for (int r = 0; r < kReduceCtas; ++r) v += total[r][threadIdx.x];
+    const int iw = threadIdx.x / 4, c = threadIdx.x % 4;
+    if (c < 2)
+      reinterpret_cast<double*>(d.ach)[2 * iw + c] = v * d.ach_scale;
+    else
+      reinterpret_cast<double*>(d.asx)[2 * iw + c - 2] = v;
   }
 }
 
@@ -422,10 +445,12 @@ int batched_blocks_per_sm(int threads, int nw, bool f32, int igpt) {
 
 cudaError_t launch_batched_main(const BatchInst* inst, int ninst, int64_t ntiles, int nw,
                                 bool f32, int grid, int threads, int igpt,
-                                unsigned long long* counter, double* partials, cudaStream_t s,
-                                int64_t t_begin) {
-  cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return e;
+                                unsigned long long* counter, bool cleared, double* partials,
+                                cudaStream_t s, int64_t t_begin) {
+  if (!cleared) {
+    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
+    if (e != cudaSuccess) return e;
+  }
   const size_t smem = batched_smem_bytes(threads, nw, f32, igpt);
 #define GPP_BATCHED_LAUNCH(WV)                                                                    \
   if (f32)                                                                                        \
@@ -452,9 +477,9 @@ cudaError_t launch_batched_main(const BatchInst* inst, int ninst, int64_t ntiles
 cudaError_t launch_batched_reduce(const BatchInst* inst, int ninst, int nw, bool f32,
                                   const double* partials, cudaStream_t s) {
   if (f32)
-    gpp_batched_reduce_kernel<true><<<ninst, 256, 0, s>>>(inst, 4 * nw, partials);
+    gpp_batched_reduce_kernel<true><<<ninst * kReduceCtas, kReduceThreads, 0, s>>>(inst, 4 * nw, partials);
   else
-    gpp_batched_reduce_kernel<false><<<ninst, 256, 0, s>>>(inst, 4 * nw, partials);
+    gpp_batched_reduce_kernel<false><<<ninst * kReduceCtas, kReduceThreads, 0, s>>>(inst, 4 * nw, partials);
   return cudaGetLastError();
 }
 

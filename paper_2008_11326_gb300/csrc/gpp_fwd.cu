@@ -38,9 +38,8 @@ namespace gpp {
 
 namespace {
 
-// Band count up to which the gather offers the split-integer form (each of its blocks reads
-// all the frequencies).
-constexpr int64_t kFixMaxBands = 16384;
+// Band count up to which every table block of the gather reads all the frequencies.
+constexpr int64_t kScanBands = 16384;
 
 // Global column of local column p, or -1 if it contributes nothing. Counts indices that
 // are outside their arrays (the sentinel indinv[k] == G is legitimate).
@@ -59,99 +58,128 @@ __device__ __forceinline__ int column_of(int64_t p, int64_t G, const int32_t* in
   return g < G ? static_cast<int>(g) : -1;
 }
 
-// Column gather (paper §III v7: aqsmtemp_local(igp, band) stored band-contiguous),
-// band tables and index checks. am32 / bt32 (the FP32-bulk copies) may be NULL. For a
-// single-instance call the kernel also writes the instance descriptor the main kernel
-// reads (so the call needs no host-to-device copy and can be captured in a graph).
-__global__ void gpp_prep_kernel(int64_t B, int64_t G, int64_t P, int W,
-                                const double2* __restrict__ aqsm,
-                                const double* __restrict__ vcoul,
-                                const int32_t* __restrict__ inv,
-                                const int32_t* __restrict__ indinv,
-                                const double* __restrict__ wx, int* flags, int* colg,
-                                BandEntry* bt, double2* am, float4* bt32, float2* am32,
-                                bool want_fix, BatchInst* desc_out, const BatchInst desc) {
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  const int64_t tid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (desc_out && tid == 0) *desc_out = desc;
-  for (int64_t p = tid; p < P; p += stride) colg[p] = column_of(p, G, inv, indinv, flags + 1);
-  for (int64_t i = tid; i < P * B; i += stride) {
-    int64_t p = i / B, b = i - p * B;
-    int g = column_of(p, G, inv, indinv, nullptr);
-    double2 v = make_double2(0.0, 0.0);
-    if (g >= 0) {
-      double2 m = aqsm[b * G + g];
-      double vc = vcoul[g];
-      v = make_double2(m.x * vc, -m.y * vc);
-    }
-    am[i] = v;
-    if (am32) am32[i] = make_float2(static_cast<float>(v.x), static_cast<float>(v.y));
-  }
-  // For the FP64 sum's split-integer form, every block that writes band-table entries forms
-  // the ranges of the frequencies itself (a few KB from L2; 8 / W warps share a frequency), so
-  // that the table's split form and the flags need no second launch.
-  FixInfo fix{0, 0, 0.0, 0.0};
-  if (want_fix && static_cast<int64_t>(blockIdx.x) * blockDim.x < B * W) {
-    __shared__ double s_lo[8], s_hi[8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;   // 8 warps, W <= 8
-    const int iw = warp % W, part = warp / W, parts = 8 / W;
-    if (part < parts) {
-      double lo = INFINITY, hi = -INFINITY;
-#pragma unroll 4
-      for (int64_t b = part * 32 + lane; b < B; b += parts * 32) {
-        const double x = wx[b * W + iw];
-        lo = x >= 0.0 ? fmin(lo, x) : -INFINITY;   // a negative or NaN frequency: out of range
-        hi = fmax(hi, x);
-      }
+// max / min over the block of one value per thread (256 threads); every thread gets the result.
+// `buf`: 8 entries of shared memory per call.
+template <class T, class Op>
+__device__ __forceinline__ T block_fold(T v, T* buf, Op op) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-      }
-      if (lane == 0) {
-        s_lo[warp] = lo;
-        s_hi[warp] = hi;
+  for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(0xffffffffu, v, o));
+  if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = buf[0];
+#pragma unroll
+  for (int k = 1; k < 8; ++k) v = op(v, buf[k]);
+  return v;
+}
+
+// One block's share of the gather of an instance: its first `table_blocks` blocks write the
+// band tables and the flags, the others gather columns (paper §III v7: aqsmtemp_local(igp,
+// band) stored band-contiguous), one column per warp so that the column's index chain
+// (inv_igp_index, indinv, vcoul) is read once and the bands' loads are independent. A
+// single-instance call also writes the instance descriptor the main kernel reads and clears
+// its tile counter (so the call needs no host-to-device copy and no memset, and can be
+// captured in a graph).
+__device__ __forceinline__ void prep_block(const PrepArgs& a, int block, int nblocks) {
+  const int64_t B = a.B, G = a.G, P = a.P;
+  const int W = a.W, lane = threadIdx.x & 31;
+  if (block >= a.table_blocks) {
+    const int64_t nwarps = static_cast<int64_t>(nblocks - a.table_blocks) * 8;
+    for (int64_t p = static_cast<int64_t>(block - a.table_blocks) * 8 + (threadIdx.x >> 5); p < P;
+         p += nwarps) {
+      const int g = column_of(p, G, a.inv, a.indinv, lane == 0 && a.debug ? a.flags + 1 : nullptr);
+      const double vc = g >= 0 ? a.vcoul[g] : 0.0;
+      if (lane == 0) a.colg[p] = g;
+#pragma unroll 4
+      for (int64_t b = lane; b < B; b += 32) {
+        double2 v = make_double2(0.0, 0.0);
+        if (g >= 0) {
+          const double2 m = a.aqsm[b * G + g];
+          v = make_double2(m.x * vc, -m.y * vc);
+        }
+        a.am[p * B + b] = v;
+        if (a.am32) a.am32[p * B + b] = make_float2(static_cast<float>(v.x), static_cast<float>(v.y));
       }
     }
-    __syncthreads();
-    double lo = s_lo[0], hi = s_hi[0];
-    for (int k = 1; k < parts * W; ++k) {
-      lo = fmin(lo, s_lo[k]);
-      hi = fmax(hi, s_hi[k]);
+    return;
+  }
+  // The flags, and for the FP64 sum's split-integer form the ranges of the frequencies: every
+  // table block reads all of them (a few KB from L2) and the first writes the result, so that
+  // neither a second launch nor atomics are needed; with more bands than kScanBands each block
+  // raises the flags for its own entries instead, after a memset.
+  __shared__ double s_lo[8], s_hi[8];
+  __shared__ unsigned long long s_max[8];
+  if (a.desc_out && block == 0 && threadIdx.x == 0) {
+    *a.desc_out = a.desc;
+    *a.counter = 0;
+  }
+  const int64_t n = B * W;
+  const int64_t i0 = static_cast<int64_t>(block) * blockDim.x + threadIdx.x;
+  FixInfo fix{0, 0, 0.0, 0.0};
+  auto bits = [](double x) { return static_cast<unsigned long long>(__double_as_longlong(fabs(x))); };
+  if (a.scan) {
+    double lo = INFINITY, hi = -INFINITY;   // of all frequencies; -inf for a negative one or NaN
+    unsigned long long top = 0;             // the bits of max |wx|
+#pragma unroll 4
+    for (int64_t i = threadIdx.x; i < n; i += 256) {
+      const double x = a.wx[i];
+      lo = x >= 0.0 ? fmin(lo, x) : -INFINITY;
+      hi = fmax(hi, x);
+      top = max(top, bits(x));
     }
-    fix = fix_info(lo, hi);
-    if (blockIdx.x == 0 && threadIdx.x < W) {
-      double* range = reinterpret_cast<double*>(flags + kFlagRange);
-      double l = s_lo[threadIdx.x], h = s_hi[threadIdx.x];
-      for (int k = 1; k < parts; ++k) {
-        l = fmin(l, s_lo[k * W + threadIdx.x]);
-        h = fmax(h, s_hi[k * W + threadIdx.x]);
+    top = block_fold(top, s_max, [](unsigned long long u, unsigned long long v) { return max(u, v); });
+    lo = block_fold(lo, s_lo, [](double u, double v) { return fmin(u, v); });
+    hi = block_fold(hi, s_hi, [](double u, double v) { return fmax(u, v); });
+    if (a.want_fix) fix = fix_info(lo, hi);
+    if (block == 0) {
+      if (threadIdx.x == 0) {
+        a.flags[0] = lo >= 0.0 ? 0 : 1;
+        a.flags[2] = top < bits(kFp32MaxX) ? 0 : 1;
+        if (!a.debug) a.flags[1] = 0;
+        *reinterpret_cast<unsigned long long*>(a.flags + kFlagXmax) = top;
       }
-      range[threadIdx.x] = l;
-      range[kMaxNw + threadIdx.x] = h;
+      double* range = reinterpret_cast<double*>(a.flags + kFlagRange);
+      for (int iw = threadIdx.x >> 5; fix.ok && iw < W; iw += 8) {   // a warp per frequency
+        double l = INFINITY, h = -INFINITY;
+#pragma unroll 4
+        for (int64_t b = lane; b < B; b += 32) {
+          const double x = a.wx[b * W + iw];
+          l = fmin(l, x);
+          h = fmax(h, x);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          l = fmin(l, __shfl_xor_sync(0xffffffffu, l, o));
+          h = fmax(h, __shfl_xor_sync(0xffffffffu, h, o));
+        }
+        if (lane == 0) {
+          range[iw] = l;
+          range[kMaxNw + iw] = h;
+        }
+      }
     }
   }
-  if (tid == 0) *reinterpret_cast<FixInfo*>(flags + kFlagFix) = fix;
-  for (int64_t i = tid; i < B * W; i += stride) {
-    double x = wx[i];
-    bt[i] = BandEntry{make_double2(x, x * x), fix.ok ? fix_x(x, fix.E) : make_int4(0, 0, 0, 0)};
-    if (!(x >= 0.0)) flags[0] = 1;
-    if (!(fabs(x) < kFp32MaxX)) flags[2] = 1;
-    // max |wx|: non-negative doubles order as their bit patterns
-    atomicMax(reinterpret_cast<unsigned long long*>(flags + kFlagXmax),
-              static_cast<unsigned long long>(__double_as_longlong(fabs(x))));
-    if (bt32) {  // layout of f32_band_quads (gpp_device.cuh)
+  if (i0 == 0) *reinterpret_cast<FixInfo*>(a.flags + kFlagFix) = fix;
+  for (int64_t i = i0; i < n; i += static_cast<int64_t>(a.table_blocks) * 256) {
+    const double x = a.wx[i];
+    a.bt[i] = BandEntry{make_double2(x, x * x), fix.ok ? fix_x(x, fix.E) : make_int4(0, 0, 0, 0)};
+    if (!a.scan) {
+      if (!(x >= 0.0)) a.flags[0] = 1;
+      if (!(fabs(x) < kFp32MaxX)) a.flags[2] = 1;
+      // max |wx|: non-negative doubles order as their bit patterns
+      atomicMax(reinterpret_cast<unsigned long long*>(a.flags + kFlagXmax), bits(x));
+    }
+    if (a.bt32) {  // layout of f32_band_quads (gpp_device.cuh)
       const float xf = static_cast<float>(x);
       const int64_t b0 = i / W, iw = i - b0 * W;
       const int nq = (W + 4) / 4;
-      float* fb = reinterpret_cast<float*>(bt32 + b0 * (2 * nq));
+      float* fb = reinterpret_cast<float*>(a.bt32 + b0 * (2 * nq));
       fb[iw] = xf;
       fb[4 * nq + iw] = static_cast<float>(x - static_cast<double>(xf));
       if (iw == 0) {  // the band's frequency range, rounded outwards, and the padding
         float lo = __int_as_float(0x7f800000), hi = -lo;
         for (int k = 0; k < W; ++k) {
-          lo = fminf(lo, __double2float_rd(wx[b0 * W + k]));
-          hi = fmaxf(hi, __double2float_ru(wx[b0 * W + k]));
+          lo = fminf(lo, __double2float_rd(a.wx[b0 * W + k]));
+          hi = fmaxf(hi, __double2float_ru(a.wx[b0 * W + k]));
         }
         fb[W] = lo;
         fb[4 * nq + W] = hi;
@@ -159,6 +187,14 @@ __global__ void gpp_prep_kernel(int64_t B, int64_t G, int64_t P, int W,
       }
     }
   }
+}
+
+__global__ void __launch_bounds__(256) gpp_prep_kernel(const PrepArgs a) {
+  prep_block(a, blockIdx.x, gridDim.x);
+}
+// Many instances in one launch: blockIdx.y is the instance.
+__global__ void __launch_bounds__(256) gpp_prep_batch_kernel(const PrepArgs* __restrict__ list) {
+  prep_block(list[blockIdx.y], blockIdx.x, gridDim.x);
 }
 
 // Complex128 -> complex64 (round to nearest) over a block of rows x columns: the FP32-bulk
@@ -195,30 +231,74 @@ cudaError_t launch_convert_c64(const gpp_c128* src, int64_t ld_src, gpp_c64* dst
   return cudaGetLastError();
 }
 
-cudaError_t launch_prep(const gpp_problem& p, const FwdPlan& plan, char* ws, bool fp32,
+PrepArgs prep_args(const gpp_problem& p, const FwdPlan& plan, char* ws, bool fp32, bool debug) {
+  PrepArgs a;
+  a.B = p.number_bands;
+  a.G = p.ncouls;
+  a.P = p.ngpown;
+  a.W = static_cast<int>(p.nw);
+  a.aqsm = reinterpret_cast<const double2*>(p.aqsmtemp);
+  a.vcoul = p.vcoul;
+  a.inv = p.inv_igp_index;
+  a.indinv = p.indinv;
+  a.wx = p.wx_array;
+  a.flags = reinterpret_cast<int*>(ws + plan.off_flags);
+  a.colg = reinterpret_cast<int*>(ws + plan.off_colvalid);
+  a.bt = reinterpret_cast<BandEntry*>(ws + plan.off_bt);
+  a.am = reinterpret_cast<double2*>(ws + plan.off_am);
+  a.bt32 = fp32 ? reinterpret_cast<float4*>(ws + plan.off_bt32) : nullptr;
+  a.am32 = fp32 ? reinterpret_cast<float2*>(ws + plan.off_am32) : nullptr;
+  a.scan = p.number_bands <= kScanBands;
+  a.want_fix = !fp32;
+  a.debug = debug;
+  a.table_blocks = static_cast<int>(std::min<int64_t>((p.number_bands * p.nw + 255) / 256, 1024));
+  return a;
+}
+
+namespace {
+int prep_blocks(const PrepArgs& a) {
+  return a.table_blocks + static_cast<int>(std::min<int64_t>((a.P + 7) / 8, 4096));
+}
+// The flags start at zero where the kernel only raises them.
+cudaError_t prep_clear(const PrepArgs& a, cudaStream_t s) {
+  return a.scan && !a.debug ? cudaSuccess : cudaMemsetAsync(a.flags, 0, kFlagBytes, s);
+}
+}  // namespace
+
+cudaError_t launch_prep(const gpp_problem& p, const FwdPlan& plan, char* ws, bool fp32, bool debug,
                         const BatchInst* desc, cudaStream_t s) {
-  int* flags = reinterpret_cast<int*>(ws + plan.off_flags);
-  cudaError_t e = cudaMemsetAsync(flags, 0, kFlagBytes, s);
+  PrepArgs a = prep_args(p, plan, ws, fp32, debug);
+  cudaError_t e = prep_clear(a, s);
   if (e != cudaSuccess) return e;
   if (fp32 && plan.convert_c64) {
     e = launch_convert_c64(p.aqsntemp, p.ncouls, reinterpret_cast<gpp_c64*>(ws + plan.off_aqsn32),
                            p.ncouls, p.number_bands, 0, p.ncouls, s);
     if (e != cudaSuccess) return e;
   }
-  const bool want_fix = !fp32 && p.number_bands <= kFixMaxBands;
-  const int64_t work = p.ngpown * p.number_bands + p.number_bands * p.nw + p.ngpown;
-  int64_t blocks = (work + 255) / 256;
-  if (blocks < 1) blocks = 1;
-  if (blocks > 4096) blocks = 4096;
-  gpp_prep_kernel<<<static_cast<int>(blocks), 256, 0, s>>>(
-      p.number_bands, p.ncouls, p.ngpown, static_cast<int>(p.nw),
-      reinterpret_cast<const double2*>(p.aqsmtemp), p.vcoul, p.inv_igp_index, p.indinv,
-      p.wx_array, flags, reinterpret_cast<int*>(ws + plan.off_colvalid),
-      reinterpret_cast<BandEntry*>(ws + plan.off_bt), reinterpret_cast<double2*>(ws + plan.off_am),
-      fp32 ? reinterpret_cast<float4*>(ws + plan.off_bt32) : nullptr,
-      fp32 ? reinterpret_cast<float2*>(ws + plan.off_am32) : nullptr,
-      want_fix, desc ? reinterpret_cast<BatchInst*>(ws + plan.off_desc) : nullptr, desc ? *desc : BatchInst());
+  if (desc) {
+    a.desc = *desc;
+    a.desc_out = reinterpret_cast<BatchInst*>(ws + plan.off_desc);
+    a.counter = reinterpret_cast<unsigned long long*>(ws + plan.off_counter);
+  }
+  gpp_prep_kernel<<<prep_blocks(a), 256, 0, s>>>(a);
   return cudaGetLastError();
+}
+
+cudaError_t launch_prep_batch(const PrepArgs* host_list, const PrepArgs* dev_list, int n,
+                              cudaStream_t s) {
+  int blocks = 1;
+  for (int i = 0; i < n; ++i) {
+    cudaError_t e = prep_clear(host_list[i], s);
+    if (e != cudaSuccess) return e;
+    blocks = std::max(blocks, prep_blocks(host_list[i]));
+  }
+  for (int i = 0; i < n; i += 65535) {   // the grid's y limit
+    const int m = std::min(n - i, 65535);
+    gpp_prep_batch_kernel<<<dim3(blocks, m), 256, 0, s>>>(dev_list + i);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace gpp

@@ -42,11 +42,6 @@ inline size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
 struct BatchInst;
 
-// Column gather, band tables and index checks (one kernel); with `desc` it also writes the
-// single-instance descriptor to plan.off_desc. With plan.convert_c64 the complex64 copy of
-// aqsntemp is written to plan.off_aqsn32 first.
-cudaError_t launch_prep(const gpp_problem& p, const FwdPlan& plan, char* ws, bool fp32,
-                        const BatchInst* desc, cudaStream_t s);
 // dst[r][c] = complex64(src[r][c]) (round to nearest) for rows [0, rows) and columns
 // [c0, c1); leading dimensions in elements.
 cudaError_t launch_convert_c64(const gpp_c128* src, int64_t ld_src, gpp_c64* dst, int64_t ld_dst,
@@ -93,15 +88,49 @@ struct BatchInst {
   double sx2 = 0.0;        // sexcut^2 with GPP_PHYS_SX_CUTOFF, else 0
 };
 
+// What the gather kernel reads and writes for one instance. counter and desc: only with
+// desc_out (a single-instance call).
+struct PrepArgs {
+  int64_t B = 0, G = 0, P = 0;
+  int W = 0, table_blocks = 0;
+  const double2* aqsm = nullptr;
+  const double* vcoul = nullptr;
+  const int32_t* inv = nullptr;
+  const int32_t* indinv = nullptr;
+  const double* wx = nullptr;
+  int* flags = nullptr;
+  int* colg = nullptr;
+  BandEntry* bt = nullptr;
+  double2* am = nullptr;
+  float4* bt32 = nullptr;
+  float2* am32 = nullptr;
+  bool scan = false, want_fix = false, debug = false;
+  unsigned long long* counter = nullptr;
+  BatchInst* desc_out = nullptr;
+  BatchInst desc;
+};
+PrepArgs prep_args(const gpp_problem& p, const FwdPlan& plan, char* ws, bool fp32, bool debug);
+
+// Column gather, band tables and index checks (one kernel; `debug` counts bad indices); with
+// `desc` it also writes the single-instance descriptor to plan.off_desc and clears the tile
+// counter at plan.off_counter. With plan.convert_c64 the complex64 copy of aqsntemp is written
+// to plan.off_aqsn32 first.
+cudaError_t launch_prep(const gpp_problem& p, const FwdPlan& plan, char* ws, bool fp32, bool debug,
+                        const BatchInst* desc, cudaStream_t s);
+// The gathers of a batch in one launch (the list in host and in device memory).
+cudaError_t launch_prep_batch(const PrepArgs* host_list, const PrepArgs* dev_list, int n,
+                              cudaStream_t s);
+
 // Lets the main kernel take the shared memory the launch shape needs; before occupancy
 // queries and launches.
 cudaError_t batched_prepare(int threads, int nw, bool f32, int igpt);
 int batched_blocks_per_sm(int threads, int nw, bool f32, int igpt);
-// Resets the tile counter and runs the persistent main kernel over tiles [t_begin, ntiles).
+// Runs the persistent main kernel over tiles [t_begin, ntiles), after clearing the tile
+// counter unless it is `cleared` already.
 cudaError_t launch_batched_main(const BatchInst* inst, int ninst, int64_t ntiles, int nw,
                                 bool f32, int grid, int threads, int igpt,
-                                unsigned long long* counter, double* partials, cudaStream_t s,
-                                int64_t t_begin = 0);
+                                unsigned long long* counter, bool cleared, double* partials,
+                                cudaStream_t s, int64_t t_begin = 0);
 // Per-instance fixed-order sum of the tile partials into the outputs.
 cudaError_t launch_batched_reduce(const BatchInst* inst, int ninst, int nw, bool f32,
                                   const double* partials, cudaStream_t s);
