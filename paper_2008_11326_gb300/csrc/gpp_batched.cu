@@ -150,6 +150,7 @@ __device__ __forceinline__ void f64_body(const BatchInst* __restrict__ inst, int
     const bool col_ok = d.colg[p] >= 0;
     const bool x_fast = d.flags[0] == 0;
     const FixInfo fix = *reinterpret_cast<const FixInfo*>(d.flags + kFlagFix);
+    const bool fix_on = fix.ok == 1 || (fix.ok == 2 && d.sx2 > 0.0);
     const double* xrange = reinterpret_cast<const double*>(d.flags + kFlagRange);
     const double2* am = d.am + p * B;
 #pragma unroll
@@ -166,10 +167,15 @@ __device__ __forceinline__ void f64_body(const BatchInst* __restrict__ inst, int
       }
       const double2* an = d.aqsn + (live ? ig : 0);
       const double wabs2 = fma(w.x, w.x, w.y * w.y);
-      if (fix.ok && __all_sync(0xffffffffu, fix_lane(w, wabs2, fix) || !live) &&
-          fix_band_loop<W>(B, G, nocc, an, am, d.bt, live, w, live ? d.wt + p * G + ig : d.wt, I,
-                           fix.E, xrange, dyn_smem, acc))
-        continue;
+      if (fix_on && __all_sync(0xffffffffu, fix_lane(w, wabs2, fix) || !live)) {
+        const double2* w64 = live ? d.wt + p * G + ig : d.wt;
+        const bool done =
+            fix.ok == 1 ? fix_band_loop<W, false>(B, G, nocc, an, am, d.bt, live, w, w64, I, fix.E,
+                                                  0.0, xrange, dyn_smem, acc)
+                        : fix_band_loop<W, true>(B, G, nocc, an, am, d.bt, live, w, w64, I, fix.E,
+                                                 d.sx2, xrange, dyn_smem, acc);
+        if (done) continue;
+      }
       // the FP64 fast form's conditions, with the partial fractions' bound on x / |w|
       const bool fast_lane = w.x >= 0.0 && gt_nonneg(wabs2, kFastWabs2Lo) &&
                              lt_nonneg(wabs2, kFastWabs2Hi) &&

@@ -106,7 +106,7 @@ __device__ __forceinline__ void prep_block(const PrepArgs& a, int block, int nbl
   // table block reads all of them (a few KB from L2) and the first writes the result, so that
   // neither a second launch nor atomics are needed; with more bands than kScanBands each block
   // raises the flags for its own entries instead, after a memset.
-  __shared__ double s_lo[8], s_hi[8];
+  __shared__ double s_lo[8];
   __shared__ unsigned long long s_max[8];
   if (a.desc_out && block == 0 && threadIdx.x == 0) {
     *a.desc_out = a.desc;
@@ -117,22 +117,21 @@ __device__ __forceinline__ void prep_block(const PrepArgs& a, int block, int nbl
   FixInfo fix{0, 0, 0.0, 0.0};
   auto bits = [](double x) { return static_cast<unsigned long long>(__double_as_longlong(fabs(x))); };
   if (a.scan) {
-    double lo = INFINITY, hi = -INFINITY;   // of all frequencies; -inf for a negative one or NaN
-    unsigned long long top = 0;             // the bits of max |wx|
+    double lo = INFINITY;         // the least frequency (NaN apart)
+    unsigned long long top = 0;   // the bits of max |wx| (NaN above infinity)
 #pragma unroll 4
     for (int64_t i = threadIdx.x; i < n; i += 256) {
       const double x = a.wx[i];
-      lo = x >= 0.0 ? fmin(lo, x) : -INFINITY;
-      hi = fmax(hi, x);
+      lo = fmin(lo, x);
       top = max(top, bits(x));
     }
     top = block_fold(top, s_max, [](unsigned long long u, unsigned long long v) { return max(u, v); });
     lo = block_fold(lo, s_lo, [](double u, double v) { return fmin(u, v); });
-    hi = block_fold(hi, s_hi, [](double u, double v) { return fmax(u, v); });
-    if (a.want_fix) fix = fix_info(lo, hi);
+    const double xmax = __longlong_as_double(static_cast<long long>(top));
+    if (a.want_fix) fix = fix_info(lo, xmax);
     if (block == 0) {
       if (threadIdx.x == 0) {
-        a.flags[0] = lo >= 0.0 ? 0 : 1;
+        a.flags[0] = lo >= 0.0 && xmax == xmax ? 0 : 1;
         a.flags[2] = top < bits(kFp32MaxX) ? 0 : 1;
         if (!a.debug) a.flags[1] = 0;
         *reinterpret_cast<unsigned long long*>(a.flags + kFlagXmax) = top;

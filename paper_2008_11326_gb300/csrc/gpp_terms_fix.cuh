@@ -32,7 +32,8 @@
 // 1.9e-16 / 2.0, 2.1 / 2.1, 2.2 / 2.4, 2.5 for 1 / 5 / 64 / 200 bands; the FP64 form: 1.8,
 // 2.8 / 2.1, 2.4 / 3.1, 3.6 / 4.4, 5.0.
 //
-// Range (fix_lane, FixInfo): 0 <= x <= 48, Re w >= 0, 2^(E-7) <= |w| <= 1.375 2^E - max x with
+// Range (fix_lane, FixInfo): |x| <= 48, x >= 0 unless the screened-exchange cutoff bounds the
+// terms near x = -w, Re w >= 0, 2^(E-7) <= |w| <= 1.375 2^E - max x with
 // the binary scale E of the instance's frequencies; weights whose row and column maxima over
 // the bands are finite and of ordinary exponent, and whose largest product over the bands is
 // within 2^-7 of the product of those maxima (the product of the split weights is exact to
@@ -46,6 +47,7 @@ namespace gpp {
 constexpr int kStageBands = 64;    // bands of one warp's staged weights in shared memory
 constexpr int kLowBands = 8;       // bands between moves of the FP32 low sums to the integers
 constexpr int kFlushBands = 1024;  // bands of the modular sums between flushes
+constexpr int kFixMaxGroup = 3;    // frequencies per group: more accumulators would not fit
 constexpr float kFixKappa = 1.0f - 0x1p-12f;
 constexpr float kFixNear = 0x1p-20f;  // |(|wdiff|^2 - 1/4)| below which FP64 decides
 constexpr int kFixMinTop = 55;        // fewest bits of the largest weight (of at most 62)
@@ -91,11 +93,12 @@ __device__ __forceinline__ int mad_lo(int a, int b, int c) {
   return d;
 }
 
-// What the split-integer form needs to know of an instance's frequencies, which lie in
-// [xmin, xmax]: whether they are in its range, the binary scale E, and the bounds on |w|^2.
+// What the split-integer form needs to know of an instance's frequencies, whose least is xmin
+// and whose largest magnitude is xmax: whether they are in its range (1: all >= 0, 2: some
+// negative), the binary scale E, and the bounds on |w|^2.
 __device__ __forceinline__ FixInfo fix_info(double xmin, double xmax) {
   FixInfo f;
-  f.ok = xmin >= 0.0 && xmax <= 48.0;
+  f.ok = !(xmax <= 48.0) ? 0 : xmin >= 0.0 ? 1 : 2;
   int E = 2;
   while (E < 6 && xmax > 0.75 * static_cast<double>(1 << E)) ++E;
   const double lim = 1.375 * static_cast<double>(1 << E) - xmax;
@@ -133,6 +136,7 @@ __device__ __forceinline__ int4 fix_x(double x, int E) {
   int hi, lo;
   float a, b;
   fix_value(x, (62 - E) << 20, hi, lo);
+  if (x < 0.0 && hi == 0 && lo == 0) lo = -1;   // the sign tells the cutoff's terms
   fix_floats(hi, lo, E, a, b);
   return make_int4(hi, lo, __float_as_int(a), __float_as_int(b));
 }
@@ -187,8 +191,8 @@ __device__ __forceinline__ FixN fix_norm(const FixPair& w, float xa, float xb) {
 }
 
 // 1/(Ar - i wi) with Ar = x - Re w (SIDE_A) or x + Re w (then that is conj(v)), from its norm;
-// zero where `on` is false.
-template <bool SIDE_A>
+// with MASK zero where `on` is false.
+template <bool SIDE_A, bool MASK>
 __device__ __forceinline__ FixU fix_term(const FixPair& w, const FixN& n, int xh, int xl, float2 sc,
                                          bool on) {
   FixU o;
@@ -198,7 +202,7 @@ __device__ __forceinline__ FixU fix_term(const FixPair& w, const FixN& n, int xh
   const int Al = static_cast<int>(a64);
   const int Ah = static_cast<int>(a64 >> 32) - (Al >> 31);   // signed low word
   float rho = fix_rcp(fmaf(n.N1, 1.0f + 0x1p-12f, n.Nm));    // kappa / |A|^2
-  if (SIDE_A) rho = on ? rho : 0.0f;
+  if (MASK) rho = on ? rho : 0.0f;
   float eps = fmaf(-rho, n.N1, kFixKappa);                   // kappa - rho |A|^2
   eps = fmaf(-rho, n.Nm, eps);
   const float rs = rho * sc.x, re = rs * eps;
@@ -237,9 +241,6 @@ __host__ __device__ constexpr size_t fix_smem_bytes(int threads, int wg) {
   return static_cast<size_t>(threads) * (4 * wg * 8 + 2 * wg * 8) +
          static_cast<size_t>(threads / 32) * kStageBands * sizeof(FixAm);
 }
-
-// Largest frequency group: more accumulators than 16 x 3 would not fit the register budget.
-constexpr int kFixMaxGroup = 3;
 
 // The weight M = am an of a band, times 2^(ka + kn - sh): M1 + M0.
 struct FixM {
@@ -283,18 +284,36 @@ struct FixCtx {
   FixAm* stage;
 };
 
+// The screened-exchange cutoff (negative frequencies only): a term whose |ssx| / |I|, which is
+// |w|^2 / (|A| |S|) on branch 1 and |w| / (2 |S|) on branch 2, exceeds sexcut leaves asxtemp.
+// So |w|^4 > sx2 |S|^2 (branch 1: |A|^2, branch 2: 4 |w|^2) is tested, in FP32 and, within
+// kFixNearCut of equality, in FP64 as the general form does. A kept term has
+//   |S| >= |w| min(sqrt(1 + 1 / sexcut) - 1, 1 / (2 sexcut)),
+// which bounds v near x = -w; v there, above the bound the sums are scaled for, is taken at a
+// scale 2^-delta and its product shifted back (the sums are modular).
+constexpr float kFixNearCut = 0x1p-18f;
+struct FixCut {
+  float w4, w24, sx2f;   // |w|^4, 4 |w|^2
+  double sx2;
+  int delta[kFixMaxGroup];
+};
+
 // Bands [b0, b1) of the thread's pair, WG frequencies from iw0, into the thread's FP64 sums
 // st[k blockDim.x] (units of kappa 2^ks M with the ks of u; values 4 iw + {0, 1}: sum M u, and
 // with OCC + {2, 3}: sum M u - sum M v), added to them, or with `fresh` replacing them.
-template <int WG, bool OCC>
+template <int WG, bool OCC, bool CUT>
 __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixCtx& ctx, int iw0,
-                                          const FixPair& w, double* st, const float2* sc) {
+                                          const FixPair& w, const FixCut& cut, double* st,
+                                          const float2* sc) {
   const int nt = blockDim.x, lane = threadIdx.x & 31;
   const int64_t G = ctx.G;
   FixAm* const stage = ctx.stage;
+  // bands of the modular sums: the FP32 sum beside them has to be good to 2^62 (terms below
+  // 2^62, with the cutoff's scale 2^69)
+  constexpr int kFlush = CUT ? 128 : kFlushBands;
 #pragma unroll 1
-  for (int f0 = b0; f0 < b1; f0 += kFlushBands) {
-    const int f1 = min(f0 + kFlushBands, b1);
+  for (int f0 = b0; f0 < b1; f0 += kFlush) {
+    const int f1 = min(f0 + kFlush, b1);
     long long acc[4 * WG];
     float aH[4 * WG], aL[4 * WG];
 #pragma unroll
@@ -347,7 +366,7 @@ __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixC
 #pragma unroll
           for (int k = 0; k < WG; ++k) {
             {
-              const FixU u = fix_term<true>(w, na[k], xv[k].x, xv[k].y, sc[2 * k * nt], d[k] > 0.0f);
+              const FixU u = fix_term<true, true>(w, na[k], xv[k].x, xv[k].y, sc[2 * k * nt], d[k] > 0.0f);
               acc[4 * k] = mad_wide(m.r1, u.Ur, mad_wide(m.ni1, u.Ui, acc[4 * k]));
               acc[4 * k + 1] = mad_wide(m.r1, u.Ui, mad_wide(m.i1, u.Ur, acc[4 * k + 1]));
               aH[4 * k] = fmaf(m.r1f, u.ur, fmaf(-m.i1f, u.ui, aH[4 * k]));
@@ -357,7 +376,51 @@ __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixC
             }
             if (OCC) {   // v = conj of the computed value
               const FixN ns = fix_norm<false>(w, __int_as_float(xv[k].z), __int_as_float(xv[k].w));
-              const FixU u = fix_term<false>(w, ns, xv[k].x, xv[k].y, sc[(2 * k + 1) * nt], true);
+              const float2 ss = sc[(2 * k + 1) * nt];
+              bool on = true;
+              if (CUT && (xv[k].x < 0 || (xv[k].x == 0 && xv[k].y < 0))) {   // x < 0: warp-uniform
+                const float NS = ns.N1 + ns.Nm;
+                const bool b1 = d[k] > 0.0f;
+                const float lim = cut.sx2f * NS * (b1 ? na[k].N1 + na[k].Nm : cut.w24);
+                bool drop = cut.w4 > lim;
+                const bool edge = fabsf(cut.w4 - lim) <= kFixNearCut * cut.w4;
+                if (__any_sync(0xffffffffu, edge)) {
+                  const double2 wv = ldg2(ctx.w64);
+                  const double x = __ldg(&btb[k].lo.x), a = x - wv.x, s = x + wv.x, i2 = wv.y * wv.y;
+                  const double A2 = fma(a, a, i2), S2 = fma(s, s, i2), w2 = fma(wv.x, wv.x, i2);
+                  const bool e = b1 ? gt_nonneg(w2 * w2 * rcp_refined(A2 * S2), cut.sx2)
+                                    : gt_nonneg(w2, 4.0 * cut.sx2 * S2);
+                  drop = edge ? e : drop;
+                }
+                // |S| below 2^(31 - ks): beyond this scale
+                const int e = __float_as_int(ss.x) >> 23;   // ks + 127
+                const bool small = !drop && NS < __int_as_float((443 - 2 * e) << 23);
+                on = !drop && !small;
+                if (__any_sync(0xffffffffu, drop && b1)) {   // take sum M u back out of asxtemp
+                  const FixU u = fix_term<true, true>(w, na[k], xv[k].x, xv[k].y, ss, drop && b1);
+                  acc[4 * k + 2] = mad_wide(m.r1, u.Ur, mad_wide(m.ni1, u.Ui, acc[4 * k + 2]));
+                  acc[4 * k + 3] = mad_wide(m.r1, u.Ui, mad_wide(m.i1, u.Ur, acc[4 * k + 3]));
+                  aH[4 * k + 2] = fmaf(m.r1f, u.ur, fmaf(-m.i1f, u.ui, aH[4 * k + 2]));
+                  aH[4 * k + 3] = fmaf(m.r1f, u.ui, fmaf(m.i1f, u.ur, aH[4 * k + 3]));
+                  aL[4 * k + 2] += fmaf(m.r1f, u.gr, fmaf(-m.i1f, u.gi, fmaf(m.r0, u.ur, -m.i0 * u.ui)));
+                  aL[4 * k + 3] += fmaf(m.r1f, u.gi, fmaf(m.i1f, u.gr, fmaf(m.r0, u.ui, m.i0 * u.ur)));
+                }
+                if (__any_sync(0xffffffffu, small)) {
+                  const int dl = cut.delta[k];
+                  const float up = exp2if(dl);
+                  const FixU u = fix_term<false, true>(w, ns, xv[k].x, xv[k].y,
+                                                       make_float2(ss.x * exp2if(-dl), ss.y * up), small);
+                  const long long pr = mad_wide(m.r1, u.Ur, mad_wide(m.i1, u.Ui, 0));
+                  const long long pi = mad_wide(m.i1, u.Ur, mad_wide(m.nr1, u.Ui, 0));
+                  acc[4 * k + 2] += static_cast<long long>(static_cast<unsigned long long>(pr) << dl);
+                  acc[4 * k + 3] += static_cast<long long>(static_cast<unsigned long long>(pi) << dl);
+                  aH[4 * k + 2] = fmaf(up, fmaf(m.r1f, u.ur, m.i1f * u.ui), aH[4 * k + 2]);
+                  aH[4 * k + 3] = fmaf(up, fmaf(m.i1f, u.ur, -m.r1f * u.ui), aH[4 * k + 3]);
+                  aL[4 * k + 2] = fmaf(up, fmaf(m.r1f, u.gr, fmaf(m.i1f, u.gi, fmaf(m.r0, u.ur, m.i0 * u.ui))), aL[4 * k + 2]);
+                  aL[4 * k + 3] = fmaf(up, fmaf(m.i1f, u.gr, fmaf(-m.r1f, u.gi, fmaf(m.i0, u.ur, -m.r0 * u.ui))), aL[4 * k + 3]);
+                }
+              }
+              const FixU u = fix_term<false, CUT>(w, ns, xv[k].x, xv[k].y, ss, on);
               acc[4 * k + 2] = mad_wide(m.r1, u.Ur, mad_wide(m.i1, u.Ui, acc[4 * k + 2]));
               acc[4 * k + 3] = mad_wide(m.i1, u.Ur, mad_wide(m.nr1, u.Ui, acc[4 * k + 3]));
               aH[4 * k + 2] = fmaf(m.r1f, u.ur, fmaf(m.i1f, u.ui, aH[4 * k + 2]));
@@ -367,13 +430,13 @@ __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixC
             }
           }
         }
-        // the low sums (below 2^36) into the integer sums in units of 2^6; the rest stays
+        // the low sums (below 2^43) into the integer sums in units of 2^12; the rest stays
 #pragma unroll
         for (int k = 0; k < 4 * WG; ++k)
           if (OCC || (k & 2) == 0) {
-            const int r = __float2int_rn(aL[k] * 0x1p-6f);
-            acc[k] = mad_wide(r, 64, acc[k]);
-            aL[k] = fmaf(-64.0f, static_cast<float>(r), aL[k]);
+            const int r = __float2int_rn(aL[k] * 0x1p-12f);
+            acc[k] = mad_wide(r, 4096, acc[k]);
+            aL[k] = fmaf(-4096.0f, static_cast<float>(r), aL[k]);
           }
       }
     }
@@ -438,12 +501,12 @@ __device__ __forceinline__ bool fix_exponent(unsigned m, int& k) {
 
 // All bands of the thread's pair by the split-integer form, multiplied by Iw = I w and added
 // to tacc[4 W]. Returns false (nothing added) if any lane of the warp is out of range. B >= 1.
-template <int W>
+template <int W, bool CUT>
 __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
                                            const double2* __restrict__ an_ptr,
                                            const double2* __restrict__ am_ptr,
                                            const BandEntry* __restrict__ bt, bool live, double2 wv,
-                                           const double2* __restrict__ w_ptr, double2 I, int E,
+                                           const double2* __restrict__ w_ptr, double2 I, int E, double sx2,
                                            const double* __restrict__ xrange, unsigned char* smem,
                                            double* tacc) {
   constexpr int WG = W < kFixMaxGroup ? W : kFixMaxGroup;
@@ -474,6 +537,17 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
                        warp * kStageBands};
   const FixPair w = fix_pair(wv, E);
   const double Iwr = fma(I.x, wv.x, -I.y * wv.y), Iwi = fma(I.x, wv.y, I.y * wv.x);
+  const float w2f = fmaf(w.w1, w.w1, w.i1 * w.i1);
+  float dcut = 0.0f;   // the least |S| of a kept term with x < 0
+  FixCut cut{w2f * w2f, 4.0f * w2f, static_cast<float>(sx2), sx2, {}};
+  if (CUT) {
+    const float sc = sqrtf(cut.sx2f);
+    dcut = sqrtf(w2f) * fminf(1.0f, fminf(sqrtf(1.0f + 1.0f / sc) - 1.0f, 0.5f / sc)) * (1.0f - 0x1p-17f);
+    // a cutoff so high that its least |S| needs a scale far from the others', or so low that
+    // its tests leave FP32's range
+    const bool good = dcut >= 0x1p-6f * fminf(sqrtf(w2f), 0.25f) && sc > 0x1p-20f;
+    if (!__all_sync(0xffffffffu, good)) return false;
+  }
   auto group = [&](auto tag, int iw0) {
     constexpr int N = decltype(tag)::value;
     int ks[2 * N];
@@ -483,9 +557,17 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
       const float lo = static_cast<float>(xrange[iw0 + k]);
       const float hi = static_cast<float>(xrange[kMaxNw + iw0 + k]);
       const float dA = fmaxf(0.5f, fmaxf(lo - w.w1, w.w1 - hi) * (1.0f - 0x1p-17f));
-      const float sr = lo + w.w1;
+      const float sr = fmaxf(lo + w.w1, -(hi + w.w1));
+      const float dr = CUT ? fmaxf(sr, 0.0f) : sr;
+      float dS2 = fmaf(dr, dr, w.i1 * w.i1) * (1.0f - 0x1p-17f);
+      if (CUT) {
+        // the scale of most terms, and how far below it the kept terms near x = -w may lie
+        const float least = fmaxf(dS2, dcut * dcut), most = fminf(w2f * (1.0f - 0x1p-17f), 0.0625f);
+        dS2 = fmaxf(least, most);
+        cut.delta[k] = fix_ks(dS2) - fix_ks(least);
+      }
       ks[2 * k] = fix_ks(dA * dA);
-      ks[2 * k + 1] = fix_ks(fmaf(sr, sr, w.i1 * w.i1) * (1.0f - 0x1p-17f));
+      ks[2 * k + 1] = fix_ks(dS2);
       sc[2 * k * nt] = fix_scale(ks[2 * k], E);
       sc[(2 * k + 1) * nt] = fix_scale(ks[2 * k + 1], E);
     }
@@ -495,7 +577,7 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
 #pragma unroll
     for (int k = 0; k < 2 * N; ++k) ax[k] = 0.0;
     if (nocc > 0) {
-      fix_range<N, true>(0, nocc, true, ctx, iw0, w, st, sc);
+      fix_range<N, true, CUT>(0, nocc, true, ctx, iw0, w, cut, st, sc);
 #pragma unroll
       for (int k = 0; k < N; ++k) {
         const double fa = exp2i(ex - ks[2 * k] - 1) * (1.0 / kFixKappa);
@@ -503,7 +585,7 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
         ax[2 * k + 1] = fa * st[(4 * k + 3) * nt];
       }
     }
-    if (nocc < B) fix_range<N, false>(nocc, B, nocc == 0, ctx, iw0, w, st, sc);
+    if (nocc < B) fix_range<N, false, false>(nocc, B, nocc == 0, ctx, iw0, w, cut, st, sc);
 #pragma unroll
     for (int k = 0; k < N; ++k) {   // tacc += I w times the pair's sums
       const double fa = exp2i(ex - ks[2 * k]) * (1.0 / kFixKappa);

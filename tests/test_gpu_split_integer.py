@@ -124,3 +124,32 @@ def test_limb_edges(gpp):
     am[4] = 1.0 - 2.0 ** -53
     am[5] = -1.0 + 2.0 ** -53
     check(gpp, prob.replace(wtilde_array=wt, wx_array=wx, aqsmtemp=am, aqsntemp=an))
+
+
+@pytest.mark.parametrize("sexcut", [1e-3, 0.3, 1.2, 4.0, 8.0, 15.0, 40.0])
+@pytest.mark.parametrize("occ", ["all", "occupied"])
+def test_negative_frequencies_with_cutoff(gpp, sexcut, occ):
+    """The screened-exchange cutoff on the split-integer form: frequencies of both signs, many
+    next to -Re w, poles from 0.15 up (the lowest need the reduced scale, the highest cutoffs
+    send warps to the FP64 form).
+
+    Tolerance: a kept term next to x = -w is taken at a scale up to 2^-6 below the others', so
+    with a relative error up to 2^-47, and such terms are few: 2^-45 of the outputs' root mean
+    square."""
+    import torch
+    rng = np.random.Generator(np.random.PCG64(int(1000 * sexcut) + len(occ)))
+    prob = inputs.make_problem(40, 17, 300, 12, 3, seed=29)
+    wx = rng.uniform(-9.0, 9.0, size=prob.wx_array.shape)
+    wx[::3] = -rng.uniform(0.1, 3.1, size=wx[::3].shape)
+    wx[1] = [0.0, -0.0, -1e-12]
+    wt = prob.wtilde_array.copy()
+    wt[3] = rng.uniform(0.15, 0.3, size=300) + 1j * rng.uniform(-0.01, 0.01, size=300)
+    prob = prob.replace(wx_array=wx, wtilde_array=wt)
+    dp = gpp.DeviceProblem.from_host(prob, device="cuda")
+    got = gpp.sigma(dp, sexcut=sexcut, ch_half=True, occ_mode=occ)
+    torch.cuda.synchronize()
+    ref = oracle.sigma(prob, sexcut=sexcut, ch_half=True, occ_mode=0 if occ == "all" else 1)
+    for g, r in zip(got, ref):
+        rms = np.sqrt(np.mean(np.abs(r) ** 2))
+        err = np.max(np.abs(g.cpu().numpy() - r))
+        assert err <= 2.0 ** -45 * rms, err / rms
