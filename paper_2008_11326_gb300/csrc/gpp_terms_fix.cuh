@@ -537,7 +537,7 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
                        warp * kStageBands};
   const FixPair w = fix_pair(wv, E);
   const double Iwr = fma(I.x, wv.x, -I.y * wv.y), Iwi = fma(I.x, wv.y, I.y * wv.x);
-  const float w2f = fmaf(w.w1, w.w1, w.i1 * w.i1);
+  const float wrf = w.w1 + w.w2, w2f = fmaf(wrf, wrf, w.i1 * w.i1);
   float dcut = 0.0f;   // the least |S| of a kept term with x < 0
   FixCut cut{w2f * w2f, 4.0f * w2f, static_cast<float>(sx2), sx2, {}};
   if (CUT) {

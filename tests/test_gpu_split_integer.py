@@ -153,3 +153,37 @@ def test_negative_frequencies_with_cutoff(gpp, sexcut, occ):
         rms = np.sqrt(np.mean(np.abs(r) ** 2))
         err = np.max(np.abs(g.cpu().numpy() - r))
         assert err <= 2.0 ** -45 * rms, err / rms
+
+
+@pytest.mark.parametrize("sexcut", [0.7, 4.0, 10.0])
+def test_cutoff_decisions_near_the_edge(gpp, sexcut):
+    """Terms on both sides of the cutoff, down to a relative distance of 2^-45, on both
+    branches and for poles from 0.15 to 9: every one is decided as the oracle decides it. Each
+    term is a problem of its own in the comparison (one column's G-vectors carry the distances;
+    a wrong decision changes the sum by a term, 1e-3 of it)."""
+    import torch
+    rng = np.random.Generator(np.random.PCG64(int(10 * sexcut)))
+    B = 12
+    prob = inputs.make_problem(B, 2, 256, B, 1, seed=31)
+    delta = 2.0 ** -rng.uniform(3, 45, 256) * rng.choice([-1.0, 1.0], 256)
+    w0 = np.geomspace(0.16, 6.0, B)
+    wx = np.empty((B, 1))
+    wt = prob.wtilde_array.copy()
+    for b in range(B):
+        if b % 2 == 0:   # branch 1, |x| > w: w^2 / (x^2 - w^2) = sexcut (1 + delta)
+            x = -w0[b] * np.sqrt(1 + 1 / sexcut)
+            t = sexcut * (1 + delta)
+            wt[b] = abs(x) * np.sqrt(t / (1 + t))
+        else:            # |x| < w: w^2 / (w^2 - x^2) where that can reach the cutoff
+            x = -w0[b] * np.sqrt(max(1 - 1 / sexcut, 0.1))
+            t = np.maximum(sexcut * (1 + delta), 1.05)
+            wt[b] = abs(x) * np.sqrt(t / (t - 1))
+        wx[b, 0] = x
+    prob = prob.replace(wx_array=wx, wtilde_array=wt)
+    for b in range(B):
+        sub = prob.columns(slice(b, b + 1))
+        dp = gpp.DeviceProblem.from_host(sub, device="cuda")
+        got = gpp.sigma(dp, sexcut=sexcut)[1]
+        torch.cuda.synchronize()
+        ref = oracle.sigma(sub, sexcut=sexcut)[1]
+        assert abs(got.cpu().numpy()[0] - ref[0]) <= 1e-9 * np.abs(sub.vcoul).max() * 256, b
