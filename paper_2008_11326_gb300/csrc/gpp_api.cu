@@ -271,6 +271,8 @@ int make_bwd_plan(const gpp_problem& p, const gpp_options& o, gpp::BwdPlan* plan
   size_t off = bp.fwd.total;
   bp.off_bwd_bt = off;
   off = gpp::align_up(off + static_cast<size_t>(p.number_bands) * p.nw * 128);
+  bp.off_bwd_fix = off;
+  off = gpp::align_up(off + 1024);
   bp.off_part_n = off;
   off = gpp::align_up(off + static_cast<size_t>(bg) * per_group);
   bp.off_part_r = off;
@@ -278,6 +280,8 @@ int make_bwd_plan(const gpp_problem& p, const gpp_options& o, gpp::BwdPlan* plan
                                 gpp::bwd_tile_cols() * 16);
   bp.off_rtot = off;
   off = gpp::align_up(off + static_cast<size_t>(p.number_bands) * p.ngpown * 16);
+  bp.off_links = off;
+  off = gpp::align_up(off + static_cast<size_t>(p.ngpown) * 2 * sizeof(int));
   bp.total = off;
   *plan = bp;
   return GPP_OK;

@@ -16,18 +16,29 @@
 // Terms are recomputed, not stored. One reciprocal r = 1/(|x-w|^2 |x+w|^2) per term gives
 // u = conj(x-w)|x+w|^2 r, v = conj(x+w)|x-w|^2 r and u v = conj(x^2-w^2) r.
 //
-// Decomposition: a CTA owns a tile of 8 columns (threadIdx.y) x 32 G-vectors (threadIdx.x),
+// Decomposition: a CTA owns a tile of 8 columns (one per warp) x 32 G-vectors (one per lane),
 // one (p, ig) pair per thread, and walks every band. wtilde / I_eps gradients stay in
-// registers. Per band, the CTA reduces am Q over its 8 columns and aqsntemp Q over its 32
-// G-vectors in shared memory with a fixed tree and writes one partial per tile; columns are
-// processed in batches of kBatchGroups column groups per launch, and a finishing kernel
-// adds each batch's partials into the outputs in a fixed order. No atomics: results are
-// deterministic.
+// registers. Every kRedBands bands, the CTA sums am Q over its 8 columns and aqsntemp Q over
+// its 32 G-vectors from shared memory in a fixed order and writes one partial per tile; columns
+// are processed in batches of column groups per launch, and a finishing kernel adds each
+// batch's partials into the outputs in a fixed order. No atomics: results are deterministic.
+//
+// Split-integer form. Warps in the range of the forward's split-integer form
+// (gpp_terms_fix.cuh) take u and v from there (U + gamma), with the cotangent products as
+// 31-bit integers and remainders. With x u = 1 + w u and x v = 1 - w v, on the fast path
+//   GI = sum_iw cap u + csh v,   GW = GI + w H,   H = sum_iw cap u^2 - csh v^2
+// (cap = c_a + c_s/2, csh = -c_s/2; the bands outside asxtemp: c_a and no v), so a term adds
+// u and u^2 (squared in 64 bits) to 62-bit sums GI and H, which are multiplied by M and summed
+// over the bands as in the forward:
+//   grad I_eps = conj(w sum_b M GI),   grad wtilde = conj(I (sum_b M GI + w sum_b M H)).
+// Q and its two weighted sums stay FP64 (20 FP64 instructions per unit, which run beside the
+// integer work; the FP64 form has 141).
 
 #include <cuda_runtime.h>
 
 #include "gpp_device.cuh"
 #include "gpp_internal.h"
+#include "gpp_terms_fix.cuh"
 
 namespace gpp {
 
@@ -65,12 +76,74 @@ struct BoolTag {
   static constexpr bool value = V;
 };
 
+// A cotangent product for the split-integer form: c = (r1 + r0, i1 + i0) 2^(ec - 31), with
+// the negatives and the FP32 value of the integer part.
+struct alignas(16) FixC {
+  int r1, i1, nr1, ni1;
+  float r0, i0, r1f, i1f;
+};
+// The cotangent products of every frequency; ok: finite and of ordinary exponent. The sums of
+// the moduli of all of cap and csh, and of all of ca, are below 2^ec (1 - 2^-21); sum_a, sum_s: of cap
+// (or ca) and of csh alone, over 2^ec.
+struct FixBwd {
+  int ok, ec;
+  float sum_a, sum_s;
+  FixC cap[kMaxNw], csh[kMaxNw], ca[kMaxNw];
+};
+static_assert(sizeof(FixBwd) <= 1024, "workspace segment of the cotangent products");
+
+__device__ inline FixC fix_c(double2 c, int ec) {
+  const double sr = c.x * exp2i(31 - ec), si = c.y * exp2i(31 - ec);
+  const double rr = rint(sr), ri = rint(si);
+  FixC o;
+  o.r1 = static_cast<int>(rr);
+  o.i1 = static_cast<int>(ri);
+  o.nr1 = -o.r1;
+  o.ni1 = -o.i1;
+  o.r0 = static_cast<float>(sr - rr);
+  o.i0 = static_cast<float>(si - ri);
+  o.r1f = static_cast<float>(rr);
+  o.i1f = static_cast<float>(ri);
+  return o;
+}
+
+// One warp, a lane per frequency: the split-integer form's cotangent products.
+__device__ inline void fix_cotangents(int W, const double2* g_ach, const double2* g_asx,
+                                      double ach_scale, FixBwd* out) {
+  const int iw = threadIdx.x;
+  const double2 zero = make_double2(0.0, 0.0);
+  const double2 ga = iw < W ? g_ach[iw] : zero, gs = iw < W ? g_asx[iw] : zero;
+  const double2 ca = make_double2(ach_scale * ga.x, -ach_scale * ga.y);
+  const double2 csh = make_double2(-0.5 * gs.x, 0.5 * gs.y);
+  const double2 cap = make_double2(ca.x - csh.x, ca.y - csh.y);
+  auto total = [](double2 c) { return warp_sum(sqrt(c.x * c.x + c.y * c.y)); };
+  const double sa = total(ca), sc = total(cap), ss = total(csh);
+  const double m = fmax(sc + ss, sa) * (1.0 + 0x1p-20);
+  const bool ok = m == 0.0 || (m > 1e-90 && m < 1e90);   // false for NaN
+  const int ec = m == 0.0 ? 0 : ((__double2hiint(m) >> 20) & 0x7ff) - 1022;
+  if (iw == 0) {
+    out->ok = ok;
+    out->ec = ec;
+    out->sum_a = ok ? static_cast<float>(fmax(sc, sa) * exp2i(-ec)) : 0.0f;
+    out->sum_s = ok ? static_cast<float>(ss * exp2i(-ec)) : 0.0f;
+  }
+  if (ok && iw < W) {
+    out->cap[iw] = fix_c(cap, ec);
+    out->csh[iw] = fix_c(csh, ec);
+    out->ca[iw] = fix_c(ca, ec);
+  }
+}
+
 // ach_scale: 1/2 with the half Coulomb-hole factor (it scales every achtemp cotangent).
 __global__ void gpp_bwd_prep_kernel(int64_t B, int W, const double* __restrict__ wx,
                                     const double2* __restrict__ g_ach,
                                     const double2* __restrict__ g_asx, double ach_scale,
-                                    BwdBand* bt) {
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+                                    BwdBand* bt, FixBwd* fixc) {
+  if (blockIdx.x == gridDim.x - 1) {   // a block of its own for the split-integer products
+    if (threadIdx.x < 32) fix_cotangents(W, g_ach, g_asx, ach_scale, fixc);
+    return;
+  }
+  const int64_t stride = static_cast<int64_t>(gridDim.x - 1) * blockDim.x;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < B * W;
        i += stride) {
     const int iw = static_cast<int>(i % W);
@@ -178,60 +251,188 @@ __device__ __forceinline__ void bwd_terms(const BwdBand* __restrict__ e, double 
   }
 }
 
-// Fixed shared-memory trees: sums s_a[ty][tx] over ty (into s_a[0][tx]) and s_r[ty][tx]
-// over tx (into s_r[ty][0]). The 256 threads are numbered L = 32 ty + tx and each level's
-// additions go to the lowest L, so every level but the last two of the row tree runs on
-// whole warps (a partly masked warp costs the FP64 pipe as much as a full one): 32 warp
-// additions per band instead of 94 with one row per warp. The two trees share the
-// barriers.
-__device__ __forceinline__ void tile_reduce(double2 (*s_a)[kTX], double2 (*s_r)[kTX]) {
-  const int L = threadIdx.y * kTX + threadIdx.x;
-#pragma unroll
-  for (int lev = 0; lev < 5; ++lev) {
-    const int hr = (kTX / 2) >> lev;           // row tree: 16, 8, 4, 2, 1
-    if (L < kTY * hr) {
-      const int row = L / hr, col = L - row * hr;
-      s_r[row][col].x += s_r[row][col + hr].x;
-      s_r[row][col].y += s_r[row][col + hr].y;
-    }
-    if (lev < 3) {
-      const int hc = (kTY / 2) >> lev;         // column tree: 4, 2, 1
-      if (L < kTX * hc) {
-        const int row = L / kTX, col = L - row * kTX;
-        s_a[row][col].x += s_a[row + hc][col].x;
-        s_a[row][col].y += s_a[row + hc][col].y;
-      }
-    }
-    __syncthreads();
+// u^2 of u = U + gamma, in units of 2^31 of U^2's: V + its remainder and FP32 value, laid out as
+// a FixU.
+__device__ __forceinline__ FixU fix_square(const FixU& u) {
+  const long long pr = mad_wide(u.Ur, u.Ur, mad_wide(-u.Ui, u.Ui, 0));
+  const long long pi = mad_wide(u.Ur, u.Ui, 0);   // half of it
+  FixU v;
+  v.Ur = static_cast<int>((pr + (1LL << 30)) >> 31);
+  v.Ui = static_cast<int>((pi + (1LL << 29)) >> 30);
+  const float k = 0x1p-30f;   // 2 U gamma
+  v.gr = fmaf(static_cast<float>(static_cast<int>(static_cast<unsigned>(pr) << 1)), 0x1p-32f,
+              k * fmaf(u.ur, u.gr, -u.ui * u.gi));
+  v.gi = fmaf(static_cast<float>(static_cast<int>(static_cast<unsigned>(pi) << 2)), 0x1p-32f,
+              k * fmaf(u.ur, u.gi, u.ui * u.gr));
+  v.ur = static_cast<float>(v.Ur);
+  v.ui = static_cast<float>(v.Ui);
+  return v;
+}
+
+// (s + l) += c u, or with CONJ c conj(u), or with NEG minus that.
+template <bool CONJ, bool NEG>
+__device__ __forceinline__ void fix_cmac(long long (&s)[2], float (&l)[2], const FixC& c,
+                                         const FixU& u) {
+  const int r = NEG ? c.nr1 : c.r1, i = NEG ? c.ni1 : c.i1;
+  const int nr = NEG ? c.r1 : c.nr1, ni = NEG ? c.i1 : c.ni1;
+  const float g = NEG ? -1.0f : 1.0f;
+  const float rf = g * c.r1f, jf = g * c.i1f, r0 = g * c.r0, j0 = g * c.i0;
+  if (CONJ) {   // re: r Ur + i Ui, im: i Ur - r Ui
+    s[0] = mad_wide(r, u.Ur, mad_wide(i, u.Ui, s[0]));
+    s[1] = mad_wide(i, u.Ur, mad_wide(nr, u.Ui, s[1]));
+    l[0] += fmaf(rf, u.gr, fmaf(jf, u.gi, fmaf(r0, u.ur, j0 * u.ui)));
+    l[1] += fmaf(jf, u.gr, fmaf(-rf, u.gi, fmaf(j0, u.ur, -r0 * u.ui)));
+  } else {      // re: r Ur - i Ui, im: r Ui + i Ur
+    s[0] = mad_wide(r, u.Ur, mad_wide(ni, u.Ui, s[0]));
+    s[1] = mad_wide(r, u.Ui, mad_wide(i, u.Ur, s[1]));
+    l[0] += fmaf(rf, u.gr, fmaf(-jf, u.gi, fmaf(r0, u.ur, -j0 * u.ui)));
+    l[1] += fmaf(rf, u.gi, fmaf(jf, u.gr, fmaf(r0, u.ui, j0 * u.ur)));
   }
 }
 
+// s / 2^d, rounded (d >= 0).
+__device__ __forceinline__ long long fix_down(long long s, int d) {
+  return (s + ((1LL << d) >> 1)) >> d;
+}
+
+// A 62-bit sum (with its small FP32 part, moved in in units of 2^4) as 2^sh (U + gamma).
+__device__ __forceinline__ FixU fix_limbs(const long long (&s)[2], int sh) {
+  const long long half = 1LL << (sh - 1);
+  FixU v;
+  v.Ur = static_cast<int>((s[0] + half) >> sh);
+  v.Ui = static_cast<int>((s[1] + half) >> sh);
+  v.gr = static_cast<float>(static_cast<int>(static_cast<unsigned>(s[0]) << (32 - sh))) * 0x1p-32f;
+  v.gi = static_cast<float>(static_cast<int>(static_cast<unsigned>(s[1]) << (32 - sh))) * 0x1p-32f;
+  v.ur = static_cast<float>(v.Ur);
+  v.ui = static_cast<float>(v.Ui);
+  return v;
+}
+
+// A complex sum over the bands of M u in the split form (see gpp_terms_fix.cuh): 64-bit sums
+// modulo 2^64, the FP32 sum that tells their multiple of 2^64, and the small parts.
+struct FixSum {
+  long long acc[2];
+  float aH[2], aL[2];
+  __device__ __forceinline__ void clear() {
+    acc[0] = acc[1] = 0;
+    aH[0] = aH[1] = aL[0] = aL[1] = 0.0f;
+  }
+  __device__ __forceinline__ void add(const FixM& m, const FixU& u) {
+    acc[0] = mad_wide(m.r1, u.Ur, mad_wide(m.ni1, u.Ui, acc[0]));
+    acc[1] = mad_wide(m.r1, u.Ui, mad_wide(m.i1, u.Ur, acc[1]));
+    aH[0] = fmaf(m.r1f, u.ur, fmaf(-m.i1f, u.ui, aH[0]));
+    aH[1] = fmaf(m.r1f, u.ui, fmaf(m.i1f, u.ur, aH[1]));
+    aL[0] += fmaf(m.r1f, u.gr, fmaf(-m.i1f, u.gi, fmaf(m.r0, u.ur, -m.i0 * u.ui)));
+    aL[1] += fmaf(m.r1f, u.gi, fmaf(m.i1f, u.gr, fmaf(m.r0, u.ui, m.i0 * u.ur)));
+  }
+  __device__ __forceinline__ void settle() {   // the small parts, after at most 8 bands
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int r = __float2int_rn(aL[k] * 0x1p-12f);
+      acc[k] = mad_wide(r, 4096, acc[k]);
+      aL[k] = fmaf(-4096.0f, static_cast<float>(r), aL[k]);
+    }
+  }
+  __device__ __forceinline__ double2 take() {   // the value so far; clears
+    double v[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      acc[k] += __float2int_rn(aL[k]);
+      const float top = static_cast<float>(static_cast<int>(acc[k] >> 32)) * 0x1p-32f;
+      const int j = __float2int_rn(fmaf(aH[k], 0x1p-64f, -top));
+      v[k] = fma(static_cast<double>(j), 18446744073709551616.0, static_cast<double>(acc[k]));
+    }
+    clear();
+    return make_double2(v[0], v[1]);
+  }
+};
+
+// The FP64 form's branch decision for one term, as the sign of |wdiff|^2 - 1/4. Not inlined: it
+// is taken about once in 1e6 terms, and inlined the compiler executes it for every term.
+__device__ __noinline__ float fix_exact_sign(const BandEntry* f, double2 w) {
+  const double a = __ldg(&f->lo.x) - w.x;
+  return gt_nonneg(fma(a, a, w.y * w.y), kLimitTwo) ? 1.0f : -1.0f;
+}
+
+// Bands between two reductions of a CTA (shared memory: 8 KB per band).
+constexpr int kRedBands = 4;
+constexpr int kTile = kTX * kTY;
+
+// The sums of the last nb bands (from b0): over the 8 columns of am Q (s_c, written to part_n),
+// over the 32 G-vectors of aqsntemp Q (s_r, written to part_r), each [component][band][column]
+// [G-vector] doubles. A column sum is one thread's; a row sum is four neighbouring lanes', 8
+// G-vectors each (started at different places: no bank conflicts), then two shuffles.
+__device__ __forceinline__ void tile_reduce(const double* s_c, const double* s_r, int nb, int B,
+                                            int b0, int64_t G, int64_t ig0, int gl, int64_t igt,
+                                            int ngroups, double* __restrict__ part_n,
+                                            double* __restrict__ part_r) {
+  const int L = threadIdx.x;
+  {
+    const int ig = L & 31, c = (L >> 5) & 1, bb = L >> 6;   // kRedBands = 4: 256 column sums
+    if (bb < nb && ig0 + ig < G) {
+      const double* v = s_c + (c * kRedBands + bb) * kTile + ig;
+      double sum = v[0];
+#pragma unroll
+      for (int y = 1; y < kTY; ++y) sum += v[y * kTX];
+      part_n[2 * ((static_cast<int64_t>(gl) * B + b0 + bb) * G + ig0 + ig) + c] = sum;
+    }
+  }
+  const int q = L & 3, y = (L >> 2) & 7, c = (L >> 5) & 1, bb = L >> 6;   // 64 row sums
+  double sum = 0.0;
+  const double* v = s_r + (c * kRedBands + bb) * kTile + y * kTX + q;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) sum += v[4 * ((i + y) & 7)];
+  sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+  sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+  if (q == 0 && bb < nb)
+    part_r[2 * ((igt * B + b0 + bb) * (static_cast<int64_t>(ngroups) * kTY) + gl * kTY + y) + c] = sum;
+}
+
+// Dynamic shared memory: the reductions' 2 x 2 x kRedBands x kTile doubles, then each warp's
+// staged weights.
+constexpr size_t kBwdSmem = static_cast<size_t>(4 * kRedBands) * kTile * sizeof(double) +
+                            kTY * kStageBands * sizeof(FixAm);
+
 template <int W>
-__global__ void __launch_bounds__(kTX * kTY, 2) gpp_bwd_kernel(
+__global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
     int B, int64_t G, int64_t P, int nocc, int64_t group0, int ngroups, int64_t n_ig_tiles,
     const double2* __restrict__ aqsn, const double2* __restrict__ eps,
     const double2* __restrict__ wt, const double2* __restrict__ am,
-    const BwdBand* __restrict__ bt, const int* __restrict__ colg, const int* __restrict__ flags,
+    const BwdBand* __restrict__ bt, const BandEntry* __restrict__ ft,
+    const FixBwd* __restrict__ fixc, const int* __restrict__ colg, const int* __restrict__ flags,
     double2* __restrict__ grad_w, double2* __restrict__ grad_I,
     double2* __restrict__ part_n,  // [ngroups][B][G]
     double2* __restrict__ part_r,  // [n_ig_tiles][B][ngroups * kTY]
     double sx2)                    // screened-exchange cutoff, sexcut^2 (0 = off)
 {
-  __shared__ double2 s_a[kTY][kTX];
-  __shared__ double2 s_r[kTY][kTX];
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  __shared__ FixC s_cap[W], s_csh[W], s_ca[W];
+  double* const s_c = reinterpret_cast<double*>(dyn_smem);
+  double* const s_r = s_c + 2 * kRedBands * kTile;
+  const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  FixAm* const stage = reinterpret_cast<FixAm*>(s_r + 2 * kRedBands * kTile) + ty * kStageBands;
   const bool x_nonneg = flags[0] == 0;
   const double wabs2_pf = pf_wabs2_min(flags);   // the partial fractions' bound (gpp_device.cuh)
+  const double xmax2 = wabs2_pf / kPfRatio2;
+  const FixInfo fix = *reinterpret_cast<const FixInfo*>(flags + kFlagFix);
+  const double* xrange = reinterpret_cast<const double*>(flags + kFlagRange);
+  const bool fix_on = fix.ok == 1 && fixc->ok;
+  for (int k = threadIdx.x; k < W; k += kTile) {
+    s_cap[k] = fixc->cap[k];
+    s_csh[k] = fixc->csh[k];
+    s_ca[k] = fixc->ca[k];
+  }
+  __syncthreads();
   const int64_t ntiles = static_cast<int64_t>(ngroups) * n_ig_tiles;
-  const int tx = threadIdx.x, ty = threadIdx.y;
   for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     // G-vector tile slowest, so the CTAs running together share one slab of aqsntemp
     const int64_t igt = t / ngroups;
     const int gl = static_cast<int>(t - igt * ngroups);       // group within the batch
     const int64_t p = (group0 + gl) * kTY + ty;
-    const int64_t ig = igt * kTX + tx;
+    const int64_t ig0 = igt * kTX, ig = ig0 + lane;
     const bool col_ok = p < P && colg[p] >= 0;
     const bool live = col_ok && ig < G;
-    double2 w = make_double2(0.5, 1.0);  // inert lane: finite terms, zero weight
+    double2 w = make_double2(1.0, 0.5);  // inert lane: finite terms, zero weight
     double2 I = make_double2(0.0, 0.0);
     if (live) {
       w = ldg2(wt + p * G + ig);
@@ -240,20 +441,151 @@ __global__ void __launch_bounds__(kTX * kTY, 2) gpp_bwd_kernel(
     const double wr = w.x, wi = w.y;
     const double wi2 = wi * wi;
     const double wabs2 = fma(wr, wr, wi2);
-    const double mw2r = -fma(wr, wr, -wi2);
-    const double w2i = 2.0 * wr * wi;
     const double2 Iw = cmul(I, w);
-    const bool fast_lane = wr >= 0.0 && gt_nonneg(wabs2, kFastWabs2Lo) &&
-                           lt_nonneg(wabs2, kFastWabs2Hi) && !lt_nonneg(wabs2, wabs2_pf);
-    const bool fast = __all_sync(0xffffffffu, fast_lane) && x_nonneg;
     const double2* an_ptr = aqsn + (ig < G ? ig : 0);
     const double2* am_ptr = am + (col_ok ? p : 0) * B;
+    auto load_an = [&](int b) {
+      return live ? ldg2(an_ptr + static_cast<int64_t>(b) * G) : make_double2(0.0, 0.0);
+    };
     double2 gw = make_double2(0.0, 0.0), gI = make_double2(0.0, 0.0);
-    // bands [0, nocc) enter asxtemp too; OCC is a template parameter of the band body
-    auto band = [&](int b, auto occ_tag) {
+    // one band's am Q and aqsntemp Q into the reduction's slot bb
+    auto put = [&](int bb, double2 amv, double2 an, double2 Q) {
+      const double2 c = cmul(amv, Q), r = cmul(an, Q);
+      s_c[bb * kTile + threadIdx.x] = c.x;
+      s_c[(kRedBands + bb) * kTile + threadIdx.x] = c.y;
+      s_r[bb * kTile + threadIdx.x] = r.x;
+      s_r[(kRedBands + bb) * kTile + threadIdx.x] = r.y;
+    };
+    auto reduce = [&](int b0, int nb) {
+      __syncthreads();
+      tile_reduce(s_c, s_r, nb, B, b0, G, ig0, gl, igt, ngroups, reinterpret_cast<double*>(part_n),
+                  reinterpret_cast<double*>(part_r));
+      __syncthreads();
+    };
+    auto load_am = [&](int b) { return col_ok ? ldg2(am_ptr + b) : make_double2(0.0, 0.0); };
+
+    // Split-integer form: the pair's scales, if the whole warp is in its range. GW = GI + w H
+    // cancels where x << |w|, so |w| may not exceed twice the largest frequency.
+    bool use_fix = fix_on && __all_sync(0xffffffffu, !live || (fix_lane(w, wabs2, fix) &&
+                                                               !gt_nonneg(wabs2, 4.0 * xmax2)));
+    int kn = 0, ka = 0, sh = 1;
+    if (use_fix) {
+      unsigned mn = 0, ma = 0, mp = 0;
+#pragma unroll 8
+      for (int b = 0; b < B; ++b) {
+        const unsigned hn = fix_hi_max(load_an(b)), ha = fix_hi_max(load_am(b));
+        mn = max(mn, hn);
+        ma = max(ma, ha);
+        mp = max(mp, hn + ha);
+      }
+      const bool ok = fix_weight_scale(mn, ma, mp, kn, ka, sh);
+      use_fix = __all_sync(0xffffffffu, ok);
+    }
+    const FixPair wf = fix_pair(w, fix.E);
+    float2 scA = make_float2(0.0f, 0.0f), scS = scA;   // the scales of u and of v
+    int ks = 0, down = 0, shG = 1, shH = 1;
+    double unitG = 1.0;   // GI in units of the FP64 form's (1) or of the integer sum's last bit
+    if (use_fix) {
+      float dA = 3.0e38f, dS2 = 3.0e38f;   // over the frequencies
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        const float lo = static_cast<float>(xrange[k]), hi = static_cast<float>(xrange[kMaxNw + k]);
+        dA = fminf(dA, fmaxf(0.5f, fmaxf(lo - wf.w1, wf.w1 - hi) * (1.0f - 0x1p-17f)));
+        const float sr = lo + wf.w1;
+        dS2 = fminf(dS2, fmaf(sr, sr, wf.i1 * wf.i1) * (1.0f - 0x1p-17f));
+      }
+      // u at its own scale, v at most as fine; the sums of the u terms are brought to v's scale
+      const int ksA = fix_ks(dA * dA);
+      ks = nocc > 0 ? min(ksA, fix_ks(dS2)) : ksA;
+      down = ksA - ks;
+      scA = fix_scale(ksA, fix.E);
+      scS = fix_scale(ks, fix.E);
+      // |GI| 2^(31 + ks - ec) and |H| 2^(2 ks - ec) stay below 2^(31 + shG), 2^(31 + shH)
+      const float cs = nocc > 0 ? fixc->sum_s : 0.0f;
+      const float bG = (fixc->sum_a / dA + cs * rsqrtf(dS2)) * 1.01f + 1e-30f;
+      const float bH = (fixc->sum_a / (dA * dA) + cs / dS2) * 1.01f + 1e-30f;
+      shG = min(max(ks + (__float_as_int(bG) >> 23) - 126, 1), 31);
+      shH = min(max(2 * ks - 31 + (__float_as_int(bH) >> 23) - 126, 1), 31);
+      unitG = exp2i(fixc->ec - 31 - ks) * (1.0 / kFixKappa);
+    }
+    double2 Iws = live ? make_double2(Iw.x * unitG, Iw.y * unitG) : make_double2(0.0, 0.0);
+    asm volatile("" : "+d"(Iws.x), "+d"(Iws.y));
+    int nkhi = (kn + 32) << 20, akhi = (ka + 32) << 20;
+    // (keeps the compiler from forming these again in every band)
+    asm volatile("" : "+f"(scA.x), "+f"(scA.y), "+f"(scS.x), "+f"(scS.y), "+r"(shG), "+r"(shH),
+                      "+r"(down), "+r"(nkhi), "+r"(akhi), "+r"(sh));
+    FixSum X, Y;
+    X.clear();
+    Y.clear();
+    double2 an_next = load_an(0);
+    // One band of a warp in the split-integer form; returns GI in units of unitG.
+    auto band_fix = [&](int b, double2 an, auto occ_tag) {
       constexpr bool OCC = decltype(occ_tag)::value;
-      const double2 an = (ig < G) ? ldg2(an_ptr + static_cast<int64_t>(b) * G) : make_double2(0.0, 0.0);
-      const double2 amv = col_ok ? ldg2(am_ptr + b) : make_double2(0.0, 0.0);
+      if ((b & (kStageBands - 1)) == 0) {   // this warp's weights of the next bands
+        __syncwarp();
+        for (int q = lane; q < kStageBands && b + q < B; q += 32) {
+          const double2 a = load_am(b + q);
+          FixAm e;
+          fix_value(a.x, akhi, e.r1, e.r0);
+          fix_value(a.y, akhi, e.i1, e.i0);
+          stage[q] = e;
+        }
+        __syncwarp();
+      }
+      const FixM m = fix_weight(stage[b & (kStageBands - 1)], an, nkhi, sh);
+      const BandEntry* f = ft + static_cast<int64_t>(b) * W;
+      long long g[2] = {0, 0}, h[2] = {0, 0};
+      float g0[2] = {0.0f, 0.0f}, h0[2] = {0.0f, 0.0f};
+      // the FP32 parts (below 2^31 kLow, 2^32 kLow) into the sums
+      constexpr int kLow = W <= 3 ? 4 : 8;
+      auto settle = [&]() {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          g[k] = mad_wide(__float2int_rn(g0[k] * (1.0f / kLow)), kLow, g[k]);
+          h[k] = mad_wide(__float2int_rn(h0[k] * (0.5f / kLow)), 2 * kLow, h[k]);
+          g0[k] = h0[k] = 0.0f;
+        }
+      };
+#pragma unroll(W <= 3 ? W : 1)
+      for (int k = 0; k < W; ++k) {
+        const int4 xv = __ldg(&f[k].fx);
+        const FixN na = fix_norm<true>(wf, __int_as_float(xv.z), __int_as_float(xv.w));
+        float d = (na.N1 - 0.25f) + na.Nm;
+        if (__any_sync(0xffffffffu, fabsf(d) <= kFixNear)) d = fix_exact_sign(f + k, w);
+        const FixC c = OCC ? s_cap[k] : s_ca[k];
+        const FixU u = fix_term<true, true>(wf, na, xv.x, xv.y, scA, d > 0.0f);
+        fix_cmac<false, false>(g, g0, c, u);
+        fix_cmac<false, false>(h, h0, c, fix_square(u));
+      }
+      settle();
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        g[k] = fix_down(g[k], down);
+        h[k] = fix_down(h[k], 2 * down);
+      }
+      if (OCC) {
+#pragma unroll(W <= 3 ? W : 1)
+        for (int k = 0; k < W; ++k) {   // v is the conjugate of what fix_term gives
+          const int4 xv = __ldg(&f[k].fx);
+          const FixC c = s_csh[k];
+          const FixN ns = fix_norm<false>(wf, __int_as_float(xv.z), __int_as_float(xv.w));
+          const FixU u = fix_term<false, false>(wf, ns, xv.x, xv.y, scS, true);
+          fix_cmac<true, false>(g, g0, c, u);
+          fix_cmac<true, true>(h, h0, c, fix_square(u));
+        }
+        settle();
+      }
+      X.add(m, fix_limbs(g, shG));
+      Y.add(m, fix_limbs(h, shH));
+      return make_double2(static_cast<double>(g[0]), static_cast<double>(g[1]));
+    };
+    // One band of a warp in FP64: its M GI and M GW into gI and gw; returns GI.
+    const double mw2r = -fma(wr, wr, -wi2), w2i = 2.0 * wr * wi;
+    const bool fast_lane = wr >= 0.0 && gt_nonneg(wabs2, kFastWabs2Lo) &&
+                           lt_nonneg(wabs2, kFastWabs2Hi) && !lt_nonneg(wabs2, wabs2_pf);
+    const bool fast = __all_sync(0xffffffffu, fast_lane || !live) && x_nonneg;
+    auto band_f64 = [&](int b, double2 an, double2 amv, auto occ_tag) {
+      constexpr bool OCC = decltype(occ_tag)::value;
       double2 GI = make_double2(0.0, 0.0), GW = make_double2(0.0, 0.0);
       const BwdBand* e = bt + static_cast<int64_t>(b) * W;
       if (fast)
@@ -264,19 +596,44 @@ __global__ void __launch_bounds__(kTX * kTY, 2) gpp_bwd_kernel(
       const double2 M = cmul(amv, an);
       cmac(gI, M, GI);
       cmac(gw, M, GW);
-      const double2 Q = live ? cmul(Iw, GI) : make_double2(0.0, 0.0);
-      s_a[ty][tx] = cmul(amv, Q);
-      s_r[ty][tx] = cmul(an, Q);
-      __syncthreads();
-      tile_reduce(s_a, s_r);
-      if (ty == 0 && ig < G)
-        part_n[(static_cast<int64_t>(gl) * B + b) * G + ig] = s_a[0][tx];
-      if (tx == 0)
-        part_r[(igt * B + b) * (static_cast<int64_t>(ngroups) * kTY) + gl * kTY + ty] = s_r[ty][0];
-      __syncthreads();
+      return GI;
     };
-    for (int b = 0; b < nocc; ++b) band(b, BoolTag<true>());
-    for (int b = nocc; b < B; ++b) band(b, BoolTag<false>());
+    auto run = [&](int b0, int b1, auto occ_tag) {
+      for (int c0 = b0; c0 < b1; c0 += kRedBands) {
+        const int nb = min(kRedBands, b1 - c0);
+#pragma unroll 1
+        for (int bb = 0; bb < nb; ++bb) {
+          const int b = c0 + bb;
+          const double2 an = an_next, amv = load_am(b);
+          if (b + 1 < B) an_next = load_an(b + 1);
+          const double2 GI = use_fix ? band_fix(b, an, occ_tag) : band_f64(b, an, amv, occ_tag);
+          put(bb, amv, an, cmul(Iws, GI));
+        }
+        if (use_fix) {
+          X.settle();
+          Y.settle();
+          if (((c0 - b0) & (kFlushBands - kRedBands)) == kFlushBands - kRedBands) {
+            const double2 x = X.take(), y = Y.take();
+            gI = make_double2(gI.x + x.x, gI.y + x.y);
+            gw = make_double2(gw.x + y.x, gw.y + y.y);
+          }
+        }
+        reduce(c0, nb);
+      }
+    };
+    run(0, nocc, BoolTag<true>());
+    run(nocc, B, BoolTag<false>());
+    if (use_fix) {
+      const double2 x = X.take(), y = Y.take();
+      // back to M GI and M H; H's unit: u^2 = V 2^(31 - 2 ks) / kappa^2
+      const int em = sh - ka - kn;
+      const double fx = unitG * exp2i(shG + em);
+      const double fy = exp2i(fixc->ec - 2 * ks + shH) * (1.0 / kFixKappa) * (1.0 / kFixKappa) *
+                        exp2i(em);
+      gI = make_double2(fx * (gI.x + x.x), fx * (gI.y + x.y));
+      gw = cmul(w, make_double2(fy * (gw.x + y.x), fy * (gw.y + y.y)));
+      gw = make_double2(gI.x + gw.x, gI.y + gw.y);   // M GW = M GI + w M H
+    }
     gI = cmul(w, gI);
     gw = cmul(I, gw);
     if (live) {
@@ -325,43 +682,52 @@ __global__ void gpp_bwd_finish_batch_kernel(int64_t B, int64_t G, int64_t P, int
   }
 }
 
-// grad_aqsm[b][g] = vcoul[g] * sum over columns p with g(p) = g, in increasing p; zero for
-// global columns no column reaches. One thread per (b, g).
-__global__ void gpp_bwd_aqsm_kernel(int64_t B, int64_t G, int64_t P, const int* __restrict__ colg,
-                                    const double* __restrict__ vcoul,
-                                    const double2* __restrict__ rtot, double2* __restrict__ grad_m) {
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < B * G;
-       i += stride)
-    grad_m[i] = make_double2(0.0, 0.0);
-  // second phase handled by gpp_bwd_aqsm_scatter_kernel (after this kernel completes)
+// The columns that share a global column, as lists in increasing p: next[p] is the next column
+// with p's global column (-1: none), first[p] whether p is the first of its list. A column per
+// warp.
+__global__ void gpp_bwd_links_kernel(int64_t P, const int* __restrict__ colg, int* __restrict__ next,
+                                     int* __restrict__ first) {
+  const int lane = threadIdx.x & 31;
+  const int64_t p = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  if (p >= P) return;
+  const int g = colg[p];
+  int nx = 0x7fffffff;
+  bool before = false;
+  for (int64_t q = lane; q < P; q += 32)
+    if (colg[q] == g) {
+      if (q < p) before = true;
+      if (q > p) nx = min(nx, static_cast<int>(q));
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) nx = min(nx, __shfl_xor_sync(0xffffffffu, nx, o));
+  before = __any_sync(0xffffffffu, before);
+  if (lane == 0) {
+    next[p] = nx == 0x7fffffff ? -1 : nx;
+    first[p] = !before && g >= 0;
+  }
 }
 
+// grad_aqsm[b][g] = vcoul[g] * sum over columns p with g(p) = g, in increasing p (zero elsewhere:
+// the array is cleared first). One thread per (b, p).
 __global__ void gpp_bwd_aqsm_scatter_kernel(int64_t B, int64_t P, int64_t G,
                                             const int* __restrict__ colg,
                                             const double* __restrict__ vcoul,
                                             const double2* __restrict__ rtot,
+                                            const int* __restrict__ next,
+                                            const int* __restrict__ first,
                                             double2* __restrict__ grad_m) {
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < B * P;
        i += stride) {
     const int64_t b = i / P, p = i - b * P;
+    if (!first[p]) continue;   // the first column with this g sums all of them, in order
     const int g = colg[p];
-    if (g < 0) continue;
-    bool first = true;
-    for (int64_t q = 0; q < p; ++q)
-      if (colg[q] == g) {
-        first = false;
-        break;
-      }
-    if (!first) continue;  // the first column with this g sums all of them, in order
     double2 s = make_double2(0.0, 0.0);
-    for (int64_t q = p; q < P; ++q)
-      if (colg[q] == g) {
-        const double2 v = rtot[b * P + q];
-        s.x += v.x;
-        s.y += v.y;
-      }
+    for (int q = static_cast<int>(p); q >= 0; q = next[q]) {
+      const double2 v = rtot[b * P + q];
+      s.x += v.x;
+      s.y += v.y;
+    }
     const double vc = vcoul[g];
     grad_m[b * G + g] = make_double2(vc * s.x, vc * s.y);
   }
@@ -386,6 +752,11 @@ const void* bwd_kernel_ptr(int nw) {
   }
 }
 
+cudaError_t bwd_allow_smem(const void* fn) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(kBwdSmem));
+}
+
 int grid_for(int64_t work) {
   int64_t b = (work + 255) / 256;
   if (b < 1) b = 1;
@@ -399,7 +770,9 @@ int bwd_blocks_per_sm(int nw) {
   const void* fn = bwd_kernel_ptr(nw);
   if (!fn) return 0;
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kTX * kTY, 0) != cudaSuccess) return 0;
+  if (bwd_allow_smem(fn) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kTile, kBwdSmem) != cudaSuccess)
+    return 0;
   return n;
 }
 
@@ -415,10 +788,10 @@ cudaError_t launch_bwd(const gpp_problem& p, int occ_mode, double ach_scale, dou
   int64_t nocc = B;
   if (occ_mode == GPP_OCC_OCCUPIED) nocc = p.nvband < B ? p.nvband : B;
   BwdBand* bt = reinterpret_cast<BwdBand*>(ws + plan.off_bwd_bt);
-  gpp_bwd_prep_kernel<<<grid_for(B * W), 256, 0, s>>>(B, W, p.wx_array,
-                                                      reinterpret_cast<const double2*>(g_ach),
-                                                      reinterpret_cast<const double2*>(g_asx),
-                                                      ach_scale, bt);
+  FixBwd* fixc = reinterpret_cast<FixBwd*>(ws + plan.off_bwd_fix);
+  gpp_bwd_prep_kernel<<<grid_for(B * W) + 1, 256, 0, s>>>(
+      B, W, p.wx_array, reinterpret_cast<const double2*>(g_ach),
+      reinterpret_cast<const double2*>(g_asx), ach_scale, bt, fixc);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const double2* am = reinterpret_cast<const double2*>(ws + plan.fwd.off_am);
@@ -429,17 +802,17 @@ cudaError_t launch_bwd(const gpp_problem& p, int occ_mode, double ach_scale, dou
   double2* rtot = reinterpret_cast<double2*>(ws + plan.off_rtot);
   const int64_t ngroups_total = bwd_groups(P);
   const int64_t n_ig_tiles = (G + kTX - 1) / kTX;
-  const dim3 block(kTX, kTY);
+  const BandEntry* ft = reinterpret_cast<const BandEntry*>(ws + plan.fwd.off_bt);
   for (int64_t g0 = 0; g0 < ngroups_total; g0 += plan.batch_groups) {
     const int ng = static_cast<int>(ngroups_total - g0 < plan.batch_groups ? ngroups_total - g0
                                                                             : plan.batch_groups);
     const int64_t ntiles = ng * n_ig_tiles;
     int grid = static_cast<int>(ntiles < plan.max_grid ? ntiles : plan.max_grid);
 #define GPP_BWD_LAUNCH(WV)                                                                        \
-  gpp_bwd_kernel<WV><<<grid, block, 0, s>>>(                                                      \
+  gpp_bwd_kernel<WV><<<grid, kTile, kBwdSmem, s>>>(                                                      \
       static_cast<int>(B), G, P, static_cast<int>(nocc), g0, ng, n_ig_tiles,                      \
       reinterpret_cast<const double2*>(p.aqsntemp), reinterpret_cast<const double2*>(p.I_eps_array), \
-      reinterpret_cast<const double2*>(p.wtilde_array), am, bt, colg, flags,                      \
+      reinterpret_cast<const double2*>(p.wtilde_array), am, bt, ft, fixc, colg, flags,            \
       reinterpret_cast<double2*>(out.wtilde_array), reinterpret_cast<double2*>(out.I_eps_array),  \
       part_n, part_r, sx2)
     switch (W) {
@@ -461,11 +834,13 @@ cudaError_t launch_bwd(const gpp_problem& p, int occ_mode, double ach_scale, dou
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (out.aqsmtemp) {
-    gpp_bwd_aqsm_kernel<<<grid_for(B * G), 256, 0, s>>>(B, G, P, colg, p.vcoul, rtot,
-                                                        reinterpret_cast<double2*>(out.aqsmtemp));
+    int* next = reinterpret_cast<int*>(ws + plan.off_links);
+    e = cudaMemsetAsync(out.aqsmtemp, 0, static_cast<size_t>(B) * G * 16, s);
+    if (e != cudaSuccess) return e;
+    gpp_bwd_links_kernel<<<static_cast<unsigned>((P + 7) / 8), 256, 0, s>>>(P, colg, next, next + P);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     gpp_bwd_aqsm_scatter_kernel<<<grid_for(B * P), 256, 0, s>>>(
-        B, P, G, colg, p.vcoul, rtot, reinterpret_cast<double2*>(out.aqsmtemp));
+        B, P, G, colg, p.vcoul, rtot, next, next + P, reinterpret_cast<double2*>(out.aqsmtemp));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;

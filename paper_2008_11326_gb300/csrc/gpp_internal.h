@@ -52,9 +52,11 @@ struct BwdPlan {
   int batch_groups = 1;    // column groups (8 columns each) per main-kernel launch
   int max_grid = 1;        // persistent grid of the main kernel
   size_t off_bwd_bt = 0;   // BwdBand[B][W]
+  size_t off_bwd_fix = 0;  // FixBwd (1024 bytes)
   size_t off_part_n = 0;   // c128[batch_groups][B][G]
   size_t off_part_r = 0;   // c128[ceil(G/32)][B][batch_groups * 8]
   size_t off_rtot = 0;     // c128[B][P]
+  size_t off_links = 0;    // int32[2][P]: columns of the same global column
   size_t total = 0;
 };
 

@@ -499,6 +499,19 @@ __device__ __forceinline__ bool fix_exponent(unsigned m, int& k) {
   return m == 0 || (k >= 0 && k <= 400);
 }
 
+// The weights' scales from the largest high words over the bands of the column of aqsntemp
+// (mn), of the row of weights (ma) and of their products' sums (mp): kn, ka, and the shift sh
+// that takes the largest |M| comp to 31 bits. False outside the range.
+__device__ __forceinline__ bool fix_weight_scale(unsigned mn, unsigned ma, unsigned mp, int& kn,
+                                                 int& ka, int& sh) {
+  const bool n_ok = fix_exponent(mn, kn), a_ok = fix_exponent(ma, ka);
+  // every |M| comp 2^(ka + kn) < 2^top: twice (complex) the largest product, 0.18 for its
+  // logarithm
+  const int top = static_cast<int>((mp + (1u << 20) + 188744u) >> 20) + 1 - 2046 + ka + kn;
+  sh = max(min(top - 31, 30), 1);
+  return n_ok && a_ok && (mn == 0 || ma == 0 || top >= kFixMinTop);
+}
+
 // All bands of the thread's pair by the split-integer form, multiplied by Iw = I w and added
 // to tacc[4 W]. Returns false (nothing added) if any lane of the warp is out of range. B >= 1.
 template <int W, bool CUT>
@@ -515,7 +528,7 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
   float2* sc = reinterpret_cast<float2*>(smem + static_cast<size_t>(nt) * 4 * WG * 8) + threadIdx.x;
   // the magnitudes of the column of aqsntemp, of the row of weights and of their products
   unsigned mn = 0, ma = 0, mp = 0;
-  int kn, ka;
+  int kn, ka, sh;
 #pragma unroll 8
   for (int b = 0; b < B; ++b) {
     const unsigned hn = fix_hi_max(ldg2(an_ptr + static_cast<int64_t>(b) * G));
@@ -524,14 +537,8 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
     ma = max(ma, ha);
     mp = max(mp, hn + ha);
   }
-  const bool n_ok = fix_exponent(mn, kn), a_ok = fix_exponent(ma, ka);
-  if (!live) kn = 0;   // whatever its column holds: the values stay finite and I is zero
-  // every |M| comp 2^(ka + kn) < 2^top: twice (complex) the largest product, 0.18 for its
-  // logarithm; sh takes the largest to 31 bits
-  const int top = static_cast<int>((mp + (1u << 20) + 188744u) >> 20) + 1 - 2046 + ka + kn;
-  const bool m_ok = n_ok && (mn == 0 || ma == 0 || top >= kFixMinTop);
-  if (!a_ok || !__all_sync(0xffffffffu, m_ok || !live)) return false;
-  const int sh = max(min(top - 31, 30), 1);
+  if (!live) mn = mp = 0;   // whatever its column holds: the values stay finite and I is zero
+  if (!__all_sync(0xffffffffu, fix_weight_scale(mn, ma, mp, kn, ka, sh))) return false;
   const FixCtx ctx{G, an_ptr, am_ptr, w_ptr, bt, W, (kn + 32) << 20, (ka + 32) << 20, sh,
                    reinterpret_cast<FixAm*>(smem + static_cast<size_t>(nt) * 6 * WG * 8) +
                        warp * kStageBands};
