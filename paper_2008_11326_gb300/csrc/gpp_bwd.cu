@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
         float d = (na.N1 - 0.25f) + na.Nm;
         if (__any_sync(0xffffffffu, fabsf(d) <= kFixNear)) d = fix_exact_sign(f + k, w);
         const FixC c = OCC ? s_cap[k] : s_ca[k];
-        const FixU u = fix_term<true, true>(wf, na, xv.x, xv.y, scA, d > 0.0f);
+        const FixU u = fix_term<true, true>(wf, na, fix_biased(xv), scA, d > 0.0f);
         fix_cmac<false, false>(g, g0, c, u);
         fix_cmac<false, false>(h, h0, c, fix_square(u));
       }
@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
           const int4 xv = __ldg(&f[k].fx);
           const FixC c = s_csh[k];
           const FixN ns = fix_norm<false>(wf, __int_as_float(xv.z), __int_as_float(xv.w));
-          const FixU u = fix_term<false, false>(wf, ns, xv.x, xv.y, scS, true);
+          const FixU u = fix_term<false, false>(wf, ns, fix_biased(xv), scS, true);
           fix_cmac<true, false>(g, g0, c, u);
           fix_cmac<true, true>(h, h0, c, fix_square(u));
         }

@@ -59,7 +59,8 @@ struct alignas(16) FixAm {
 
 // Per-thread constants of a (p, ig) pair.
 struct FixPair {
-  int wh, wl, ih, il;  // Re w, Im w = hi 2^-h + lo 2^-(h+32)
+  long long w64;       // Re w 2^(h+32)
+  int ih, il;          // Im w = ih 2^-h + il 2^-(h+32)
   float w1, w2;        // Re w = w1 (multiple of 2^(E-23)) + w2
   float i1, i2;        // Im w = i1 + i2
   float n1, n2;        // (Im w)^2 = n1 (multiple of 2^(2E-21)) + n2
@@ -131,22 +132,30 @@ __device__ __forceinline__ void fix_floats(int hi, int lo, int E, float& a, floa
   b = fmaf(static_cast<float>(lo), exp2if(E - 62), static_cast<float>(hi - (q << 7)) * exp2if(E - 30));
 }
 
-// One band-table entry's split frequency.
+// One band-table entry's split frequency: x 2^(h+32) + 2^31 as a 64-bit integer (of its sums and
+// differences with Re w the high word is then the rounded one, without a carry from the signed
+// low word), and the two floats.
 __device__ __forceinline__ int4 fix_x(double x, int E) {
   int hi, lo;
   float a, b;
   fix_value(x, (62 - E) << 20, hi, lo);
   if (x < 0.0 && hi == 0 && lo == 0) lo = -1;   // the sign tells the cutoff's terms
   fix_floats(hi, lo, E, a, b);
-  return make_int4(hi, lo, __float_as_int(a), __float_as_int(b));
+  const long long i = (static_cast<long long>(hi) << 32) + lo + 0x80000000LL;
+  return make_int4(static_cast<int>(i >> 32), static_cast<int>(i), __float_as_int(a), __float_as_int(b));
+}
+__device__ __forceinline__ long long fix_biased(const int4& xv) {
+  return (static_cast<long long>(xv.x) << 32) | static_cast<unsigned>(xv.y);
 }
 
 __device__ __forceinline__ FixPair fix_pair(double2 w, int E) {
   FixPair q;
-  fix_value(w.x, (62 - E) << 20, q.wh, q.wl);
+  int wh, wl;
+  fix_value(w.x, (62 - E) << 20, wh, wl);
+  q.w64 = (static_cast<long long>(wh) << 32) + wl;
   fix_value(w.y, (62 - E) << 20, q.ih, q.il);
   q.il = max(q.il, -0x7fffffff);   // its negative is taken (2^-32 of the unit is below rounding)
-  fix_floats(q.wh, q.wl, E, q.w1, q.w2);
+  fix_floats(wh, wl, E, q.w1, q.w2);
   // Im w = i1 + i2: the leading 24 bits of the high part, and the rest
   const float r = static_cast<float>(q.ih);
   q.i1 = r * exp2if(E - 30);
@@ -193,14 +202,12 @@ __device__ __forceinline__ FixN fix_norm(const FixPair& w, float xa, float xb) {
 // 1/(Ar - i wi) with Ar = x - Re w (SIDE_A) or x + Re w (then that is conj(v)), from its norm;
 // with MASK zero where `on` is false.
 template <bool SIDE_A, bool MASK>
-__device__ __forceinline__ FixU fix_term(const FixPair& w, const FixN& n, int xh, int xl, float2 sc,
+__device__ __forceinline__ FixU fix_term(const FixPair& w, const FixN& n, long long xb, float2 sc,
                                          bool on) {
   FixU o;
-  const long long x64 = (static_cast<long long>(xh) << 32) + xl;
-  const long long w64 = (static_cast<long long>(w.wh) << 32) + w.wl;
-  const long long a64 = SIDE_A ? x64 - w64 : x64 + w64;
-  const int Al = static_cast<int>(a64);
-  const int Ah = static_cast<int>(a64 >> 32) - (Al >> 31);   // signed low word
+  const long long a64 = SIDE_A ? xb - w.w64 : xb + w.w64;    // A 2^(h+32) + 2^31
+  const int Ah = static_cast<int>(a64 >> 32);
+  const int Al = static_cast<int>(static_cast<unsigned>(a64) - 0x80000000u);
   float rho = fix_rcp(fmaf(n.N1, 1.0f + 0x1p-12f, n.Nm));    // kappa / |A|^2
   if (MASK) rho = on ? rho : 0.0f;
   float eps = fmaf(-rho, n.N1, kFixKappa);                   // kappa - rho |A|^2
@@ -298,6 +305,21 @@ struct FixCut {
   int delta[kFixMaxGroup];
 };
 
+// v 2^k for a zero v or one that stays normal.
+__device__ __forceinline__ double fix_shift(double v, int k) {
+  const int hi = __double2hiint(v);
+  return __hiloint2double((hi & 0x7fffffff) == 0 ? hi : hi + (k << 20), __double2loint(v));
+}
+// D 2^e, rounded by one conversion: an FP64 instruction takes as long as 30 of these. (By FP64
+// arithmetic on halves of the sums a pair's FP64 instructions were 107, now 44: B = 37, P = 95,
+// G = 1901, nw = 2: 181 -> 168 us; B = 32, P = 64, G = 512, nw = 3: 69.8 -> 65.9 us.)
+static __device__ __noinline__ double fix_round(__int128 D, int e) {
+  const long long hi = static_cast<long long>(D >> 64), lo = static_cast<long long>(D);
+  // the bits beyond the conversion's 64 are dropped (|D| >= 2^63 then)
+  const int k = hi == (lo >> 63) ? 0 : 65 - __clzll(hi ^ (hi >> 63));
+  return fix_shift(static_cast<double>(static_cast<long long>(D >> k)), k + e);
+}
+
 // Bands [b0, b1) of the thread's pair, WG frequencies from iw0, into the thread's FP64 sums
 // st[k blockDim.x] (units of kappa 2^ks M with the ks of u; values 4 iw + {0, 1}: sum M u, and
 // with OCC + {2, 3}: sum M u - sum M v), added to them, or with `fresh` replacing them.
@@ -366,7 +388,7 @@ __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixC
 #pragma unroll
           for (int k = 0; k < WG; ++k) {
             {
-              const FixU u = fix_term<true, true>(w, na[k], xv[k].x, xv[k].y, sc[2 * k * nt], d[k] > 0.0f);
+              const FixU u = fix_term<true, true>(w, na[k], fix_biased(xv[k]), sc[2 * k * nt], d[k] > 0.0f);
               acc[4 * k] = mad_wide(m.r1, u.Ur, mad_wide(m.ni1, u.Ui, acc[4 * k]));
               acc[4 * k + 1] = mad_wide(m.r1, u.Ui, mad_wide(m.i1, u.Ur, acc[4 * k + 1]));
               aH[4 * k] = fmaf(m.r1f, u.ur, fmaf(-m.i1f, u.ui, aH[4 * k]));
@@ -378,7 +400,7 @@ __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixC
               const FixN ns = fix_norm<false>(w, __int_as_float(xv[k].z), __int_as_float(xv[k].w));
               const float2 ss = sc[(2 * k + 1) * nt];
               bool on = true;
-              if (CUT && (xv[k].x < 0 || (xv[k].x == 0 && xv[k].y < 0))) {   // x < 0: warp-uniform
+              if (CUT && fix_biased(xv[k]) < 0x80000000LL) {   // x < 0: warp-uniform
                 const float NS = ns.N1 + ns.Nm;
                 const bool b1 = d[k] > 0.0f;
                 const float lim = cut.sx2f * NS * (b1 ? na[k].N1 + na[k].Nm : cut.w24);
@@ -397,7 +419,7 @@ __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixC
                 const bool small = !drop && NS < __int_as_float((443 - 2 * e) << 23);
                 on = !drop && !small;
                 if (__any_sync(0xffffffffu, drop && b1)) {   // take sum M u back out of asxtemp
-                  const FixU u = fix_term<true, true>(w, na[k], xv[k].x, xv[k].y, ss, drop && b1);
+                  const FixU u = fix_term<true, true>(w, na[k], fix_biased(xv[k]), ss, drop && b1);
                   acc[4 * k + 2] = mad_wide(m.r1, u.Ur, mad_wide(m.ni1, u.Ui, acc[4 * k + 2]));
                   acc[4 * k + 3] = mad_wide(m.r1, u.Ui, mad_wide(m.i1, u.Ur, acc[4 * k + 3]));
                   aH[4 * k + 2] = fmaf(m.r1f, u.ur, fmaf(-m.i1f, u.ui, aH[4 * k + 2]));
@@ -408,7 +430,7 @@ __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixC
                 if (__any_sync(0xffffffffu, small)) {
                   const int dl = cut.delta[k];
                   const float up = exp2if(dl);
-                  const FixU u = fix_term<false, true>(w, ns, xv[k].x, xv[k].y,
+                  const FixU u = fix_term<false, true>(w, ns, fix_biased(xv[k]),
                                                        make_float2(ss.x * exp2if(-dl), ss.y * up), small);
                   const long long pr = mad_wide(m.r1, u.Ur, mad_wide(m.i1, u.Ui, 0));
                   const long long pi = mad_wide(m.i1, u.Ur, mad_wide(m.nr1, u.Ui, 0));
@@ -420,7 +442,7 @@ __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixC
                   aL[4 * k + 3] = fmaf(up, fmaf(m.i1f, u.gr, fmaf(-m.r1f, u.gi, fmaf(m.i0, u.ur, -m.r0 * u.ui))), aL[4 * k + 3]);
                 }
               }
-              const FixU u = fix_term<false, CUT>(w, ns, xv[k].x, xv[k].y, ss, on);
+              const FixU u = fix_term<false, CUT>(w, ns, fix_biased(xv[k]), ss, on);
               acc[4 * k + 2] = mad_wide(m.r1, u.Ur, mad_wide(m.i1, u.Ui, acc[4 * k + 2]));
               acc[4 * k + 3] = mad_wide(m.i1, u.Ur, mad_wide(m.nr1, u.Ui, acc[4 * k + 3]));
               aH[4 * k + 2] = fmaf(m.r1f, u.ur, fmaf(m.i1f, u.ui, aH[4 * k + 2]));
@@ -451,10 +473,8 @@ __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixC
       any |= j[k];
     }
     const bool carry = __any_sync(0xffffffffu, any != 0);
-    auto sum = [&](int k) {
-      const double v = static_cast<double>(acc[k]);
-      return carry ? fma(static_cast<double>(j[k]), 18446744073709551616.0, v) : v;
-    };
+    auto total = [&](int k) { return static_cast<__int128>(j[k]) * (static_cast<__int128>(1) << 64) + acc[k]; };
+    auto sum = [&](int k) { return carry ? fix_round(total(k), 0) : static_cast<double>(acc[k]); };
     auto put = [&](int k, double v) { st[k * nt] = (!fresh || f0 > b0) ? st[k * nt] + v : v; };
 #pragma unroll
     for (int k = 0; k < WG; ++k) {
@@ -463,22 +483,13 @@ __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixC
         put(4 * k + 1, sum(4 * k + 1));
         continue;
       }
-      const double r = -exp2i((__float_as_int(sc[2 * k * nt].x) - __float_as_int(sc[(2 * k + 1) * nt].x)) >> 23);
+      const int dl = (__float_as_int(sc[2 * k * nt].x) - __float_as_int(sc[(2 * k + 1) * nt].x)) >> 23;
 #pragma unroll
       for (int c = 4 * k; c < 4 * k + 2; ++c) {
-        double a, d;
-        if (carry) {
-          a = sum(c);
-          d = fma(r, sum(c + 2), a);
-        } else {   // by halves: the difference (which may cancel) is rounded once
-          constexpr double k32 = 4294967296.0;
-          const double ah = static_cast<int>(acc[c] >> 32), al = static_cast<unsigned>(acc[c]);
-          const double sh = static_cast<int>(acc[c + 2] >> 32), sl = static_cast<unsigned>(acc[c + 2]);
-          a = fma(ah, k32, al);
-          d = fma(fma(r, sh, ah), k32, fma(r, sl, al));
-        }
-        put(c, a);
-        put(c + 2, d);
+        put(c, sum(c));
+        // the difference (which may cancel) is exact and rounded once
+        const int q = max(-dl, 0);
+        put(c + 2, fix_round((total(c) << q) - (total(c + 2) << max(dl, 0)), -q));
       }
     }
   }
@@ -543,7 +554,9 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
                    reinterpret_cast<FixAm*>(smem + static_cast<size_t>(nt) * 6 * WG * 8) +
                        warp * kStageBands};
   const FixPair w = fix_pair(wv, E);
-  const double Iwr = fma(I.x, wv.x, -I.y * wv.y), Iwi = fma(I.x, wv.y, I.y * wv.x);
+  // I w / (2 kappa); the 2 is in the shifts below (so that nothing overflows that I w does not)
+  const double Ir = I.x * (0.5 / kFixKappa), Ii = I.y * (0.5 / kFixKappa);
+  const double Iwr = fma(Ir, wv.x, -Ii * wv.y), Iwi = fma(Ir, wv.y, Ii * wv.x);
   const float wrf = w.w1 + w.w2, w2f = fmaf(wrf, wrf, w.i1 * w.i1);
   float dcut = 0.0f;   // the least |S| of a kept term with x < 0
   FixCut cut{w2f * w2f, 4.0f * w2f, static_cast<float>(sx2), sx2, {}};
@@ -587,16 +600,15 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
       fix_range<N, true, CUT>(0, nocc, true, ctx, iw0, w, cut, st, sc);
 #pragma unroll
       for (int k = 0; k < N; ++k) {
-        const double fa = exp2i(ex - ks[2 * k] - 1) * (1.0 / kFixKappa);
-        ax[2 * k] = fa * st[(4 * k + 2) * nt];
-        ax[2 * k + 1] = fa * st[(4 * k + 3) * nt];
+        ax[2 * k] = fix_shift(st[(4 * k + 2) * nt], ex - ks[2 * k]);
+        ax[2 * k + 1] = fix_shift(st[(4 * k + 3) * nt], ex - ks[2 * k]);
       }
     }
     if (nocc < B) fix_range<N, false, false>(nocc, B, nocc == 0, ctx, iw0, w, cut, st, sc);
 #pragma unroll
-    for (int k = 0; k < N; ++k) {   // tacc += I w times the pair's sums
-      const double fa = exp2i(ex - ks[2 * k]) * (1.0 / kFixKappa);
-      const double ar = fa * st[4 * k * nt], ai = fa * st[(4 * k + 1) * nt];
+    for (int k = 0; k < N; ++k) {   // tacc += I w times the pair's sums (units: I w / (2 kappa))
+      const double ar = fix_shift(st[4 * k * nt], ex - ks[2 * k] + 1);
+      const double ai = fix_shift(st[(4 * k + 1) * nt], ex - ks[2 * k] + 1);
       double* o = tacc + 4 * (iw0 + k);
       o[0] = fma(Iwr, ar, fma(-Iwi, ai, o[0]));
       o[1] = fma(Iwr, ai, fma(Iwi, ar, o[1]));

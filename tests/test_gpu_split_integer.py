@@ -187,3 +187,27 @@ def test_cutoff_decisions_near_the_edge(gpp, sexcut):
         torch.cuda.synchronize()
         ref = oracle.sigma(sub, sexcut=sexcut)[1]
         assert abs(got.cpu().numpy()[0] - ref[0]) <= 1e-9 * np.abs(sub.vcoul).max() * 256, b
+
+
+# weights of nearly one phase, so that the sums of 300 bands pass 2^64 many times over, upwards
+# and downwards, with the scale of u above ("far": |x - w| >= 1/2, |x + w| > 2) and below that
+# of v ("low": |x + w| < 1/2); (x + |w|) / 2 |w| is at most 4, so the difference of the two sums
+# that asxtemp takes costs two of the tolerance's bits
+@pytest.mark.parametrize("where", ["far", "low"])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_sums_beyond_64_bits(gpp, where, sign):
+    rng = np.random.Generator(np.random.PCG64(77))
+    prob = inputs.make_problem(300, 120, 70, 3, 2, seed=78)
+    B, G = prob.aqsmtemp.shape
+    P = prob.wtilde_array.shape[0]
+
+    def near_one(shape):
+        return 1.0 + 0.01 * (rng.standard_normal(shape) + 1j * rng.standard_normal(shape))
+    far = where == "far"
+    w = rng.uniform(1.0, 3.0, (P, G)) if far else rng.uniform(0.2, 0.4, (P, G))
+    x = rng.uniform(0.0, 7.0, (B, 2)) if far else rng.uniform(0.0, 1.2, (B, 2))
+    prob = prob.replace(aqsmtemp=sign * (0.9 - 0.3j) * near_one((B, G)),
+                        aqsntemp=(0.6 + 0.5j) * near_one((B, G)), wx_array=x,
+                        wtilde_array=w + 1j * rng.uniform(-0.05, 0.05, (P, G)))
+    check(gpp, prob)
+    check(gpp, prob, occ="occupied")
