@@ -100,6 +100,8 @@ class GppError(RuntimeError):
 def lib():
     """The loaded libgpp (raises if it has not been built)."""
     global _lib
+    if _lib is not None:   # set once, complete
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib

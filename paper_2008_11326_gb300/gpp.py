@@ -99,7 +99,7 @@ class DeviceProblem:
         dev = self.aqsmtemp.device
         for name, dt, shape in spec:
             x = getattr(self, name)
-            if (x.dtype != dt or tuple(x.shape) != shape or x.device != dev
+            if (x.dtype != dt or x.shape != shape or x.device != dev
                     or not x.is_contiguous()):
                 raise ValueError(f"{name}: want a contiguous {dt} tensor of shape {shape} on "
                                  f"{dev}, got {x.dtype} {tuple(x.shape)} on {x.device}")
@@ -115,9 +115,10 @@ class DeviceProblem:
         self.check(ach, asx)
         return N.GppProblem(
             self.number_bands, self.nvband, self.ncouls, self.ngpown, self.nw,
-            ptr(self.aqsmtemp), ptr(self.aqsntemp), ptr(self.I_eps_array),
-            ptr(self.wtilde_array), ptr(self.vcoul), ptr(self.inv_igp_index), ptr(self.indinv),
-            ptr(self.wx_array), ptr(self.aqsntemp_c64), ptr(ach), ptr(asx))
+            self.aqsmtemp.data_ptr(), self.aqsntemp.data_ptr(), self.I_eps_array.data_ptr(),
+            self.wtilde_array.data_ptr(), self.vcoul.data_ptr(), self.inv_igp_index.data_ptr(),
+            self.indinv.data_ptr(), self.wx_array.data_ptr(), ptr(self.aqsntemp_c64), ptr(ach),
+            ptr(asx))
 
 
 def _stream_handle(stream, device):
@@ -310,7 +311,8 @@ def _problem_from(aqsmtemp, aqsntemp, I_eps_array, wtilde_array, vcoul, inv_igp_
     B, G = aqsmtemp.shape
     P = wtilde_array.shape[0]
     W = wx_array.shape[1]
-    c = lambda x, dt: x.detach().to(dt).contiguous()  # noqa: E731
+    def c(x, dt):   # the three calls only where they change something: 4 us of host time each
+        return x if x.dtype == dt and x.is_contiguous() else x.detach().to(dt).contiguous()
     return DeviceProblem(B, int(nvband), G, P, W, c(aqsmtemp, torch.complex128),
                          c(aqsntemp, torch.complex128), c(I_eps_array, torch.complex128),
                          c(wtilde_array, torch.complex128), c(vcoul, torch.float64),
