@@ -9,7 +9,7 @@
 // persistent grid take tiles from an atomic counter; the counter only schedules, and every
 // tile writes its own partial slot, so the result does not depend on which CTA ran which
 // tile. A per-instance kernel then sums the instance's tile partials in tile order. The
-// per-tile arithmetic is the single-instance kernels' (gpp_terms_f64.cuh / gpp_terms_f32.cuh).
+// per-pair arithmetic is in gpp_terms_fix.cuh, gpp_terms_f64.cuh and gpp_terms_f32.cuh.
 
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -319,8 +319,8 @@ __device__ __forceinline__ void f32_body(const BatchInst* __restrict__ inst, int
 // GPP_F32_MAXNREG registers (80 for nw > 5, whose band loop would spill at fewer).
 //
 // Measured (GB300, main sum with the split-integer form against the FP64 form alone):
-// B = 512, P = 819, G = 16384, nw = 3: 163.6 against 692.8 ms; B = 128, P = 410, G = 8192:
-// 10.5 against 44.4 ms; B = 32, P = 64, G = 512: 0.057 against 0.30 ms (with shallower tiles
+// B = 512, P = 819, G = 16384, nw = 3: 162.7 against 692.6 ms; B = 128, P = 410, G = 8192:
+// 10.5 against 44.4 ms; B = 32, P = 64, G = 512: 0.053 against 0.30 ms (with shallower tiles
 // and the cheaper reduction). Bound now: the instruction issue of the integer and FP32 pipes.
 template <int W>
 __global__ void __launch_bounds__(256, 2)

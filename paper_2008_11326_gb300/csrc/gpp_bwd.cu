@@ -31,8 +31,10 @@
 // u and u^2 (squared in 64 bits) to 62-bit sums GI and H, which are multiplied by M and summed
 // over the bands as in the forward:
 //   grad I_eps = conj(w sum_b M GI),   grad wtilde = conj(I (sum_b M GI + w sum_b M H)).
-// Q and its two weighted sums stay FP64 (20 FP64 instructions per unit, which run beside the
-// integer work; the FP64 form has 141).
+// Q and its two weighted sums stay FP64 (21 FP64 instructions per unit, which run beside the
+// integer work; the FP64 form has 141). Bound: dispatch of the integer and FP32 instructions
+// (ALU 315, FMA pipe 665 per unit and 32 lanes), with the FP64 pipe 56% busy and its latency on
+// top. B = 128, P = 410, G = 8192, nw = 3: 25.6 ms (FP64 form 108.3).
 
 #include <cuda_runtime.h>
 

@@ -1,14 +1,13 @@
 // Forward GPP sum: the column gather. The main sum runs in gpp_batched.cu (a single
-// instance is a batch of one) with the per-band arithmetic of gpp_terms_f64.cuh and
-// gpp_terms_f32.cuh.
+// instance is a batch of one) with the per-band arithmetic of gpp_terms_fix.cuh (FP64-accurate,
+// on the integer and FP32 pipes), gpp_terms_f64.cuh and gpp_terms_f32.cuh.
 //
 // Work decomposition (paper §III v4: the band loop runs serially inside a thread while
 // (igp, ig) are spread over threads, which keeps every ig-contiguous array coalesced).
 // A tile is one local column p and `threads * ig_per_thread` consecutive G-vectors; each
 // thread owns (p, ig) pairs of the tile, hoists everything that depends on (p, ig) only,
 // and walks all bands, evaluating every frequency iw from registers (the paper's v5 split
-// of iw into separate launches would recompute the shared terms, which the narrow FP64
-// pipe of GB300 cannot afford). Every tile writes its own partial and the partials are
+// of iw into separate launches would recompute the shared weights). Every tile writes its own partial and the partials are
 // summed in tile order, so every bit of the result is fixed.
 //
 // Arithmetic (paper §III v1: reciprocals instead of divides; §III v3: squared moduli).
