@@ -127,7 +127,8 @@ typedef struct gpp_options {
     int32_t blocks_per_sm; /* resident CTAs per SM for the persistent grid: 0 = as many as fit */
     int32_t debug_checks;  /* 1: validate indices on the device and synchronise (GPP_ERR_BAD_INDEX) */
     int32_t ig_per_thread; /* G-vectors each thread takes per tile: 0 = by the number of tiles (1, 2
-                              or 4 in GPP_FP64, 1 or 2 in GPP_FP32_BULK), max 8; a tile is
+                              or 4 in GPP_FP64; 1 or 2, with few bands up to 8, in GPP_FP32_BULK),
+                              max 8; a tile is
                               one igp column x block_threads * ig_per_thread G-vectors x all bands */
     int32_t physics;       /* bit set of gpp_physics: 0 = the paper's sum */
     int32_t reserved;      /* must be 0 */

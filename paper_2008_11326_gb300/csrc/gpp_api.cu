@@ -128,9 +128,19 @@ int check_pointers(const gpp_problem& p, int precision, bool outputs = true) {
 // us at 1 / 2 / 4: B=128 P=410 G=8192 (43 tiles per SM at 4) 10650 / 10590 / 10790; B=64 P=200
 // G=3000 (16 at 2) 1068 / 1063 / 1102; B=32 P=64 G=512 (0.8 at 2) 88 / 115 / 190.
 // FP32-bulk: 2 from 2 tiles per SM on, else 1: benchmark instance 93.6 / 92.6 / 94.2 ms at
-// 1 / 2 / 4; B=37 P=95 G=1901 (5 at 2) 85 / 77 / 92 us; B=32 P=64 G=512 (0.8 at 2) 55 / 64 / 83.
-int default_igpt(int precision, double columns, int sms) {
-  if (precision == GPP_FP32_BULK) return columns >= 2.0 * 2 * sms ? 2 : 1;
+// 1 / 2 / 4; B=32 P=95 G=1901 (5 at 2) 61 / 60 / 80 us; B=32 P=40 G=600 (0.7 at 2) 39 / 43 / 62.
+// With few bands (of the instance with the most; up to 40) and three or four frequencies the
+// tile's overhead in FP32-bulk weighs more: 4 from 32 tiles per SM on, 8 from 64. us at 2 / 4 / 8,
+// nw = 3: P=300 G=8000 (31 tiles per SM at 4) B=7 181 / 167 / 173, B=40 477 / 464 / 503; P=500
+// G=9000 (58 at 4) 344 / 312 / 300 and 948 / 908 / 891; P=550 G=20000 (71 at 8) 736 / 671 / 635 and
+// 1968 / 1885 / 1861; nw = 4, B=7: P=500 455 / 417 / 415. Beyond the lines: P=250 G=4000 (13 at 4)
+// B=28 171 / 171 / 168; B=64 nw=3 P=333 G=7777 747 / 754 / 761; B=64 nw=1 P=500 859 / 1034 / 1139.
+int default_igpt(int precision, double columns, int64_t bands, int64_t nw, int sms) {
+  if (precision == GPP_FP32_BULK) {
+    if (bands <= 40 && (nw == 3 || nw == 4) && columns >= 4.0 * 32 * sms)
+      return columns >= 8.0 * 64 * sms ? 8 : 4;
+    return columns >= 2.0 * 2 * sms ? 2 : 1;
+  }
   return columns >= 4.0 * 64 * sms ? 4 : columns >= 2.0 * 16 * sms ? 2 : 1;
 }
 double tile_columns(const gpp_problem& p, int threads) {
@@ -177,7 +187,8 @@ int make_plan(const gpp_problem& p, const gpp_options& o, gpp::FwdPlan* plan,
     int dev = 0, sms = 0;
     cudaError_t e = checked(cudaGetDevice(&dev));
     if (e == cudaSuccess) e = checked(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (!o.ig_per_thread) pl.igpt = default_igpt(o.precision, tile_columns(p, pl.threads), sms);
+    if (!o.ig_per_thread) pl.igpt = default_igpt(o.precision, tile_columns(p, pl.threads), p.number_bands,
+                                                  p.nw, sms);
     if (e == cudaSuccess) e = gpp::batched_prepare(pl.threads, pl.nw, f32, pl.igpt);
     if (e != cudaSuccess) return cuda_fail(e, "querying the device");
     int bps = o.blocks_per_sm ? o.blocks_per_sm
@@ -520,8 +531,12 @@ int batched_layout(const gpp_problem* probs, int n, const gpp_options* opt, bool
   cudaError_t e = checked(cudaGetDevice(&dev));
   if (e == cudaSuccess) e = checked(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   double columns = 0.0;
-  for (int i = 0; i < n; ++i) columns += tile_columns(probs[i], bp->threads);
-  bp->igpt = o.ig_per_thread ? o.ig_per_thread : default_igpt(o.precision, columns, sms);
+  int64_t bands = 0;
+  for (int i = 0; i < n; ++i) {
+    columns += tile_columns(probs[i], bp->threads);
+    bands = std::max<int64_t>(bands, probs[i].number_bands);
+  }
+  bp->igpt = o.ig_per_thread ? o.ig_per_thread : default_igpt(o.precision, columns, bands, bp->nw, sms);
   if (e == cudaSuccess) e = gpp::batched_prepare(bp->threads, bp->nw, bp->f32, bp->igpt);
   if (e != cudaSuccess) return cuda_fail(e, "querying the device");
   int bps = o.blocks_per_sm ? o.blocks_per_sm

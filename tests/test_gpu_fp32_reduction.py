@@ -35,3 +35,19 @@ def test_every_value_lands_in_its_place(gpp, nw, threads):
     torch.cuda.synchronize()
     for g, r in zip(got, oracle.sigma(prob)):
         assert np.max(np.abs(g.cpu().numpy() - r)) <= TOL * np.sqrt(np.mean(np.abs(r) ** 2))
+
+
+# at and past the lines of the default tile depth for few bands, on any count of SMs up to 160:
+# the default gives the bits of the depth it stands for
+@pytest.mark.parametrize("B,P,G,depth", [(3, 330, 8192, 4), (40, 330, 8065, 4), (41, 330, 8065, 2),
+                                         (3, 1300, 8192, 8), (5, 100, 1000, 2)])
+def test_default_depth(gpp, B, P, G, depth):
+    import torch
+    prob = inputs.make_problem(B, 2, G, P, 3, seed=B)
+    dp = gpp.DeviceProblem.from_host(prob, device="cuda", c64=True)
+    got = gpp.sigma(dp, precision="fp32_bulk")
+    want = gpp.sigma(dp, precision="fp32_bulk", ig_per_thread=depth)
+    torch.cuda.synchronize()
+    for g, w, r in zip(got, want, oracle.sigma(prob)):
+        assert torch.equal(g, w)
+        assert np.max(np.abs(g.cpu().numpy() - r)) <= TOL * np.sqrt(np.mean(np.abs(r) ** 2))
