@@ -40,7 +40,8 @@
 // the binary scale E of the instance's frequencies; weights whose row and column maxima over
 // the bands are finite and of ordinary exponent, and whose largest product over the bands is
 // within 2^-7 of the product of those maxima (the product of the split weights is exact to
-// 2^-60 of that). A warp with a lane outside takes the FP64 form.
+// 2^-60 of that), in the bands of asxtemp and in the others each by itself. A warp with a lane
+// outside takes the FP64 form.
 #pragma once
 
 #include "gpp_device.cuh"
@@ -283,7 +284,8 @@ __device__ __forceinline__ FixM fix_weight(const FixAm& a, double2 an, int nkhi,
   return m;
 }
 
-// What a pair's band loops share.
+// What a pair's band loops share, and the scales of the weights of one class of bands (the bands
+// of asxtemp, or the others; see FixScale), nkhi = (kn + 32) 2^20 and so on.
 struct FixCtx {
   int64_t G;
   const double2* an;   // the pair's column of aqsntemp (stride G)
@@ -526,8 +528,58 @@ __device__ __forceinline__ bool fix_weight_scale(unsigned mn, unsigned ma, unsig
   return n_ok && a_ok && (mn == 0 || ma == 0 || top >= kFixMinTop);
 }
 
+// The scales of one class of bands [b0, b1) for a pair, from the magnitudes of the column of
+// aqsntemp, of the row of weights and of their products: am 2^ka and an 2^kn as integers, their
+// product shifted by sh.
+struct FixScale {
+  int kn, ka, sh;
+  __device__ __forceinline__ int unit() const { return sh - ka - kn; }   // log2 of M1's unit
+};
+__device__ __forceinline__ bool fix_scales(int b0, int b1, int64_t G, const double2* an_ptr,
+                                           const double2* am_ptr, bool live, FixScale& s) {
+  unsigned mn = 0, ma = 0, mp = 0;
+#pragma unroll 8
+  for (int b = b0; b < b1; ++b) {
+    const unsigned hn = fix_hi_max(ldg2(an_ptr + static_cast<int64_t>(b) * G));
+    const unsigned ha = fix_hi_max(ldg2(am_ptr + b));
+    mn = max(mn, hn);
+    ma = max(ma, ha);
+    mp = max(mp, hn + ha);
+  }
+  if (!live) mn = mp = 0;   // whatever its column holds: the values stay finite and I is zero
+  return fix_weight_scale(mn, ma, mp, s.kn, s.ka, s.sh);
+}
+
+// The scales of one frequency's u and v, from the distance of its frequencies [lo, hi] from w and
+// -w, less the FP32 rounding. CUT: dcut is the least |S| of a kept term with x < 0; `delta` is
+// how far below the scale of most terms the kept ones near x = -w may lie.
+template <bool CUT>
+__device__ __forceinline__ void fix_distances(const FixPair& w, float w2f, float lo, float hi,
+                                              float dcut, int& ksu, int& ksv, int& delta) {
+  const float da = fmaxf(0.0f, fmaxf(lo - w.w1, w.w1 - hi));
+  const float dA2 = fmaxf(0.25f, fmaf(da, da, w.i1 * w.i1) * (1.0f - 0x1p-16f));
+  const float sr = fmaxf(lo + w.w1, -(hi + w.w1));
+  const float dr = CUT ? fmaxf(sr, 0.0f) : sr;
+  float dS2 = fmaf(dr, dr, w.i1 * w.i1) * (1.0f - 0x1p-17f);
+  if (CUT) {
+    const float least = fmaxf(dS2, dcut * dcut), most = fminf(w2f * (1.0f - 0x1p-17f), 0.0625f);
+    dS2 = fmaxf(least, most);
+    delta = fix_ks(dS2) - fix_ks(least);
+  }
+  ksu = fix_ks(dA2);
+  ksv = fix_ks(dS2);
+}
+// The least |S| of a kept term with x < 0 (see FixCut).
+__device__ __forceinline__ float fix_dcut(float w2f, float sx2f) {
+  const float sc = sqrtf(sx2f);
+  return sqrtf(w2f) * fminf(1.0f, fminf(sqrtf(1.0f + 1.0f / sc) - 1.0f, 0.5f / sc)) * (1.0f - 0x1p-17f);
+}
+
 // All bands of the thread's pair by the split-integer form, multiplied by Iw = I w and added
 // to tacc[4 W]. Returns false (nothing added) if any lane of the warp is out of range. B >= 1.
+//
+// Bands [0, nocc), which enter both sums, and the rest have weight scales of their own, so that
+// asxtemp is as accurate where its bands' weights are far below the others' (or above).
 template <int W, bool CUT>
 __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
                                            const double2* __restrict__ an_ptr,
@@ -540,35 +592,27 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
   const int nt = blockDim.x, warp = threadIdx.x >> 5;
   double* st = reinterpret_cast<double*>(smem) + threadIdx.x;
   float2* sc = reinterpret_cast<float2*>(smem + static_cast<size_t>(nt) * 4 * WG * 8) + threadIdx.x;
-  // the magnitudes of the column of aqsntemp, of the row of weights and of their products
-  unsigned mn = 0, ma = 0, mp = 0;
-  int kn, ka, sh;
-#pragma unroll 8
-  for (int b = 0; b < B; ++b) {
-    const unsigned hn = fix_hi_max(ldg2(an_ptr + static_cast<int64_t>(b) * G));
-    const unsigned ha = fix_hi_max(ldg2(am_ptr + b));
-    mn = max(mn, hn);
-    ma = max(ma, ha);
-    mp = max(mp, hn + ha);
-  }
-  if (!live) mn = mp = 0;   // whatever its column holds: the values stay finite and I is zero
-  if (!__all_sync(0xffffffffu, fix_weight_scale(mn, ma, mp, kn, ka, sh))) return false;
-  const FixCtx ctx{G, an_ptr, am_ptr, w_ptr, bt, W, (kn + 32) << 20, (ka + 32) << 20, sh,
-                   reinterpret_cast<FixAm*>(smem + static_cast<size_t>(nt) * 6 * WG * 8) +
-                       warp * kStageBands};
+  FixScale o, r;
+  const bool o_ok = fix_scales(0, nocc, G, an_ptr, am_ptr, live, o);
+  const bool r_ok = fix_scales(nocc, B, G, an_ptr, am_ptr, live, r);
+  if (!__all_sync(0xffffffffu, o_ok && r_ok)) return false;
+  FixAm* const stage = reinterpret_cast<FixAm*>(smem + static_cast<size_t>(nt) * 6 * WG * 8) +
+                       warp * kStageBands;
+  const FixCtx ctx{G, an_ptr, am_ptr, w_ptr, bt, W, (o.kn + 32) << 20, (o.ka + 32) << 20, o.sh, stage};
+  const FixCtx ctx_r{G, an_ptr, am_ptr, w_ptr, bt, W, (r.kn + 32) << 20, (r.ka + 32) << 20, r.sh, stage};
+  const int exo = o.unit(), exr = r.unit(), ex = nocc < B ? exr : exo;
   const FixPair w = fix_pair(wv, E);
   // I w / (2 kappa); the 2 is in the shifts below (so that nothing overflows that I w does not)
   const double Ir = I.x * (0.5 / kFixKappa), Ii = I.y * (0.5 / kFixKappa);
   const double Iwr = fma(Ir, wv.x, -Ii * wv.y), Iwi = fma(Ir, wv.y, Ii * wv.x);
   const float wrf = w.w1 + w.w2, w2f = fmaf(wrf, wrf, w.i1 * w.i1);
-  float dcut = 0.0f;   // the least |S| of a kept term with x < 0
+  float dcut = 0.0f;
   FixCut cut{w2f * w2f, 4.0f * w2f, static_cast<float>(sx2), sx2, {}};
   if (CUT) {
-    const float sc = sqrtf(cut.sx2f);
-    dcut = sqrtf(w2f) * fminf(1.0f, fminf(sqrtf(1.0f + 1.0f / sc) - 1.0f, 0.5f / sc)) * (1.0f - 0x1p-17f);
+    dcut = fix_dcut(w2f, cut.sx2f);
     // a cutoff so high that its least |S| needs a scale far from the others', or so low that
     // its tests leave FP32's range
-    const bool good = dcut >= 0x1p-6f * fminf(sqrtf(w2f), 0.25f) && sc > 0x1p-20f;
+    const bool good = dcut >= 0x1p-6f * fminf(sqrtf(w2f), 0.25f) && sqrtf(cut.sx2f) > 0x1p-20f;
     if (!__all_sync(0xffffffffu, good)) return false;
   }
   auto group = [&](auto tag, int iw0) {
@@ -576,47 +620,38 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
     int ks[2 * N];
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-      // the distance of the frequencies from w and -w, less its FP32 rounding
-      const float lo = static_cast<float>(xrange[iw0 + k]);
-      const float hi = static_cast<float>(xrange[kMaxNw + iw0 + k]);
-      const float dA = fmaxf(0.5f, fmaxf(lo - w.w1, w.w1 - hi) * (1.0f - 0x1p-17f));
-      const float sr = fmaxf(lo + w.w1, -(hi + w.w1));
-      const float dr = CUT ? fmaxf(sr, 0.0f) : sr;
-      float dS2 = fmaf(dr, dr, w.i1 * w.i1) * (1.0f - 0x1p-17f);
-      if (CUT) {
-        // the scale of most terms, and how far below it the kept terms near x = -w may lie
-        const float least = fmaxf(dS2, dcut * dcut), most = fminf(w2f * (1.0f - 0x1p-17f), 0.0625f);
-        dS2 = fmaxf(least, most);
-        cut.delta[k] = fix_ks(dS2) - fix_ks(least);
-      }
-      ks[2 * k] = fix_ks(dA * dA);
-      ks[2 * k + 1] = fix_ks(dS2);
+      fix_distances<CUT>(w, w2f, static_cast<float>(xrange[iw0 + k]),
+                         static_cast<float>(xrange[kMaxNw + iw0 + k]), dcut, ks[2 * k], ks[2 * k + 1],
+                         cut.delta[k]);
       sc[2 * k * nt] = fix_scale(ks[2 * k], E);
       sc[(2 * k + 1) * nt] = fix_scale(ks[2 * k + 1], E);
     }
     // units: M1 = M 2^(ka + kn - sh), U = u kappa 2^ks
-    const int ex = sh - ka - kn;
-    double ax[2 * N];   // asxtemp: (its bands' achtemp - sum M v) / 2
-#pragma unroll
-    for (int k = 0; k < 2 * N; ++k) ax[k] = 0.0;
     if (nocc > 0) {
       fix_range<N, true, CUT>(0, nocc, true, ctx, iw0, w, cut, st, sc);
+      if (nocc < B) {
 #pragma unroll
-      for (int k = 0; k < N; ++k) {
-        ax[2 * k] = fix_shift(st[(4 * k + 2) * nt], ex - ks[2 * k]);
-        ax[2 * k + 1] = fix_shift(st[(4 * k + 3) * nt], ex - ks[2 * k]);
+        for (int k = 0; k < N; ++k) {   // the others' units
+          st[4 * k * nt] = fix_shift(st[4 * k * nt], exo - exr);
+          st[(4 * k + 1) * nt] = fix_shift(st[(4 * k + 1) * nt], exo - exr);
+        }
       }
     }
-    if (nocc < B) fix_range<N, false, false>(nocc, B, nocc == 0, ctx, iw0, w, cut, st, sc);
+    if (nocc < B) fix_range<N, false, false>(nocc, B, nocc == 0, ctx_r, iw0, w, cut, st, sc);
 #pragma unroll
     for (int k = 0; k < N; ++k) {   // tacc += I w times the pair's sums (units: I w / (2 kappa))
       const double ar = fix_shift(st[4 * k * nt], ex - ks[2 * k] + 1);
       const double ai = fix_shift(st[(4 * k + 1) * nt], ex - ks[2 * k] + 1);
-      double* o = tacc + 4 * (iw0 + k);
-      o[0] = fma(Iwr, ar, fma(-Iwi, ai, o[0]));
-      o[1] = fma(Iwr, ai, fma(Iwi, ar, o[1]));
-      o[2] = fma(Iwr, ax[2 * k], fma(-Iwi, ax[2 * k + 1], o[2]));
-      o[3] = fma(Iwr, ax[2 * k + 1], fma(Iwi, ax[2 * k], o[3]));
+      double sr = 0.0, si = 0.0;   // asxtemp: (its bands' achtemp - sum M v) / 2
+      if (nocc > 0) {
+        sr = fix_shift(st[(4 * k + 2) * nt], exo - ks[2 * k]);
+        si = fix_shift(st[(4 * k + 3) * nt], exo - ks[2 * k]);
+      }
+      double* p = tacc + 4 * (iw0 + k);
+      p[0] = fma(Iwr, ar, fma(-Iwi, ai, p[0]));
+      p[1] = fma(Iwr, ai, fma(Iwi, ar, p[1]));
+      p[2] = fma(Iwr, sr, fma(-Iwi, si, p[2]));
+      p[3] = fma(Iwr, si, fma(Iwi, sr, p[3]));
     }
   };
   // frequency groups of at most three; the weights are formed again for each
