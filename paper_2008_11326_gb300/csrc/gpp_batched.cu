@@ -169,12 +169,29 @@ __device__ __forceinline__ void f64_body(const BatchInst* __restrict__ inst, int
       const double wabs2 = fma(w.x, w.x, w.y * w.y);
       if (fix_on && __all_sync(0xffffffffu, fix_lane(w, wabs2, fix) || !live)) {
         const double2* w64 = live ? d.wt + p * G + ig : d.wt;
-        const bool done =
-            fix.ok == 1 ? fix_band_loop<W, false>(B, G, nocc, an, am, d.bt, live, w, w64, I, fix.E,
-                                                  0.0, xrange, dyn_smem, acc)
-                        : fix_band_loop<W, true>(B, G, nocc, an, am, d.bt, live, w, w64, I, fix.E,
-                                                 d.sx2, xrange, dyn_smem, acc);
-        if (done) continue;
+        // with several groups of frequencies the sums before them, to be put back; else a doubted
+        // pair's own (local memory, as acc)
+        double other[4 * W];
+        if (W > kFixMaxGroup) {
+#pragma unroll
+          for (int k = 0; k < 4 * W; ++k) other[k] = acc[k];
+        }
+        const bool cut = fix.ok == 2;
+        const FixResult r =
+            cut ? fix_band_loop<W, true>(B, G, nocc, an, am, d.bt, live, w, w64, I, fix.E, d.sx2,
+                                         xrange, dyn_smem, acc, other)
+                : fix_band_loop<W, false>(B, G, nocc, an, am, d.bt, live, w, w64, I, fix.E, 0.0,
+                                          xrange, dyn_smem, acc, other);
+        if (r == kFixDone) continue;
+        if (r == kFixDoubt) {   // rare
+          const bool ok =
+              cut ? fix_strong<W, true>(B, G, nocc, an, am, d.bt, live, w, I, fix.E, d.sx2, xrange)
+                  : fix_strong<W, false>(B, G, nocc, an, am, d.bt, live, w, I, fix.E, 0.0, xrange);
+          const bool add = ok && W <= kFixMaxGroup, back = !ok && W > kFixMaxGroup;
+#pragma unroll
+          for (int k = 0; k < 4 * W; ++k) acc[k] = add ? acc[k] + other[k] : back ? other[k] : acc[k];
+          if (ok) continue;
+        }
       }
       // the FP64 fast form's conditions, with the partial fractions' bound on x / |w|
       const bool fast_lane = w.x >= 0.0 && gt_nonneg(wabs2, kFastWabs2Lo) &&

@@ -40,8 +40,9 @@
 // the binary scale E of the instance's frequencies; weights whose row and column maxima over
 // the bands are finite and of ordinary exponent, and whose largest product over the bands is
 // within 2^-7 of the product of those maxima (the product of the split weights is exact to
-// 2^-60 of that), in the bands of asxtemp and in the others each by itself. A warp with a lane
-// outside takes the FP64 form.
+// 2^-60 of that), in the bands of asxtemp and in the others each by itself; and every output's
+// terms not far below the scale of its sums (kFixWeak). A warp with a lane outside, or an output
+// that is too weak, takes the FP64 form.
 #pragma once
 
 #include "gpp_device.cuh"
@@ -530,9 +531,10 @@ __device__ __forceinline__ bool fix_weight_scale(unsigned mn, unsigned ma, unsig
 
 // The scales of one class of bands [b0, b1) for a pair, from the magnitudes of the column of
 // aqsntemp, of the row of weights and of their products: am 2^ka and an 2^kn as integers, their
-// product shifted by sh.
+// product shifted by sh. `any`: it has weights that are not zero (an inert lane has none).
 struct FixScale {
   int kn, ka, sh;
+  bool any;
   __device__ __forceinline__ int unit() const { return sh - ka - kn; }   // log2 of M1's unit
 };
 __device__ __forceinline__ bool fix_scales(int b0, int b1, int64_t G, const double2* an_ptr,
@@ -547,7 +549,37 @@ __device__ __forceinline__ bool fix_scales(int b0, int b1, int64_t G, const doub
     mp = max(mp, hn + ha);
   }
   if (!live) mn = mp = 0;   // whatever its column holds: the values stay finite and I is zero
+  s.any = mn != 0 && ma != 0;
   return fix_weight_scale(mn, ma, mp, s.kn, s.ka, s.sh);
+}
+
+// Whether an output is too weak for the scale that its sums were rounded at. A sum of n terms M u
+// carries an error of about sqrt(n) 2^-56 of its scale, which is 2^62 in the units of M1 U; so
+// relative to its own terms it is as good as the FP64 form's only while these are not far below
+// that. They are where other bands hold the large weights and add nothing to this output
+// (branch 2, the cutoff), or where one light band sets the scale of u. The line, 2^-kFixWeak of sqrt(n)
+// times the scale, bounds the error by about 2^-50 of the root of the sum of the terms' squares. It is
+// drawn for the largest lane of a warp, since the results are sums over all pairs: of 60000
+// pairs of 1..512 bands drawn as in the package's inputs, that lane's terms (root mean square) lie
+// at 2^-3.5 in the median and at 2^-5.3 at the least. (On the host, 64 bands, nw = 3: error 1.4e-16
+// of the terms there, FP64 form 2.4e-16.)
+// Two stages: the sums themselves, whose squares are the terms' powers but for what cancels, cost
+// a few instructions per pair (fix_band_loop's result); only a warp that this doubts has the
+// terms' powers formed (fix_strong).
+constexpr int kFixWeak = 6;
+constexpr int kFixNone = -0x20000000;   // the logarithm of zero: below all others, and so is a sum with it
+
+// log2 (sqrt(n)) in units of 2^-18.
+__device__ __forceinline__ int fix_half_log(float n) { return (__float_as_int(n) - (127 << 23)) >> 6; }
+// The least root that n terms M1 U may add up to in one class of bands, for U in units of 1 (plus
+// 1023); `any`: the pair has weights there that are not zero.
+__device__ __forceinline__ int fix_least(bool any, int n) {
+  return any && n > 0 ? fix_half_log(static_cast<float>(n)) + ((1023 + 62 - kFixWeak) << 18) : kFixNone;
+}
+// log2 of the larger component (plus 1023), in units of 2^-18.
+__device__ __forceinline__ int fix_log_max(double re, double im) {
+  const unsigned m = fix_hi_max(make_double2(re, im));
+  return m == 0 ? kFixNone : static_cast<int>(m >> 2);
 }
 
 // The scales of one frequency's u and v, from the distance of its frequencies [lo, hi] from w and
@@ -575,19 +607,124 @@ __device__ __forceinline__ float fix_dcut(float w2f, float sx2f) {
   return sqrtf(w2f) * fminf(1.0f, fminf(sqrtf(1.0f + 1.0f / sc) - 1.0f, 0.5f / sc)) * (1.0f - 0x1p-17f);
 }
 
+// Whether every output of the warp is strong enough, by the powers of its terms: the sums over
+// the bands of |M u|^2 on branch 1 and of |M v|^2 (with the cutoff: of the kept terms' 4 |M w u v|^2
+// or |M v|^2), in FP32, counting only terms that are clearly on their side of a threshold; a weight
+// below FP32's range still counts a little, so that only an output without terms is zero.
+template <int W, bool CUT>
+__device__ __noinline__ bool fix_strong(int B, int64_t G, int nocc, const double2* __restrict__ an_ptr,
+                                        const double2* __restrict__ am_ptr,
+                                        const BandEntry* __restrict__ bt, bool live, double2 wv,
+                                        double2 I, int E, double sx2,
+                                        const double* __restrict__ xrange) {
+  const FixPair w = fix_pair(wv, E);
+  const float wr = static_cast<float>(wv.x), wi = static_cast<float>(wv.y), wi2 = wi * wi;
+  const float w2 = fmaf(wr, wr, wi2), sx2f = static_cast<float>(sx2);
+  const int lgI = live ? fix_log_max(fma(I.x, wv.x, -I.y * wv.y), fma(I.x, wv.y, I.y * wv.x)) : kFixNone;
+  float pu[2][W], pv[W];
+  int unit[2], least[2];
+#pragma unroll
+  for (int k = 0; k < W; ++k) pu[0][k] = pu[1][k] = pv[k] = 0.0f;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {   // the bands of asxtemp, the others
+    const int b0 = c == 0 ? 0 : nocc, b1 = c == 0 ? nocc : B;
+    FixScale s;
+    fix_scales(b0, b1, G, an_ptr, am_ptr, live, s);
+    unit[c] = s.unit();
+    least[c] = fix_least(s.any, b1 - b0);
+    const double sn = exp2i(s.kn - 30), sa = exp2i(s.ka - 30);
+    const float m1 = exp2if(60 - s.sh);   // of (am 2^(ka - 30)) (an 2^(kn - 30)) in M1's units
+#pragma unroll 2
+    for (int b = b0; b < b1; ++b) {
+      const double2 an = ldg2(an_ptr + static_cast<int64_t>(b) * G), am = ldg2(am_ptr + b);
+      const float nr = static_cast<float>(an.x * sn), ni = static_cast<float>(an.y * sn);
+      const float ar = static_cast<float>(am.x * sa), ai = static_cast<float>(am.y * sa);
+      const float m2 = fmaxf(fmaf(nr, nr, ni * ni) * fmaf(ar, ar, ai * ai), 1e-37f) * m1 * m1;
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        const float x = static_cast<float>(__ldg(&bt[static_cast<int64_t>(b) * W + k].lo.x));
+        const float a = x - wr, a2 = fmaf(a, a, wi2), t = x + wr, s2 = fmaf(t, t, wi2);
+        const bool b1 = a2 > 0.25f * (1.0f + 0x1p-12f), b2 = a2 < 0.25f * (1.0f - 0x1p-12f);
+        const float ra = fix_rcp(a2), rs = fix_rcp(s2);
+        if (b1) pu[c][k] = fmaf(m2, ra, pu[c][k]);
+        if (c == 0) {
+          const float h = CUT && b1 ? w2 * ra * rs : 0.25f * rs;   // with the cutoff |ssx / (I w)|^2
+          if (!CUT || ((b1 || b2) && (x >= 0.0f || h * w2 < sx2f * (1.0f - 0x1p-10f))))
+            pv[k] += m2 * (4.0f * h);
+        }
+      }
+    }
+  }
+  const float dcut = CUT ? fix_dcut(w2, sx2f) : 0.0f;
+  bool strong = true;
+#pragma unroll
+  for (int k = 0; k < W; ++k) {
+    int ku, kv, delta;
+    fix_distances<CUT>(w, w2, static_cast<float>(xrange[k]), static_cast<float>(xrange[kMaxNw + k]),
+                       dcut, ku, kv, delta);
+    // of class c, times |I w|: a power as the logarithm of its root, and a scale's least root
+    auto root = [&](float e, int c) {
+      return e > 0.0f && least[c] != kFixNone ? lgI + (1023 << 18) + fix_half_log(e) + (unit[c] << 18)
+                                              : kFixNone;
+    };
+    auto floor_of = [&](float e, int c, int ks) {
+      return e > 0.0f && least[c] != kFixNone ? lgI + least[c] + ((unit[c] - ks) << 18) : kFixNone;
+    };
+    const int lu = floor_of(pu[0][k], 0, ku);
+    const int sa = max(root(pu[0][k], 0), root(pu[1][k], 1)), la = max(lu, floor_of(pu[1][k], 1, ku));
+    const int ss = root((CUT ? 0.0f : pu[0][k]) + pv[k], 0), ls = max(lu, floor_of(pv[k], 0, kv));
+    strong = strong && __reduce_max_sync(0xffffffffu, sa) >= __reduce_max_sync(0xffffffffu, la) &&
+             __reduce_max_sync(0xffffffffu, ss) >= __reduce_max_sync(0xffffffffu, ls);
+  }
+  return strong;
+}
+
+// Whether an output of N frequencies may be too weak for its scale, by the sums alone: those of a
+// pair, as fix_range left them in st, against half the least root of each class of its terms (a warp
+// with a single pair, past the last whole 32 G-vectors, would be doubted half of the time at all of
+// it). Passed by a lane whose scale, times |I w|, is within 2^1.5 of the largest in the warp: no single
+// lane decides, whose sum may be small by chance. (A pair without weights in a class may be doubted
+// for nothing.)
+template <int N>
+__device__ __noinline__ bool fix_doubt(const double* st, const float2* sc, int nt, int nocc, int B,
+                                       int exo, int exr, double Iwr, double Iwi) {
+  const int lgI = static_cast<int>(fix_hi_max(make_double2(Iwr, Iwi)) >> 2), one = 1 << 18;
+  const int no = fix_least(true, nocc) + exo * one, nr = fix_least(true, B - nocc) + exr * one;
+  bool doubt = false;
+  auto test = [&](double re, double im, int unit, int least) {
+    const int m = fix_log_max(re, im);
+    const int strong = m != kFixNone && m + unit * one >= least - one ? lgI + least : kFixNone;
+    doubt |= __reduce_max_sync(0xffffffffu, strong) <
+             __reduce_max_sync(0xffffffffu, lgI + least) - 3 * one / 2;
+  };
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    auto ks = [&](int q) { return (__float_as_int(sc[q * nt].x) >> 23) - 127; };
+    const int ku = ks(2 * k), kv = ks(2 * k + 1);
+    test(st[4 * k * nt], st[(4 * k + 1) * nt], (nocc < B ? exr : exo) - ku, max(no, nr) - ku * one);
+    if (nocc > 0)
+      test(st[(4 * k + 2) * nt], st[(4 * k + 3) * nt], exo - ku, no - min(ku, kv) * one);
+  }
+  return doubt;
+}
+
 // All bands of the thread's pair by the split-integer form, multiplied by Iw = I w and added
-// to tacc[4 W]. Returns false (nothing added) if any lane of the warp is out of range. B >= 1.
+// to tacc[4 W]. kFixOut (nothing added): a lane of the warp is out of range. kFixDoubt: an output
+// of the warp may be too weak for its scale; the sums are then in `apart` (W <= kFixMaxGroup) or
+// added to tacc all the same. B >= 1.
 //
 // Bands [0, nocc), which enter both sums, and the rest have weight scales of their own, so that
 // asxtemp is as accurate where its bands' weights are far below the others' (or above).
+enum FixResult { kFixOut, kFixDoubt, kFixDone };
 template <int W, bool CUT>
-__device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
-                                           const double2* __restrict__ an_ptr,
-                                           const double2* __restrict__ am_ptr,
-                                           const BandEntry* __restrict__ bt, bool live, double2 wv,
-                                           const double2* __restrict__ w_ptr, double2 I, int E, double sx2,
-                                           const double* __restrict__ xrange, unsigned char* smem,
-                                           double* tacc) {
+__device__ __noinline__ FixResult fix_band_loop(int B, int64_t G, int nocc,
+                                                const double2* __restrict__ an_ptr,
+                                                const double2* __restrict__ am_ptr,
+                                                const BandEntry* __restrict__ bt, bool live,
+                                                double2 wv, const double2* __restrict__ w_ptr,
+                                                double2 I, int E, double sx2,
+                                                const double* __restrict__ xrange,
+                                                unsigned char* smem, double* tacc, double* apart) {
   constexpr int WG = W < kFixMaxGroup ? W : kFixMaxGroup;
   const int nt = blockDim.x, warp = threadIdx.x >> 5;
   double* st = reinterpret_cast<double*>(smem) + threadIdx.x;
@@ -595,7 +732,7 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
   FixScale o, r;
   const bool o_ok = fix_scales(0, nocc, G, an_ptr, am_ptr, live, o);
   const bool r_ok = fix_scales(nocc, B, G, an_ptr, am_ptr, live, r);
-  if (!__all_sync(0xffffffffu, o_ok && r_ok)) return false;
+  if (!__all_sync(0xffffffffu, o_ok && r_ok)) return kFixOut;
   FixAm* const stage = reinterpret_cast<FixAm*>(smem + static_cast<size_t>(nt) * 6 * WG * 8) +
                        warp * kStageBands;
   const FixCtx ctx{G, an_ptr, am_ptr, w_ptr, bt, W, (o.kn + 32) << 20, (o.ka + 32) << 20, o.sh, stage};
@@ -613,8 +750,9 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
     // a cutoff so high that its least |S| needs a scale far from the others', or so low that
     // its tests leave FP32's range
     const bool good = dcut >= 0x1p-6f * fminf(sqrtf(w2f), 0.25f) && sqrtf(cut.sx2f) > 0x1p-20f;
-    if (!__all_sync(0xffffffffu, good)) return false;
+    if (!__all_sync(0xffffffffu, good)) return kFixOut;
   }
+  bool doubt = false;
   auto group = [&](auto tag, int iw0) {
     constexpr int N = decltype(tag)::value;
     int ks[2 * N];
@@ -638,6 +776,8 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
       }
     }
     if (nocc < B) fix_range<N, false, false>(nocc, B, nocc == 0, ctx_r, iw0, w, cut, st, sc);
+    doubt |= fix_doubt<N>(st, sc, nt, nocc, B, exo, exr, Iwr, Iwi);
+    const bool aside = W <= kFixMaxGroup && doubt;
 #pragma unroll
     for (int k = 0; k < N; ++k) {   // tacc += I w times the pair's sums (units: I w / (2 kappa))
       const double ar = fix_shift(st[4 * k * nt], ex - ks[2 * k] + 1);
@@ -648,10 +788,14 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
         si = fix_shift(st[(4 * k + 3) * nt], exo - ks[2 * k]);
       }
       double* p = tacc + 4 * (iw0 + k);
-      p[0] = fma(Iwr, ar, fma(-Iwi, ai, p[0]));
-      p[1] = fma(Iwr, ai, fma(Iwi, ar, p[1]));
-      p[2] = fma(Iwr, sr, fma(-Iwi, si, p[2]));
-      p[3] = fma(Iwr, si, fma(Iwi, sr, p[3]));
+      double v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = aside ? 0.0 : p[i];
+      if (aside) p = apart + 4 * (iw0 + k);
+      p[0] = fma(Iwr, ar, fma(-Iwi, ai, v[0]));
+      p[1] = fma(Iwr, ai, fma(Iwi, ar, v[1]));
+      p[2] = fma(Iwr, sr, fma(-Iwi, si, v[2]));
+      p[3] = fma(Iwr, si, fma(Iwi, sr, v[3]));
     }
   };
   // frequency groups of at most three; the weights are formed again for each
@@ -665,7 +809,7 @@ __device__ __noinline__ bool fix_band_loop(int B, int64_t G, int nocc,
     else
       group(IntTag<LO>(), iw0);
   }
-  return true;
+  return doubt ? kFixDoubt : kFixDone;
 }
 
 }  // namespace gpp

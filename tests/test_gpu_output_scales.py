@@ -1,9 +1,10 @@
 """Accuracy of every output relative to its own terms, where other bands hold far larger
-weights: the occupied bands against the rest.
+weights: the occupied bands against the rest, a heavy band that branch 2 or the cutoff
+removes, a light band that alone sets the scale of the reciprocals.
 
-Tolerance, derived before the first run: at a scale of its own an output carries about 2^-52 of the
-root of the sum of its terms' squares; partial fractions, FP64 sums and the oracle add a few
-2^-52 each: 2^-48 of that root.
+Tolerance, derived before the first run: an output whose terms are 2^-6 of its scale carries at
+most 2^-50 of the root of the sum of its terms' squares, weaker ones are FP64's, and partial
+fractions, FP64 sums and the oracle add a few 2^-52 each: 2^-48 of that root.
 """
 
 import numpy as np
@@ -69,3 +70,66 @@ def test_occupied_weights_of_another_size(gpp, scale, nw):
         a = getattr(prob, side).copy()
         a[:8] *= scale
         check(gpp, prob.replace(**{side: a}), occ="occupied")
+
+
+@pytest.mark.parametrize("heavy", [1e1, 1e2, 1e4, 1e6, 1e12])
+def test_heavy_band_in_branch_2(gpp, heavy):
+    """Band 5 lies within 1/2 of every pole at the first of four frequencies only."""
+    rng = np.random.Generator(np.random.PCG64(43))
+    prob = inputs.make_problem(24, 24, 96, 4, 4, seed=43)
+    w = rng.uniform(1.5, 1.7, (4, 96)) + 1j * rng.uniform(-0.05, 0.05, (4, 96))
+    wx = prob.wx_array.copy()
+    wx[:, 0] = np.where(np.abs(wx[:, 0] - 1.6) < 0.7, 2.5, wx[:, 0])
+    wx[5] = [1.6, 4.0, 5.0, 6.0]
+    am = prob.aqsmtemp.copy()
+    am[5] *= heavy
+    check(gpp, prob.replace(wtilde_array=w, wx_array=wx, aqsmtemp=am))
+    # some lanes of each warp only
+    w[:, ::3] += 3.0
+    check(gpp, prob.replace(wtilde_array=w, wx_array=wx, aqsmtemp=am))
+
+
+@pytest.mark.parametrize("light", [1.0, 1e-2, 1e-6])
+def test_light_band_at_the_pole(gpp, light):
+    """All bands far from the poles, where |u| is about 1/40, but one light one at |x - w| = 0.55."""
+    rng = np.random.Generator(np.random.PCG64(44))
+    prob = inputs.make_problem(32, 32, 96, 4, 2, seed=44)
+    wx = rng.uniform(40.0, 46.0, (32, 2))
+    wx[7] = 3.0
+    am = prob.aqsmtemp.copy()
+    am[7] *= light
+    check(gpp, prob.replace(wtilde_array=2.45 + 0.01j * rng.standard_normal((4, 96)), wx_array=wx,
+                            aqsmtemp=am), tol=2.0 ** -47)   # the partial fractions' x / |w|: 2^4.2
+
+
+@pytest.mark.parametrize("part", ["all", "heavy"])
+def test_terms_dropped_by_the_cutoff(gpp, part):
+    """Every term beyond the cutoff: asxtemp is exactly zero; or only one heavy band's."""
+    rng = np.random.Generator(np.random.PCG64(45))
+    prob = inputs.make_problem(12, 12, 96, 3, 2, seed=45)
+    wx = -rng.uniform(1.0, 2.0, (12, 2)) if part == "all" else rng.uniform(-8.0, -5.0, (12, 2))
+    wx[4] = -1.5
+    am = prob.aqsmtemp.copy()
+    am[4] *= 1.0 if part == "all" else 1e5
+    w = rng.uniform(1.2, 1.8, (3, 96)) + 0j
+    prob = prob.replace(wx_array=wx, aqsmtemp=am, wtilde_array=w)
+    if part == "all":
+        import torch
+        got = gpp.sigma(gpp.DeviceProblem.from_host(prob, device="cuda"), sexcut=0.05)
+        torch.cuda.synchronize()
+        assert np.all(got[1].cpu().numpy() == 0) and np.all(
+            np.asarray(oracle.sigma(prob, sexcut=0.05)[1]) == 0)
+    check(gpp, prob, sexcut=0.05 if part == "all" else 0.4)
+
+
+@pytest.mark.parametrize("nw", [2, 3, 7])
+@pytest.mark.parametrize("occ", ["all", "occupied"])
+def test_sums_that_cancel(gpp, nw, occ):
+    """Bands in pairs of opposite weights and almost equal frequencies: every sum is far below its
+    terms, which are strong all the same."""
+    prob = inputs.make_problem(20, 12, 100, 5, nw, seed=46)
+    am, an, wx = prob.aqsmtemp.copy(), prob.aqsntemp.copy(), prob.wx_array.copy()
+    am[1::2], an[1::2], wx[1::2] = -am[::2], an[::2], wx[::2] + 1e-7
+    prob = prob.replace(aqsmtemp=am, aqsntemp=an, wx_array=wx)
+    check(gpp, prob, occ=occ)
+    check(gpp, prob.replace(wx_array=wx - 5.0), occ=occ, sexcut=3.0)
