@@ -118,7 +118,8 @@ __device__ inline void fix_cotangents(int W, const double2* g_ach, const double2
   const double2 ca = make_double2(ach_scale * ga.x, -ach_scale * ga.y);
   const double2 csh = make_double2(-0.5 * gs.x, 0.5 * gs.y);
   const double2 cap = make_double2(ca.x - csh.x, ca.y - csh.y);
-  auto total = [](double2 c) { return warp_sum(sqrt(c.x * c.x + c.y * c.y)); };
+  // (not from the squares: those of cotangents below 1e-162 are zero)
+  auto total = [](double2 c) { return warp_sum(hypot(c.x, c.y)); };
   const double sa = total(ca), sc = total(cap), ss = total(csh);
   const double m = fmax(sc + ss, sa) * (1.0 + 0x1p-20);
   const bool ok = m == 0.0 || (m > 1e-90 && m < 1e90);   // false for NaN

@@ -133,3 +133,19 @@ def test_sums_that_cancel(gpp, nw, occ):
     prob = prob.replace(aqsmtemp=am, aqsntemp=an, wx_array=wx)
     check(gpp, prob, occ=occ)
     check(gpp, prob.replace(wx_array=wx - 5.0), occ=occ, sexcut=3.0)
+
+
+def test_small_cotangents(gpp):
+    """The gradients are linear in the cotangents, also where those squared are below FP64's range."""
+    import torch
+    prob = inputs.make_problem(12, 7, 70, 9, 3, seed=47)
+    ga, gs = inputs.cotangents(48, 3)
+    dp = gpp.DeviceProblem.from_host(prob, device="cuda")
+    ref = oracle.sigma_adjoint(prob, ga, gs, occ_mode=1)
+    for k in (-300, -500, -536, -544, -600, -900):
+        s = 2.0 ** k
+        got = gpp.sigma_backward(dp, torch.from_numpy(ga * s).cuda(), torch.from_numpy(gs * s).cuda(),
+                                 occ_mode="occupied")
+        for name, r in ref.items():
+            err = np.abs(got[name].cpu().numpy() / s - r).max()
+            assert err <= 2.0 ** -47 * np.abs(r).max(), (name, k, err)
