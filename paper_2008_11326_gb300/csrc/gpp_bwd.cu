@@ -84,12 +84,13 @@ struct alignas(16) FixC {
   int r1, i1, nr1, ni1;
   float r0, i0, r1f, i1f;
 };
-// The cotangent products of every frequency; ok: finite and of ordinary exponent. The sums of
-// the moduli of all of cap and csh, and of all of ca, are below 2^ec (1 - 2^-21); sum_a, sum_s: of cap
-// (or ca) and of csh alone, over 2^ec.
+// The cotangent products of every frequency; ok: finite and of ordinary exponent. The bands of
+// asxtemp (0: cap and csh) and the others (1: ca) have a scale each, since rows of the gradients
+// belong to one of them alone: the sums of the moduli, sum_c of cap or ca and sum_s of csh, over
+// 2^ec, add up to less than 1 - 2^-21.
 struct FixBwd {
-  int ok, ec;
-  float sum_a, sum_s;
+  int ok, ec[2];
+  float sum_c[2], sum_s;
   FixC cap[kMaxNw], csh[kMaxNw], ca[kMaxNw];
 };
 static_assert(sizeof(FixBwd) <= 1024, "workspace segment of the cotangent products");
@@ -121,19 +122,26 @@ __device__ inline void fix_cotangents(int W, const double2* g_ach, const double2
   // (not from the squares: those of cotangents below 1e-162 are zero)
   auto total = [](double2 c) { return warp_sum(hypot(c.x, c.y)); };
   const double sa = total(ca), sc = total(cap), ss = total(csh);
-  const double m = fmax(sc + ss, sa) * (1.0 + 0x1p-20);
-  const bool ok = m == 0.0 || (m > 1e-90 && m < 1e90);   // false for NaN
-  const int ec = m == 0.0 ? 0 : ((__double2hiint(m) >> 20) & 0x7ff) - 1022;
+  const double m[2] = {(sc + ss) * (1.0 + 0x1p-20), sa * (1.0 + 0x1p-20)};
+  bool ok = true;
+  int ec[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    ok = ok && (m[c] == 0.0 || (m[c] > 1e-90 && m[c] < 1e90));   // false for NaN
+    ec[c] = m[c] == 0.0 ? 0 : ((__double2hiint(m[c]) >> 20) & 0x7ff) - 1022;
+  }
   if (iw == 0) {
     out->ok = ok;
-    out->ec = ec;
-    out->sum_a = ok ? static_cast<float>(fmax(sc, sa) * exp2i(-ec)) : 0.0f;
-    out->sum_s = ok ? static_cast<float>(ss * exp2i(-ec)) : 0.0f;
+    out->ec[0] = ec[0];
+    out->ec[1] = ec[1];
+    out->sum_c[0] = ok ? static_cast<float>(sc * exp2i(-ec[0])) : 0.0f;
+    out->sum_c[1] = ok ? static_cast<float>(sa * exp2i(-ec[1])) : 0.0f;
+    out->sum_s = ok ? static_cast<float>(ss * exp2i(-ec[0])) : 0.0f;
   }
   if (ok && iw < W) {
-    out->cap[iw] = fix_c(cap, ec);
-    out->csh[iw] = fix_c(csh, ec);
-    out->ca[iw] = fix_c(ca, ec);
+    out->cap[iw] = fix_c(cap, ec[0]);
+    out->csh[iw] = fix_c(csh, ec[0]);
+    out->ca[iw] = fix_c(ca, ec[1]);
   }
 }
 
@@ -473,24 +481,34 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
     // cancels where x << |w|, so |w| may not exceed twice the largest frequency.
     bool use_fix = fix_on && __all_sync(0xffffffffu, !live || (fix_lane(w, wabs2, fix) &&
                                                                !gt_nonneg(wabs2, 4.0 * xmax2)));
-    int kn = 0, ka = 0, sh = 1;
+    // The bands of asxtemp and the others have scales of their own, packed: kn | ka << 9 | sh << 18.
+    int packs[2] = {0, 0};
     if (use_fix) {
-      unsigned mn = 0, ma = 0, mp = 0;
+      bool ok = true;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        unsigned mn = 0, ma = 0, mp = 0;
 #pragma unroll 8
-      for (int b = 0; b < B; ++b) {
-        const unsigned hn = fix_hi_max(load_an(b)), ha = fix_hi_max(load_am(b));
-        mn = max(mn, hn);
-        ma = max(ma, ha);
-        mp = max(mp, hn + ha);
+        for (int b = c == 0 ? 0 : nocc; b < (c == 0 ? nocc : B); ++b) {
+          const unsigned hn = fix_hi_max(load_an(b)), ha = fix_hi_max(load_am(b));
+          mn = max(mn, hn);
+          ma = max(ma, ha);
+          mp = max(mp, hn + ha);
+        }
+        int kn, ka, sh;
+        ok &= fix_weight_scale(mn, ma, mp, kn, ka, sh);
+        packs[c] = kn | ka << 9 | sh << 18;
       }
-      const bool ok = fix_weight_scale(mn, ma, mp, kn, ka, sh);
       use_fix = __all_sync(0xffffffffu, ok);
     }
     const FixPair wf = fix_pair(w, fix.E);
     float2 scA = make_float2(0.0f, 0.0f), scS = scA;   // the scales of u and of v
-    int ks = 0, down = 0, shG = 1, shH = 1;
-    double unitG = 1.0;   // GI in units of the FP64 form's (1) or of the integer sum's last bit
-    if (use_fix) {
+    int ks = 0, down = 0, shG = 1, shH = 1, nkhi = 0, akhi = 0, sh = 1;
+    double2 Iws = live ? Iw : make_double2(0.0, 0.0);   // times the unit of GI
+    // The scales of a class of bands; GI is in units of the integer sum's last bit.
+    auto unit_of = [&](int c) { return exp2i(fixc->ec[c] - 31 - ks) * (1.0 / kFixKappa); };
+    auto begin = [&](int c) {
+      if (!use_fix) return;
       float dA = 3.0e38f, dS2 = 3.0e38f;   // over the frequencies
 #pragma unroll
       for (int k = 0; k < W; ++k) {
@@ -501,34 +519,36 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
       }
       // u at its own scale, v at most as fine; the sums of the u terms are brought to v's scale
       const int ksA = fix_ks(dA * dA);
-      ks = nocc > 0 ? min(ksA, fix_ks(dS2)) : ksA;
+      ks = c == 0 ? min(ksA, fix_ks(dS2)) : ksA;
       down = ksA - ks;
       scA = fix_scale(ksA, fix.E);
       scS = fix_scale(ks, fix.E);
       // |GI| 2^(31 + ks - ec) and |H| 2^(2 ks - ec) stay below 2^(31 + shG), 2^(31 + shH)
-      const float cs = nocc > 0 ? fixc->sum_s : 0.0f;
-      const float bG = (fixc->sum_a / dA + cs * rsqrtf(dS2)) * 1.01f + 1e-30f;
-      const float bH = (fixc->sum_a / (dA * dA) + cs / dS2) * 1.01f + 1e-30f;
+      const float ca = fixc->sum_c[c], cs = c == 0 ? fixc->sum_s : 0.0f;
+      const float bG = (ca / dA + cs * rsqrtf(dS2)) * 1.01f + 1e-30f;
+      const float bH = (ca / (dA * dA) + cs / dS2) * 1.01f + 1e-30f;
       shG = min(max(ks + (__float_as_int(bG) >> 23) - 126, 1), 31);
       shH = min(max(2 * ks - 31 + (__float_as_int(bH) >> 23) - 126, 1), 31);
-      unitG = exp2i(fixc->ec - 31 - ks) * (1.0 / kFixKappa);
-    }
-    double2 Iws = live ? make_double2(Iw.x * unitG, Iw.y * unitG) : make_double2(0.0, 0.0);
-    asm volatile("" : "+d"(Iws.x), "+d"(Iws.y));
-    int nkhi = (kn + 32) << 20, akhi = (ka + 32) << 20;
-    // (keeps the compiler from forming these again in every band)
-    asm volatile("" : "+f"(scA.x), "+f"(scA.y), "+f"(scS.x), "+f"(scS.y), "+r"(shG), "+r"(shH),
-                      "+r"(down), "+r"(nkhi), "+r"(akhi), "+r"(sh));
+      const double unit = live ? unit_of(c) : 0.0;
+      Iws = make_double2(Iw.x * unit, Iw.y * unit);
+      nkhi = ((packs[c] & 511) + 32) << 20;
+      akhi = ((packs[c] >> 9 & 511) + 32) << 20;
+      sh = packs[c] >> 18;
+      // (keeps the compiler from forming these again in every band)
+      asm volatile("" : "+d"(Iws.x), "+d"(Iws.y), "+f"(scA.x), "+f"(scA.y), "+f"(scS.x), "+f"(scS.y),
+                        "+r"(shG), "+r"(shH), "+r"(down), "+r"(nkhi), "+r"(akhi), "+r"(sh));
+    };
     FixSum X, Y;
     X.clear();
     Y.clear();
     double2 an_next = load_an(0);
     // One band of a warp in the split-integer form; returns GI in units of unitG.
-    auto band_fix = [&](int b, double2 an, auto occ_tag) {
+    auto band_fix = [&](int b, int b0, int b1, double2 an, auto occ_tag) {
       constexpr bool OCC = decltype(occ_tag)::value;
-      if ((b & (kStageBands - 1)) == 0) {   // this warp's weights of the next bands
+      const int at = (b - b0) & (kStageBands - 1);
+      if (at == 0) {   // this warp's weights of the next bands
         __syncwarp();
-        for (int q = lane; q < kStageBands && b + q < B; q += 32) {
+        for (int q = lane; q < kStageBands && b + q < b1; q += 32) {
           const double2 a = load_am(b + q);
           FixAm e;
           fix_value(a.x, akhi, e.r1, e.r0);
@@ -537,7 +557,7 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
         }
         __syncwarp();
       }
-      const FixM m = fix_weight(stage[b & (kStageBands - 1)], an, nkhi, sh);
+      const FixM m = fix_weight(stage[at], an, nkhi, sh);
       const BandEntry* f = ft + static_cast<int64_t>(b) * W;
       long long g[2] = {0, 0}, h[2] = {0, 0};
       float g0[2] = {0.0f, 0.0f}, h0[2] = {0.0f, 0.0f};
@@ -624,7 +644,7 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
           const int b = c0 + bb;
           const double2 an = an_next, amv = load_am(b);
           if (b + 1 < B) an_next = load_an(b + 1);
-          const double2 GI = use_fix ? band_fix(b, an, occ_tag) : band_f64(b, an, amv, occ_tag);
+          const double2 GI = use_fix ? band_fix(b, b0, b1, an, occ_tag) : band_f64(b, an, amv, occ_tag);
           put(bb, amv, an, cmul(Iws, GI));
         }
         if (use_fix) {
@@ -639,17 +659,32 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
         reduce(c0, nb);
       }
     };
-    run(0, nocc, BoolTag<true>());
-    run(nocc, B, BoolTag<false>());
-    if (use_fix) {
+    // The sums of a class of bands, M GI and M H, in FP64; H's unit: u^2 = V 2^(31 - 2 ks) / kappa^2.
+    double2 rI = make_double2(0.0, 0.0), rH = rI;
+    auto end = [&](int c) {
+      if (!use_fix) return;
       const double2 x = X.take(), y = Y.take();
-      // back to M GI and M H; H's unit: u^2 = V 2^(31 - 2 ks) / kappa^2
-      const int em = sh - ka - kn;
-      const double fx = unitG * exp2i(shG + em);
-      const double fy = exp2i(fixc->ec - 2 * ks + shH) * (1.0 / kFixKappa) * (1.0 / kFixKappa) *
+      const int em = sh + 64 - (nkhi >> 20) - (akhi >> 20);
+      const double fx = unit_of(c) * exp2i(shG + em);
+      const double fy = exp2i(fixc->ec[c] - 2 * ks + shH) * (1.0 / kFixKappa) * (1.0 / kFixKappa) *
                         exp2i(em);
-      gI = make_double2(fx * (gI.x + x.x), fx * (gI.y + x.y));
-      gw = cmul(w, make_double2(fy * (gw.x + y.x), fy * (gw.y + y.y)));
+      rI = make_double2(fma(fx, gI.x + x.x, rI.x), fma(fx, gI.y + x.y, rI.y));
+      rH = make_double2(fma(fy, gw.x + y.x, rH.x), fma(fy, gw.y + y.y, rH.y));
+      gI = gw = make_double2(0.0, 0.0);
+    };
+    if (nocc > 0) {
+      begin(0);
+      run(0, nocc, BoolTag<true>());
+      end(0);
+    }
+    if (nocc < B) {
+      begin(1);
+      run(nocc, B, BoolTag<false>());
+      end(1);
+    }
+    if (use_fix) {
+      gI = rI;
+      gw = cmul(w, rH);
       gw = make_double2(gI.x + gw.x, gI.y + gw.y);   // M GW = M GI + w M H
     }
     gI = cmul(w, gI);

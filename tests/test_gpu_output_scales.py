@@ -4,7 +4,8 @@ removes, a light band that alone sets the scale of the reciprocals.
 
 Tolerance, derived before the first run: an output whose terms are 2^-6 of its scale carries at
 most 2^-50 of the root of the sum of its terms' squares, weaker ones are FP64's, and partial
-fractions, FP64 sums and the oracle add a few 2^-52 each: 2^-48 of that root.
+fractions, FP64 sums and the oracle add a few 2^-52 each: 2^-48 of that root. Entries of the gradients, single and of fewer terms: 2^-47, the
+adjoint's bound elsewhere.
 """
 
 import numpy as np
@@ -149,3 +150,66 @@ def test_small_cotangents(gpp):
         for name, r in ref.items():
             err = np.abs(got[name].cpu().numpy() / s - r).max()
             assert err <= 2.0 ** -47 * np.abs(r).max(), (name, k, err)
+
+
+def natural_gradients(prob, ga, gs, nocc):
+    """The root of the sum of the squares of what every gradient entry adds up (partial fractions)."""
+    B, (P, G) = prob.number_bands, prob.wtilde_array.shape
+    g = prob.indinv[prob.inv_igp_index]
+    am2 = (np.abs(prob.aqsmtemp[:, g]) * prob.vcoul[g]) ** 2        # [B][P]
+    an2 = np.abs(prob.aqsntemp) ** 2
+    w, I = prob.wtilde_array, prob.I_eps_array
+    occ = (np.arange(B) < nocc)[:, None, None]
+    q, h = np.zeros((B, P, G)), np.zeros((B, P, G))                # of GI and of GW, squared
+    for k in range(prob.nw):
+        x = prob.wx_array[:, k][:, None, None]
+        a2, s2 = np.abs(x - w) ** 2, np.abs(x + w) ** 2
+        c = np.where(occ, abs(ga[k].conj() + gs[k].conj() / 2), abs(ga[k])) ** 2 * (a2 > 0.25)
+        s = occ * abs(gs[k] / 2) ** 2
+        q += c / a2 + s / s2
+        h += x * x * (c / a2 ** 2 + s / s2 ** 2)
+    M2, Iw2 = am2[:, :, None] * an2[:, None, :], np.abs(I * w) ** 2
+    aqsm = np.zeros((B, G))
+    aqsm[:, g] = prob.vcoul[g] * np.sqrt(np.einsum("bg,pg,bpg->bp", an2, Iw2, q))
+    return dict(I_eps=np.abs(w) * np.sqrt((M2 * q).sum(0)), wtilde=np.abs(I) * np.sqrt((M2 * h).sum(0)),
+                aqsn=np.sqrt(np.einsum("bp,pg,bpg->bg", am2, Iw2, q)), aqsm=aqsm)
+
+
+def check_gradients(gpp, prob, ga, gs, occ="occupied"):
+    import torch
+    dp = gpp.DeviceProblem.from_host(prob, device="cuda")
+    got = gpp.sigma_backward(dp, torch.from_numpy(ga).cuda(), torch.from_numpy(gs).cuda(),
+                             occ_mode=occ)
+    torch.cuda.synchronize()
+    ref = oracle.sigma_adjoint(prob, ga, gs, occ_mode=0 if occ == "all" else 1)
+    size = natural_gradients(prob, ga, gs, prob.number_bands if occ == "all" else prob.nvband)
+    for k, r in ref.items():
+        err = np.abs(got[k].cpu().numpy() - r)
+        bad = err > 2.0 ** -47 * size[k]
+        assert not bad.any(), (k, bad.sum(), np.nanmax(err[bad] / size[k][bad]), prob.shape)
+
+
+def random_cotangents(nw, seed):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    z = rng.standard_normal((4, nw))
+    return z[0] + 1j * z[1], z[2] + 1j * z[3]
+
+
+@pytest.mark.parametrize("scale", [1e-2, 1e-4, 1e-8, 1e-12, 1e6])
+def test_gradients_occupied_weights_of_another_size(gpp, scale):
+    prob = inputs.make_problem(40, 7, 70, 9, 3, seed=49)
+    am = prob.aqsmtemp.copy()
+    am[:7] *= scale
+    prob = prob.replace(aqsmtemp=am)
+    ga, gs = random_cotangents(3, 50)
+    check_gradients(gpp, prob, ga, gs)
+    check_gradients(gpp, prob, 0 * ga, gs)
+
+
+@pytest.mark.parametrize("scale", [1e-2, 1e-4, 1e-8, 1e-20, 0.0])
+@pytest.mark.parametrize("nw", [1, 3])
+def test_gradients_cotangents_of_two_sizes(gpp, scale, nw):
+    prob = inputs.make_problem(40, 17, 70, 9, nw, seed=51)
+    ga, gs = random_cotangents(nw, 52)
+    check_gradients(gpp, prob, scale * ga, gs)
+    check_gradients(gpp, prob, ga, scale * gs)
