@@ -88,9 +88,12 @@ struct alignas(16) FixC {
 // asxtemp (0: cap and csh) and the others (1: ca) have a scale each, since rows of the gradients
 // belong to one of them alone: the sums of the moduli, sum_c of cap or ca and sum_s of csh, over
 // 2^ec, add up to less than 1 - 2^-21.
+// cap2, csh2, ca2: their squared moduli over 2^(2 ec), above zero for one that is not zero; spread:
+// branch 2 may leave a band with far smaller ones than the scale is for (csh never drops out).
 struct FixBwd {
-  int ok, ec[2];
+  int ok, ec[2], spread[2];
   float sum_c[2], sum_s;
+  float cap2[kMaxNw], csh2[kMaxNw], ca2[kMaxNw];
   FixC cap[kMaxNw], csh[kMaxNw], ca[kMaxNw];
 };
 static_assert(sizeof(FixBwd) <= 1024, "workspace segment of the cotangent products");
@@ -108,6 +111,11 @@ __device__ inline FixC fix_c(double2 c, int ec) {
   o.r1f = static_cast<float>(rr);
   o.i1f = static_cast<float>(ri);
   return o;
+}
+
+__device__ inline float fix_c2(double2 c, int ec) {
+  const float r = static_cast<float>(c.x * exp2i(-ec)), i = static_cast<float>(c.y * exp2i(-ec));
+  return c.x == 0.0 && c.y == 0.0 ? 0.0f : fmaxf(fmaf(r, r, i * i), 1e-37f);
 }
 
 // One warp, a lane per frequency: the split-integer form's cotangent products.
@@ -138,10 +146,30 @@ __device__ inline void fix_cotangents(int W, const double2* g_ach, const double2
     out->sum_c[1] = ok ? static_cast<float>(sa * exp2i(-ec[1])) : 0.0f;
     out->sum_s = ok ? static_cast<float>(ss * exp2i(-ec[0])) : 0.0f;
   }
+  // per frequency's share: the least squared modulus that is not zero against the sum of them all
+  auto spread_of = [&](double2 c, double2 s, int e) {
+    float least = fix_c2(c, e), all = 0.0f, never = fix_c2(s, e);
+    least = least == 0.0f ? 3.0e38f : least;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      least = fminf(least, __shfl_xor_sync(0xffffffffu, least, o));
+      never += __shfl_xor_sync(0xffffffffu, never, o);
+    }
+    all = warp_sumf(fix_c2(c, e)) + never;
+    return ok && never < all * 0x1p-8f && least < all * 0x1p-8f;
+  };
+  const bool spread0 = spread_of(cap, csh, ec[0]), spread1 = spread_of(ca, zero, ec[1]);
+  if (iw == 0) {
+    out->spread[0] = spread0;
+    out->spread[1] = spread1;
+  }
   if (ok && iw < W) {
     out->cap[iw] = fix_c(cap, ec[0]);
     out->csh[iw] = fix_c(csh, ec[0]);
     out->ca[iw] = fix_c(ca, ec[1]);
+    out->cap2[iw] = fix_c2(cap, ec[0]);
+    out->csh2[iw] = fix_c2(csh, ec[0]);
+    out->ca2[iw] = fix_c2(ca, ec[1]);
   }
 }
 
@@ -367,6 +395,143 @@ __device__ __noinline__ float fix_exact_sign(const BandEntry* f, double2 w) {
   return gt_nonneg(fma(a, a, w.y * w.y), kLimitTwo) ? 1.0f : -1.0f;
 }
 
+// The sums M GI and M GW of a pair by the fast form, for what the split-integer form is too coarse
+// for; not inlined, as above.
+template <int W>
+__device__ __noinline__ void fix_f64_sums(int B, int nocc, int64_t G, bool live, const double2* an,
+                                          const double2* am, const BwdBand* bt, double2 w,
+                                          double2* gI, double2* gw) {
+  double2 sI = make_double2(0.0, 0.0), sw = sI;
+#pragma unroll 1
+  for (int b = 0; b < B; ++b) {
+    const double2 a = live ? ldg2(an + static_cast<int64_t>(b) * G) : make_double2(0.0, 0.0);
+    const double2 M = cmul(live ? ldg2(am + b) : make_double2(0.0, 0.0), a);
+    double2 GI = make_double2(0.0, 0.0), GW = GI;
+    const BwdBand* e = bt + static_cast<int64_t>(b) * W;
+    if (b < nocc)
+      bwd_terms_fast<W, true>(e, w.x, w.y, w.y * w.y, GI, GW);
+    else
+      bwd_terms_fast<W, false>(e, w.x, w.y, w.y * w.y, GI, GW);
+    cmac(sI, M, GI);
+    cmac(sw, M, GW);
+  }
+  *gI = sI;
+  *gw = sw;
+}
+
+// Where the split-integer form is too coarse. Its errors are about 2^-56 of a scale: of a band's GI,
+// of the bound bG on it; of the pair's sums over n bands, of sqrt(n) times the largest weight times bG
+// (for GW = GI + w H, or times |w| and the bound on H). An entry whose own terms are far below that
+// (large cotangents or heavy bands in branch 2, x << |w|, where GI and w H cancel) is taken from FP64.
+// Q's: the whole warp, where a band's terms are below 2^-8 of bG in a lane (errors are 2^-48 of them
+// above). That takes cotangents of different sizes (FixBwd::spread), so only those are
+// looked through. The pair's two sums: where those of any lane are below 2^-9 (I_eps) and 2^-11
+// (wtilde), or of half of the lanes below 2^-7 and 2^-9. Ordinary inputs lie above but for
+// one warp in a hundred with few bands (4e5 drawn lanes of 2..128 bands: median 2^-3 .. 2^-6, least
+// 2^-8 and 2^-12, of half of a warp's 2^-5 and 2^-8). The terms' powers are formed (fix_weak_sums) only
+// where the sums themselves are not above these lines (of any lane, a quarter of them: a
+// lane's sum is below its terms by chance): 2 to 3 warps in a hundred. With the powers in the band loop
+// instead the adjoint took 5% longer, with the calls there 3%.
+constexpr int kWeakBand = 8, kWeakI = 9, kWeakW = 11, kWeakHalf = 2;
+
+// Votes on a warp's sums and their least ones, as logarithms in units of 2^-18 (fix_log_max).
+__device__ __forceinline__ bool fix_weak_vote(bool live, int I, int leastI, int W, int leastW,
+                                              int slack) {
+  const int one = 1 << 18;
+  const int m = live ? min(I - leastI + kWeakI * one, W - leastW + kWeakW * one) : one * 100;
+  const unsigned half = __ballot_sync(0xffffffffu, m < kWeakHalf * one);
+  return __any_sync(0xffffffffu, m < -slack * one) || 2 * __popc(half) > __popc(__ballot_sync(0xffffffffu, live));
+}
+
+// The least |x - w| of branch 1 and |x + w|^2 over the frequencies, less the FP32 rounding.
+template <int W>
+__device__ __forceinline__ void fix_distances_all(const FixPair& wf, const double* xrange, float& dA,
+                                                  float& dS2) {
+  dA = dS2 = 3.0e38f;
+#pragma unroll
+  for (int k = 0; k < W; ++k) {
+    const float lo = static_cast<float>(xrange[k]), hi = static_cast<float>(xrange[kMaxNw + k]);
+    dA = fminf(dA, fmaxf(0.5f, fmaxf(lo - wf.w1, wf.w1 - hi) * (1.0f - 0x1p-17f)));
+    const float sr = lo + wf.w1;
+    dS2 = fminf(dS2, fmaf(sr, sr, wf.i1 * wf.i1) * (1.0f - 0x1p-17f));
+  }
+}
+
+// Whether one of the bands is too weak in a lane of the warp: its terms' power below 2^-kWeakBand of
+// the bound on them.
+template <int W>
+__device__ __noinline__ bool fix_weak_bands(int B, int nocc, const BandEntry* ft, const FixBwd* fixc,
+                                            double2 w, const FixPair wf, const double* xrange,
+                                            bool live) {
+  const float wr = static_cast<float>(w.x), wi2 = static_cast<float>(w.y) * static_cast<float>(w.y);
+  float dA, dS2;
+  fix_distances_all<W>(wf, xrange, dA, dS2);
+  bool weak = false;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    if (fixc->spread[c] == 0) continue;
+    const float bG = fixc->sum_c[c] / dA + (c == 0 ? fixc->sum_s * rsqrtf(dS2) : 0.0f);
+    const float line = bG * exp2if(-kWeakBand);
+#pragma unroll 1
+    for (int b = c == 0 ? 0 : nocc; b < (c == 0 ? nocc : B); ++b) {
+      float g = 0.0f;
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        const float x = static_cast<float>(__ldg(&ft[static_cast<int64_t>(b) * W + k].lo.x));
+        const float a = x - wr, a2 = fmaf(a, a, wi2), s = x + wr, s2 = fmaf(s, s, wi2);
+        if (a2 > 0.25f * (1.0f + 0x1p-12f))   // clearly in branch 1
+          g = fmaf(c == 0 ? fixc->cap2[k] : fixc->ca2[k], fix_rcp(a2), g);
+        if (c == 0) g = fmaf(fixc->csh2[k], fix_rcp(s2), g);
+      }
+      weak |= g > 0.0f && g < line * line;
+    }
+  }
+  return __any_sync(0xffffffffu, weak && live);
+}
+
+// Whether a warp's sums are too weak for their scales (leastI, leastW), by the powers of their
+// terms: in FP32, M as in fix_strong.
+template <int W>
+__device__ __noinline__ bool fix_weak_sums(int B, int nocc, int64_t G, bool live, const double2* an_ptr,
+                                           const double2* am_ptr, const BandEntry* ft,
+                                           const FixBwd* fixc, double2 w, int leastI, int leastW) {
+  const float wr = static_cast<float>(w.x), wi = static_cast<float>(w.y), wi2 = wi * wi;
+  int I = kFixNone, Y = kFixNone;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int b0 = c == 0 ? 0 : nocc, b1 = c == 0 ? nocc : B;
+    FixScale sc;
+    fix_scales(b0, b1, G, an_ptr, am_ptr, live, sc);
+    const float m1 = exp2if(60 - sc.sh);
+    float pI = 0.0f, pW = 0.0f;
+#pragma unroll 4
+    for (int b = b0; b < b1; ++b) {
+      const double2 an = live ? ldg2(an_ptr + static_cast<int64_t>(b) * G) : make_double2(0.0, 0.0);
+      const double2 am = live ? ldg2(am_ptr + b) : make_double2(0.0, 0.0);
+      const float m2 = fmaxf(fix_square_of(an, sc.kn - 30) * fix_square_of(am, sc.ka - 30), 1e-37f) * m1 * m1;
+      float g = 0.0f, h = 0.0f;
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        const float x = static_cast<float>(__ldg(&ft[static_cast<int64_t>(b) * W + k].lo.x));
+        const float a = x - wr, a2 = fmaf(a, a, wi2), s = x + wr, s2 = fmaf(s, s, wi2);
+        const bool b1 = a2 > 0.25f * (1.0f + 0x1p-12f);   // clearly
+        const float ra = b1 ? fix_rcp(a2) : 0.0f, rs = fix_rcp(s2);
+        const float cu = (c == 0 ? fixc->cap2[k] : fixc->ca2[k]) * ra;
+        const float sv = c == 0 ? fixc->csh2[k] * rs : 0.0f;
+        g += cu + sv;
+        h = fmaf(x * x, fmaf(cu, ra, sv * rs), h);
+      }
+      pI = fmaf(m2, g, pI);
+      pW = fmaf(m2, h, pW);
+    }
+    const int unit = (sc.unit() + fixc->ec[c] + 1023) << 18;
+    if (pI > 0.0f) I = max(I, fix_half_log(pI) + unit);
+    if (pW > 0.0f) Y = max(Y, fix_half_log(pW) + unit);
+  }
+  const bool none = I == kFixNone;   // no terms: the sums are exactly zero
+  return fix_weak_vote(live, none ? leastI : I, leastI, none ? leastW : Y, leastW, 0);
+}
+
 // Bands between two reductions of a CTA (shared memory: 8 KB per band).
 constexpr int kRedBands = 4;
 constexpr int kTile = kTX * kTY;
@@ -481,7 +646,8 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
     // cancels where x << |w|, so |w| may not exceed twice the largest frequency.
     bool use_fix = fix_on && __all_sync(0xffffffffu, !live || (fix_lane(w, wabs2, fix) &&
                                                                !gt_nonneg(wabs2, 4.0 * xmax2)));
-    // The bands of asxtemp and the others have scales of their own, packed: kn | ka << 9 | sh << 18.
+    // The bands of asxtemp and the others have scales of their own, packed: kn | ka << 9 | sh << 18,
+    // and bit 24 where there are weights that are not zero.
     int packs[2] = {0, 0};
     if (use_fix) {
       bool ok = true;
@@ -497,26 +663,23 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
         }
         int kn, ka, sh;
         ok &= fix_weight_scale(mn, ma, mp, kn, ka, sh);
-        packs[c] = kn | ka << 9 | sh << 18;
+        packs[c] = kn | ka << 9 | sh << 18 | (mn != 0 && ma != 0 ? 1 << 24 : 0);
       }
       use_fix = __all_sync(0xffffffffu, ok);
     }
     const FixPair wf = fix_pair(w, fix.E);
+    if (use_fix && (fixc->spread[0] | fixc->spread[1]) != 0)
+      use_fix = !fix_weak_bands<W>(B, nocc, ft, fixc, w, wf, xrange, live);
     float2 scA = make_float2(0.0f, 0.0f), scS = scA;   // the scales of u and of v
     int ks = 0, down = 0, shG = 1, shH = 1, nkhi = 0, akhi = 0, sh = 1;
     double2 Iws = live ? Iw : make_double2(0.0, 0.0);   // times the unit of GI
+    int leastI = kFixNone, leastW = kFixNone;   // log2 of the scales of M GI and M GW
     // The scales of a class of bands; GI is in units of the integer sum's last bit.
     auto unit_of = [&](int c) { return exp2i(fixc->ec[c] - 31 - ks) * (1.0 / kFixKappa); };
     auto begin = [&](int c) {
       if (!use_fix) return;
-      float dA = 3.0e38f, dS2 = 3.0e38f;   // over the frequencies
-#pragma unroll
-      for (int k = 0; k < W; ++k) {
-        const float lo = static_cast<float>(xrange[k]), hi = static_cast<float>(xrange[kMaxNw + k]);
-        dA = fminf(dA, fmaxf(0.5f, fmaxf(lo - wf.w1, wf.w1 - hi) * (1.0f - 0x1p-17f)));
-        const float sr = lo + wf.w1;
-        dS2 = fminf(dS2, fmaf(sr, sr, wf.i1 * wf.i1) * (1.0f - 0x1p-17f));
-      }
+      float dA, dS2;
+      fix_distances_all<W>(wf, xrange, dA, dS2);
       // u at its own scale, v at most as fine; the sums of the u terms are brought to v's scale
       const int ksA = fix_ks(dA * dA);
       ks = c == 0 ? min(ksA, fix_ks(dS2)) : ksA;
@@ -533,7 +696,7 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
       Iws = make_double2(Iw.x * unit, Iw.y * unit);
       nkhi = ((packs[c] & 511) + 32) << 20;
       akhi = ((packs[c] >> 9 & 511) + 32) << 20;
-      sh = packs[c] >> 18;
+      sh = packs[c] >> 18 & 63;
       // (keeps the compiler from forming these again in every band)
       asm volatile("" : "+d"(Iws.x), "+d"(Iws.y), "+f"(scA.x), "+f"(scA.y), "+f"(scS.x), "+f"(scS.y),
                         "+r"(shG), "+r"(shH), "+r"(down), "+r"(nkhi), "+r"(akhi), "+r"(sh));
@@ -671,6 +834,13 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
       rI = make_double2(fma(fx, gI.x + x.x, rI.x), fma(fx, gI.y + x.y, rI.y));
       rH = make_double2(fma(fy, gw.x + y.x, rH.x), fma(fy, gw.y + y.y, rH.y));
       gI = gw = make_double2(0.0, 0.0);
+      if ((packs[c] >> 24) != 0) {
+        const int n = fix_half_log(static_cast<float>(c == 0 ? nocc : B - nocc)) + ((1023 + 62 + em) << 18);
+        const int lI = n + ((fixc->ec[c] - 31 - ks + shG) << 18);
+        const int lw = fix_log_max(w.x, w.y) - (1023 << 18);
+        leastI = max(leastI, lI);
+        leastW = max(leastW, max(lI, n + lw + ((fixc->ec[c] - 2 * ks + shH) << 18)));
+      }
     };
     if (nocc > 0) {
       begin(0);
@@ -686,6 +856,13 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
       gI = rI;
       gw = cmul(w, rH);
       gw = make_double2(gI.x + gw.x, gI.y + gw.y);   // M GW = M GI + w M H
+      if (fix_weak_vote(live, fix_log_max(gI.x, gI.y), leastI, fix_log_max(gw.x, gw.y), leastW, 2) &&
+          fix_weak_sums<W>(B, nocc, G, live, an_ptr, am_ptr, ft, fixc, w, leastI, leastW)) {   // rare
+        double2 sI, sw;
+        fix_f64_sums<W>(B, nocc, G, live, an_ptr, am_ptr, bt, w, &sI, &sw);
+        gI = sI;
+        gw = sw;
+      }
     }
     gI = cmul(w, gI);
     gw = cmul(I, gw);

@@ -582,6 +582,17 @@ __device__ __forceinline__ int fix_log_max(double re, double im) {
   return m == 0 ? kFixNone : static_cast<int>(m >> 2);
 }
 
+// |v|^2 2^(2 k) in FP32 from the leading 20 bits of each component (conversions of FP64 are as slow
+// as its arithmetic); below FP32's range 0.
+__device__ __forceinline__ float fix_square_of(double2 v, int k) {
+  auto part = [&](double c) {
+    const int h = (__double2hiint(c) & 0x7fffffff) - ((896 - k) << 20);
+    return __int_as_float(max(h, 0) << 3);
+  };
+  const float r = part(v.x), i = part(v.y);
+  return fmaf(r, r, i * i);
+}
+
 // The scales of one frequency's u and v, from the distance of its frequencies [lo, hi] from w and
 // -w, less the FP32 rounding. CUT: dcut is the least |S| of a kept term with x < 0; `delta` is
 // how far below the scale of most terms the kept ones near x = -w may lie.
@@ -632,14 +643,11 @@ __device__ __noinline__ bool fix_strong(int B, int64_t G, int nocc, const double
     fix_scales(b0, b1, G, an_ptr, am_ptr, live, s);
     unit[c] = s.unit();
     least[c] = fix_least(s.any, b1 - b0);
-    const double sn = exp2i(s.kn - 30), sa = exp2i(s.ka - 30);
     const float m1 = exp2if(60 - s.sh);   // of (am 2^(ka - 30)) (an 2^(kn - 30)) in M1's units
 #pragma unroll 2
     for (int b = b0; b < b1; ++b) {
       const double2 an = ldg2(an_ptr + static_cast<int64_t>(b) * G), am = ldg2(am_ptr + b);
-      const float nr = static_cast<float>(an.x * sn), ni = static_cast<float>(an.y * sn);
-      const float ar = static_cast<float>(am.x * sa), ai = static_cast<float>(am.y * sa);
-      const float m2 = fmaxf(fmaf(nr, nr, ni * ni) * fmaf(ar, ar, ai * ai), 1e-37f) * m1 * m1;
+      const float m2 = fmaxf(fix_square_of(an, s.kn - 30) * fix_square_of(am, s.ka - 30), 1e-37f) * m1 * m1;
 #pragma unroll
       for (int k = 0; k < W; ++k) {
         const float x = static_cast<float>(__ldg(&bt[static_cast<int64_t>(b) * W + k].lo.x));

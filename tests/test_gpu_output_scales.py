@@ -213,3 +213,74 @@ def test_gradients_cotangents_of_two_sizes(gpp, scale, nw):
     ga, gs = random_cotangents(nw, 52)
     check_gradients(gpp, prob, scale * ga, gs)
     check_gradients(gpp, prob, ga, scale * gs)
+
+
+def check_weak_gradients(gpp, prob, ga, gs, occ="all"):
+    """Where entries of a warp lie on both sides of the lines below which they are taken from FP64
+    (2^-8 of the scale for a band's rows; for the pairs' sums 2^-11 and 2^-13, and for half of a warp 2^-7
+    and 2^-9), errors of 2^-56 of the scale: a tensor's root mean square error within 2^-47 of
+    its terms', a single entry's within 2^-43 of its own, four times that at the most."""
+    import torch
+    dp = gpp.DeviceProblem.from_host(prob, device="cuda")
+    got = gpp.sigma_backward(dp, torch.from_numpy(ga).cuda(), torch.from_numpy(gs).cuda(),
+                             occ_mode=occ)
+    torch.cuda.synchronize()
+    ref = oracle.sigma_adjoint(prob, ga, gs, occ_mode=0 if occ == "all" else 1)
+    size = natural_gradients(prob, ga, gs, prob.number_bands if occ == "all" else prob.nvband)
+    for k, r in ref.items():
+        err = np.abs(got[k].cpu().numpy() - r)
+        assert np.all(err <= 2.0 ** -41 * size[k]), (k, np.max(err / np.maximum(size[k], 1e-300)))
+        some = size[k] > 0      # (rows of columns that no local column reaches are zero)
+        if some.any():
+            rel = np.sqrt(np.mean((err[some] / size[k][some]) ** 2))
+            assert rel <= 2.0 ** -47, (k, rel)
+
+
+@pytest.mark.parametrize("heavy", [1e1, 1e2, 1e4, 1e8, 1e12])
+@pytest.mark.parametrize("nw", [1, 2])
+def test_gradients_heavy_band_in_branch_2(gpp, heavy, nw):
+    rng = np.random.Generator(np.random.PCG64(53))
+    prob = inputs.make_problem(24, 24, 70, 9, nw, seed=53)
+    w = rng.uniform(1.5, 1.7, (9, 70)) + 1j * rng.uniform(-0.05, 0.05, (9, 70))
+    wx = prob.wx_array.copy()
+    wx[:, 0] = np.where(np.abs(wx[:, 0] - 1.6) < 0.7, 2.5, wx[:, 0])
+    wx[5] = 1.6
+    am = prob.aqsmtemp.copy()
+    am[5] *= heavy
+    prob = prob.replace(wtilde_array=w, wx_array=wx, aqsmtemp=am)
+    ga, gs = random_cotangents(nw, 54)
+    check_weak_gradients(gpp, prob, ga, 0 * gs)
+    check_weak_gradients(gpp, prob, ga, gs)
+
+
+@pytest.mark.parametrize("small", [1.0, 1e-1, 1e-2, 1e-4, 1e-8, 0.0])
+def test_gradients_of_small_frequencies(gpp, small):
+    """x << |w| in what counts: all bands but a light one; or the one frequency with a cotangent."""
+    rng = np.random.Generator(np.random.PCG64(55))
+    prob = inputs.make_problem(40, 40, 70, 9, 3, seed=55)
+    wx = small * rng.uniform(0.0, 1.0, (40, 3))
+    wx[5] = 8.0
+    am = prob.aqsmtemp.copy()
+    am[5] *= 1e-6 if small else 0.0
+    ga, gs = random_cotangents(3, 56)
+    check_weak_gradients(gpp, prob.replace(wx_array=wx, aqsmtemp=am), ga, gs)
+    wx = prob.wx_array.copy()
+    wx[:, 0] = small * rng.uniform(0.0, 1.0, 40)
+    one = np.array([1.0, 0.0, 0.0])
+    check_weak_gradients(gpp, prob.replace(wx_array=wx), ga * one, gs * one)
+
+
+@pytest.mark.parametrize("small", [0.3, 1e-2, 1e-4, 1e-8, 1e-22, 1e-60])
+@pytest.mark.parametrize("occ", ["all", "occupied"])
+def test_gradients_cotangents_of_different_frequencies(gpp, small, occ):
+    """Rows of bands whose large cotangent meets branch 2: only the small ones reach them."""
+    rng = np.random.Generator(np.random.PCG64(57))
+    prob = inputs.make_problem(30, 12, 70, 9, 3, seed=57)
+    w = rng.uniform(1.5, 1.7, (9, 70)) + 1j * rng.uniform(-0.05, 0.05, (9, 70))
+    wx = prob.wx_array.copy()
+    wx[::5, 0] = 1.6
+    ga, gs = random_cotangents(3, 58)
+    ga = ga * np.array([1.0, small, small])
+    check_weak_gradients(gpp, prob.replace(wtilde_array=w, wx_array=wx), ga, small * gs, occ)
+    check_weak_gradients(gpp, prob.replace(wtilde_array=w, wx_array=wx), ga, 0 * gs, occ)
+    check_weak_gradients(gpp, prob.replace(wx_array=wx), ga, gs, occ)
