@@ -133,8 +133,15 @@ int check_pointers(const gpp_problem& p, int precision, bool outputs = true) {
 // tile's overhead in FP32-bulk weighs more: 4 from 32 tiles per SM on, 8 from 64. us at 2 / 4 / 8,
 // nw = 3: P=300 G=8000 (31 tiles per SM at 4) B=7 181 / 167 / 173, B=40 477 / 464 / 503; P=500
 // G=9000 (58 at 4) 344 / 312 / 300 and 948 / 908 / 891; P=550 G=20000 (71 at 8) 736 / 671 / 635 and
-// 1968 / 1885 / 1861; nw = 4, B=7: P=500 455 / 417 / 415. Beyond the lines: P=250 G=4000 (13 at 4)
-// B=28 171 / 171 / 168; B=64 nw=3 P=333 G=7777 747 / 754 / 761; B=64 nw=1 P=500 859 / 1034 / 1139.
+// 1968 / 1885 / 1861; nw = 4: P=500 G=9000 B=7 482 / 441 / 443, B=20 849 / 801 / 812, B=40 1427 /
+// 1371 / 1408; P=550 G=20000 1099 / 1004 / 955, 1861 / 1759 / 1710, 3431 / 3332 / 3304. Beyond the lines:
+// P=250 G=4000 (13 at 4) B=28 171 / 171 / 168; B=64 nw=3 P=333 G=7777 747 / 754 / 761. With one or two
+// frequencies the lines would lie at fewer bands: P=500 G=9000 nw=1 B=7 271 / 260 / 268, B=20 393 / 412 /
+// 459, B=40 606 / 702 / 770; nw=2 300 / 278 / 275, 448 / 437 / 483, 702 / 708 / 798; they keep 2. Five to
+// eight would gain at 4 too (nw=5 578 / 521 / 527, 984 / 927 / 961, 1647 / 1597 / 1688; nw=8 943 / 864 /
+// 872, 1831 / 1736 / 1844, 3146 / 3088 / 3396), but not all at 8 (nw=8 P=550 G=20000 B=40 8097 / 8069 /
+// 8771): not taken so far. A batch follows its instance of most bands: ten of 12 bands 709 / 670 / 652,
+// with one of 41 among them 789 / 751 / 736, at 2.
 int default_igpt(int precision, double columns, int64_t bands, int64_t nw, int sms) {
   if (precision == GPP_FP32_BULK) {
     if (bands <= 40 && (nw == 3 || nw == 4) && columns >= 4.0 * 32 * sms)

@@ -89,16 +89,6 @@ __device__ __noinline__ void f32_general_pair(int B, int64_t G, int nocc,
   }
 }
 
-// Tile partials: FP64 sums (double) for GPP_FP64; compensated FP32 pairs (float2, hi + lo)
-// for GPP_FP32_BULK, so that its main kernel needs no FP64 arithmetic outside the rare
-// exact-decision and near-pole branches and the once-per-pair I w. Both are 8 bytes per
-// value. The FP32-bulk instantiation is held to 72 registers per thread: with its shared
-// memory (the compensated pairs) that is 7 CTAs of 128 threads per SM either way, and on
-// GB300 (nw = 3, benchmark instance) its main kernel ran 111.2 ms at 64 registers (spilled
-// values reloaded in the band loop), 104.5 ms at 72 and 105.9 ms at 80.
-#ifndef GPP_F32_MAXNREG
-#define GPP_F32_MAXNREG 72
-#endif
 // One (igp, ig) pair of the FP64 sum in FP64 arithmetic, by the fast or the general form, for
 // the warps outside the split-integer form's range. Not inlined, so that its registers do
 // not count against the split-integer band loop.
@@ -205,6 +195,17 @@ __device__ __forceinline__ void f64_body(const BatchInst* __restrict__ inst, int
     block_partials<4 * W>(acc, red, partials + t * 4 * W);
   }
 }
+
+// Tile partials: FP64 sums (double) for GPP_FP64; compensated FP32 pairs (float2, hi + lo)
+// for GPP_FP32_BULK, so that its main kernel needs no FP64 arithmetic outside the rare
+// exact-decision and near-pole branches and the once-per-pair I w. Both are 8 bytes per
+// value. The FP32-bulk instantiation is held to 72 registers per thread: with its shared
+// memory (the compensated pairs) that is 7 CTAs of 128 threads per SM either way, and on
+// GB300 (nw = 3, benchmark instance) its main kernel ran 111.2 ms at 64 registers (spilled
+// values reloaded in the band loop), 104.5 ms at 72 and 105.9 ms at 80.
+#ifndef GPP_F32_MAXNREG
+#define GPP_F32_MAXNREG 72
+#endif
 
 template <int W>
 __device__ __forceinline__ void f32_body(const BatchInst* __restrict__ inst, int ninst,
@@ -331,14 +332,17 @@ __device__ __forceinline__ void f32_body(const BatchInst* __restrict__ inst, int
 }
 
 // The two instantiations of the main kernel. FP64: two 256-thread CTAs' worth of registers per
-// SM (128 per thread), which the split-integer band loop fits without spilling; the FP64 band
-// loop runs as fast at 128 registers as at its unconstrained 166. FP32-bulk: held to
+// SM (128 per thread), which the split-integer band loop all but fits (a few values that it
+// reads once per band are spilled); the FP64 band loop runs as fast at 128 registers as at its
+// unconstrained 166. FP32-bulk: held to
 // GPP_F32_MAXNREG registers (80 for nw > 5, whose band loop would spill at fewer).
 //
 // Measured (GB300, main sum with the split-integer form against the FP64 form alone):
-// B = 512, P = 819, G = 16384, nw = 3: 162.7 against 692.6 ms; B = 128, P = 410, G = 8192:
-// 10.5 against 44.4 ms; B = 32, P = 64, G = 512: 0.053 against 0.30 ms (with shallower tiles
-// and the cheaper reduction). Bound now: the instruction issue of the integer and FP32 pipes.
+// B = 512, P = 819, G = 16384, nw = 3: 166.0 against 692.6 ms; B = 128, P = 410, G = 8192:
+// 10.7 against 44.4 ms; B = 32, P = 64, G = 512: 0.055 against 0.30 ms (with shallower tiles
+// and the cheaper reduction). Of these, what keeps every output at its own scale (gpp_terms_fix.cuh:
+// the scales of two classes of bands, the test of the sums) is 162.3 -> 166.0, 10.52 -> 10.69 ms. Bound
+// now: the instruction issue of the integer and FP32 pipes.
 template <int W>
 __global__ void __launch_bounds__(256, 2)
     gpp_batched_kernel_f64(const BatchInst* __restrict__ inst, int ninst, int64_t t_begin,

@@ -34,7 +34,8 @@
 // Q and its two weighted sums stay FP64 (21 FP64 instructions per unit, which run beside the
 // integer work; the FP64 form has 141). Bound: dispatch of the integer and FP32 instructions
 // (ALU 315, FMA pipe 665 per unit and 32 lanes), with the FP64 pipe 56% busy and its latency on
-// top. B = 128, P = 410, G = 8192, nw = 3: 25.6 ms (FP64 form 108.3).
+// top. B = 128, P = 410, G = 8192, nw = 3: 26.0 ms (FP64 form 108.3; 25.6 without the tests that
+// send entries far below their scale to FP64, see kWeakBand).
 
 #include <cuda_runtime.h>
 
@@ -338,7 +339,7 @@ __device__ __forceinline__ long long fix_down(long long s, int d) {
 
 // A 62-bit sum (with its small FP32 part, moved in in units of 2^4) as 2^sh (U + gamma).
 __device__ __forceinline__ FixU fix_limbs(const long long (&s)[2], int sh) {
-  const long long half = 1LL << (sh - 1);
+  const unsigned half = 1u << (sh - 1);
   FixU v;
   v.Ur = static_cast<int>((s[0] + half) >> sh);
   v.Ui = static_cast<int>((s[1] + half) >> sh);

@@ -24,11 +24,11 @@ constexpr double kFastWabs2Hi = 62499.0;
 
 constexpr int kMaxNw = 8;
 
-// One (band, iw) entry of the FP64 band table: x = wx_array[b][iw], x^2, and x split into
+// One (band, iw) entry of the FP64 band table: x = wx_array[b][iw], and x split into
 // integers and floats for the split-integer form (fix_x in gpp_terms_fix.cuh; zeros when the
 // instance's frequencies are outside its range).
 struct alignas(32) BandEntry {
-  double2 lo;  // x, x^2
+  double2 lo;  // x, and padding to 32 bytes
   int4 fx;
 };
 
@@ -55,7 +55,8 @@ __host__ __device__ constexpr int f32_band_quads(int W) { return 2 * f32_half_qu
 // Flags written by the gather kernel: [0] some wx < 0 or NaN, [1] bad index count,
 // [2] some |wx| >= kFp32MaxX or NaN (the FP32 decision margin assumes smaller x); from int
 // kFlagXmax on, the bits of max |wx| as a 64-bit integer (kFlagBytes so far, cleared before
-// the gather); then, written whole by the gather, a FixInfo at int kFlagFix and, as doubles
+// the gather where it only raises them: with the index checks on, or beyond kScanBands bands);
+// then, written whole by the gather, a FixInfo at int kFlagFix and, as doubles
 // from int kFlagRange on, min wx of every frequency and max wx of every frequency (kMaxNw
 // each). kFlagAllBytes in all.
 constexpr double kFp32MaxX = 1.0e4;

@@ -159,7 +159,7 @@ __device__ __forceinline__ void prep_block(const PrepArgs& a, int block, int nbl
   if (i0 == 0) *reinterpret_cast<FixInfo*>(a.flags + kFlagFix) = fix;
   for (int64_t i = i0; i < n; i += static_cast<int64_t>(a.table_blocks) * 256) {
     const double x = a.wx[i];
-    a.bt[i] = BandEntry{make_double2(x, x * x), fix.ok ? fix_x(x, fix.E) : make_int4(0, 0, 0, 0)};
+    a.bt[i] = BandEntry{make_double2(x, 0.0), fix.ok ? fix_x(x, fix.E) : make_int4(0, 0, 0, 0)};
     if (!a.scan) {
       if (!(x >= 0.0)) a.flags[0] = 1;
       if (!(fabs(x) < kFp32MaxX)) a.flags[2] = 1;

@@ -271,7 +271,7 @@ __device__ __forceinline__ FixM fix_weight(const FixAm& a, double2 an, int nkhi,
   const int qi = static_cast<int>(mad_wide(a.r1, ni0, mad_wide(a.i1, nr0, mad_wide(a.r0, ni1, mad_wide(a.i0, nr1, h)))) >> 32);
   const long long Pr = mad_wide(a.r1, nr1, mad_wide(-a.i1, ni1, qr));
   const long long Pi = mad_wide(a.r1, ni1, mad_wide(a.i1, nr1, qi));
-  const long long half = 1LL << (sh - 1);
+  const unsigned half = 1u << (sh - 1);   // (sh <= 30: one word)
   FixM m;
   m.r1 = static_cast<int>((Pr + half) >> sh);
   m.i1 = static_cast<int>((Pi + half) >> sh);
@@ -335,6 +335,9 @@ __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixC
                                           const float2* sc) {
   const int nt = blockDim.x, lane = threadIdx.x & 31;
   const int64_t G = ctx.G;
+  int nkhi = ctx.nkhi, sh = ctx.sh;
+  // (keeps the compiler from forming these again in every band: 1%)
+  asm volatile("" : "+r"(nkhi), "+r"(sh));
   FixAm* const stage = ctx.stage;
   // bands of the modular sums: the FP32 sum beside them has to be good to 2^62 (terms below
   // 2^62, with the cutoff's scale 2^69)
@@ -370,7 +373,7 @@ __device__ __forceinline__ void fix_range(int b0, int b1, bool fresh, const FixC
         for (int b = l0; b < l1; ++b) {
           const double2 an = an_next;
           if (b + 1 < b1) an_next = ldg2(ctx.an + static_cast<int64_t>(b + 1) * G);
-          const FixM m = fix_weight(stage[b - s0], an, ctx.nkhi, ctx.sh);
+          const FixM m = fix_weight(stage[b - s0], an, nkhi, sh);
           const BandEntry* btb = ctx.bt + static_cast<int64_t>(b) * ctx.W + iw0;
           int4 xv[WG];
           FixN na[WG];

@@ -284,3 +284,14 @@ def test_gradients_cotangents_of_different_frequencies(gpp, small, occ):
     check_weak_gradients(gpp, prob.replace(wtilde_array=w, wx_array=wx), ga, small * gs, occ)
     check_weak_gradients(gpp, prob.replace(wtilde_array=w, wx_array=wx), ga, 0 * gs, occ)
     check_weak_gradients(gpp, prob.replace(wx_array=wx), ga, gs, occ)
+
+
+# bands around the FP32 low sums' eight (forward) and the reductions' four (adjoint)
+@pytest.mark.parametrize("B", [3, 4, 5, 7, 8, 9])
+@pytest.mark.parametrize("nw", [1, 3, 4])
+def test_few_bands(gpp, B, nw):
+    prob = inputs.make_problem(B, (B + 1) // 2, 65, 9, nw, seed=59)
+    ga, gs = random_cotangents(nw, 60)
+    for occ in ("all", "occupied"):
+        check(gpp, prob, occ=occ)
+        check_weak_gradients(gpp, prob, ga, gs, occ)
