@@ -835,7 +835,8 @@ __global__ void __launch_bounds__(kTile, 2) gpp_bwd_kernel(
       rI = make_double2(fma(fx, gI.x + x.x, rI.x), fma(fx, gI.y + x.y, rI.y));
       rH = make_double2(fma(fy, gw.x + y.x, rH.x), fma(fy, gw.y + y.y, rH.y));
       gI = gw = make_double2(0.0, 0.0);
-      if ((packs[c] >> 24) != 0) {
+      // (not of a class without weights or cotangents: its sums are zero, its scale is nothing's)
+      if ((packs[c] >> 24) != 0 && fixc->sum_c[c] + (c == 0 ? fixc->sum_s : 0.0f) > 0.0f) {
         const int n = fix_half_log(static_cast<float>(c == 0 ? nocc : B - nocc)) + ((1023 + 62 + em) << 18);
         const int lI = n + ((fixc->ec[c] - 31 - ks + shG) << 18);
         const int lw = fix_log_max(w.x, w.y) - (1023 << 18);
