@@ -532,6 +532,8 @@ __device__ __forceinline__ bool fix_weight_scale(unsigned mn, unsigned ma, unsig
   return n_ok && a_ok && (mn == 0 || ma == 0 || top >= kFixMinTop);
 }
 
+constexpr int kFixNoWeight = 401;   // beyond fix_exponent's
+
 // The scales of one class of bands [b0, b1) for a pair, from the magnitudes of the column of
 // aqsntemp, of the row of weights and of their products: am 2^ka and an 2^kn as integers, their
 // product shifted by sh. `any`: it has weights that are not zero (an inert lane has none).
@@ -553,7 +555,12 @@ __device__ __forceinline__ bool fix_scales(int b0, int b1, int64_t G, const doub
   }
   if (!live) mn = mp = 0;   // whatever its column holds: the values stay finite and I is zero
   s.any = mn != 0 && ma != 0;
-  return fix_weight_scale(mn, ma, mp, s.kn, s.ka, s.sh);
+  const bool ok = fix_weight_scale(mn, ma, mp, s.kn, s.ka, s.sh);
+  // without weights a unit far below any other, which tells them apart (ka stays the warp's: its
+  // lanes share the staged weights)
+  if (mn == 0) s.kn = kFixNoWeight;
+  if (ma == 0) s.ka = kFixNoWeight;
+  return ok;
 }
 
 // Whether an output is too weak for the scale that its sums were rounded at. A sum of n terms M u
@@ -694,17 +701,24 @@ __device__ __noinline__ bool fix_strong(int B, int64_t G, int nocc, const double
 // pair, as fix_range left them in st, against half the least root of each class of its terms (a warp
 // with a single pair, past the last whole 32 G-vectors, would be doubted half of the time at all of
 // it). Passed by a lane whose scale, times |I w|, is within 2^1.5 of the largest in the warp: no single
-// lane decides, whose sum may be small by chance. (A pair without weights in a class may be doubted
-// for nothing.)
+// lane decides, whose sum may be small by chance.
 template <int N>
 __device__ __noinline__ bool fix_doubt(const double* st, const float2* sc, int nt, int nocc, int B,
-                                       int exo, int exr, double Iwr, double Iwi) {
+                                       const FixCtx o, const FixCtx r, double Iwr, double Iwi) {
   const int lgI = static_cast<int>(fix_hi_max(make_double2(Iwr, Iwi)) >> 2), one = 1 << 18;
-  const int no = fix_least(true, nocc) + exo * one, nr = fix_least(true, B - nocc) + exr * one;
+  auto unit_of = [](const FixCtx& c) { return c.sh + 64 - (c.nkhi >> 20) - (c.akhi >> 20); };
+  auto least_of = [&](const FixCtx& c, int n) {
+    const int none = (kFixNoWeight + 32) << 20;
+    const int l = fix_least(c.nkhi != none && c.akhi != none, n);
+    return l == kFixNone ? l : l + unit_of(c) * one;
+  };
+  const int exo = unit_of(o), exr = unit_of(r);
+  const int no = least_of(o, nocc), nr = least_of(r, B - nocc);
   bool doubt = false;
   auto test = [&](double re, double im, int unit, int least) {
     const int m = fix_log_max(re, im);
-    const int strong = m != kFixNone && m + unit * one >= least - one ? lgI + least : kFixNone;
+    const bool ok = least == kFixNone || (m != kFixNone && m + unit * one >= least - one);
+    const int strong = ok ? lgI + least : 2 * kFixNone;
     doubt |= __reduce_max_sync(0xffffffffu, strong) <
              __reduce_max_sync(0xffffffffu, lgI + least) - 3 * one / 2;
   };
@@ -712,9 +726,10 @@ __device__ __noinline__ bool fix_doubt(const double* st, const float2* sc, int n
   for (int k = 0; k < N; ++k) {
     auto ks = [&](int q) { return (__float_as_int(sc[q * nt].x) >> 23) - 127; };
     const int ku = ks(2 * k), kv = ks(2 * k + 1);
-    test(st[4 * k * nt], st[(4 * k + 1) * nt], (nocc < B ? exr : exo) - ku, max(no, nr) - ku * one);
+    auto least = [&](int l, int ks) { return l == kFixNone ? l : l - ks * one; };
+    test(st[4 * k * nt], st[(4 * k + 1) * nt], (nocc < B ? exr : exo) - ku, least(max(no, nr), ku));
     if (nocc > 0)
-      test(st[(4 * k + 2) * nt], st[(4 * k + 3) * nt], exo - ku, no - min(ku, kv) * one);
+      test(st[(4 * k + 2) * nt], st[(4 * k + 3) * nt], exo - ku, least(no, min(ku, kv)));
   }
   return doubt;
 }
@@ -787,7 +802,7 @@ __device__ __noinline__ FixResult fix_band_loop(int B, int64_t G, int nocc,
       }
     }
     if (nocc < B) fix_range<N, false, false>(nocc, B, nocc == 0, ctx_r, iw0, w, cut, st, sc);
-    doubt |= fix_doubt<N>(st, sc, nt, nocc, B, exo, exr, Iwr, Iwi);
+    doubt |= fix_doubt<N>(st, sc, nt, nocc, B, ctx, ctx_r, Iwr, Iwi);
     const bool aside = W <= kFixMaxGroup && doubt;
 #pragma unroll
     for (int k = 0; k < N; ++k) {   // tacc += I w times the pair's sums (units: I w / (2 kappa))

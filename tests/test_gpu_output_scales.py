@@ -295,3 +295,20 @@ def test_few_bands(gpp, B, nw):
     for occ in ("all", "occupied"):
         check(gpp, prob, occ=occ)
         check_weak_gradients(gpp, prob, ga, gs, occ)
+
+
+@pytest.mark.parametrize("nw", [2, 5])
+@pytest.mark.parametrize("zero", ["occupied", "rest", "columns"])
+def test_bands_without_weights(gpp, zero, nw):
+    """A class of bands whose weights are all zero (padding), and G-vectors without any."""
+    prob = inputs.make_problem(40, 9, 100, 5, nw, seed=61)
+    am, an = prob.aqsmtemp.copy(), prob.aqsntemp.copy()
+    if zero == "columns":
+        an[:, 40:70] = 0.0
+    else:
+        am[slice(0, 9) if zero == "occupied" else slice(9, 40)] = 0.0
+    prob = prob.replace(aqsmtemp=am, aqsntemp=an)
+    ga, gs = random_cotangents(nw, 62)
+    check(gpp, prob, occ="occupied")
+    check(gpp, prob.replace(wx_array=prob.wx_array - 5.0), occ="occupied", sexcut=3.0)
+    check_weak_gradients(gpp, prob, ga, gs, "occupied")
