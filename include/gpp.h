@@ -65,7 +65,8 @@ typedef enum gpp_status {
 
 typedef enum gpp_precision {
     GPP_FP64 = 0,      /* to FP64's accuracy: terms as integers with FP32 remainders, summed in
-                          64-bit integers, where the inputs' range allows it, else in FP64 */
+                          64-bit integers, where the inputs' range and the size of every output's
+                          own terms allow it, else in FP64 */
     GPP_FP32_BULK = 1  /* FP32 complex arithmetic (complex64 aqsntemp copy), FP64 branch
                           decisions near the threshold, FP64 near the wdiff pole, compensated
                           FP32 accumulation folded into FP64 reductions */
