@@ -157,7 +157,8 @@ __device__ inline void fix_cotangents(int W, const double2* g_ach, const double2
       never += __shfl_xor_sync(0xffffffffu, never, o);
     }
     all = warp_sumf(fix_c2(c, e)) + never;
-    return ok && never < all * 0x1p-8f && least < all * 0x1p-8f;
+    // (a small csh is what is left where branch 2 takes every cap; no csh leaves nothing)
+    return ok && never < all * 0x1p-8f && (never > 0.0f || least < all * 0x1p-8f);
   };
   const bool spread0 = spread_of(cap, csh, ec[0]), spread1 = spread_of(ca, zero, ec[1]);
   if (iw == 0) {

@@ -312,3 +312,18 @@ def test_bands_without_weights(gpp, zero, nw):
     check(gpp, prob, occ="occupied")
     check(gpp, prob.replace(wx_array=prob.wx_array - 5.0), occ="occupied", sexcut=3.0)
     check_weak_gradients(gpp, prob, ga, gs, "occupied")
+
+
+@pytest.mark.parametrize("small", [0.3, 1e-2, 1e-4, 1e-8, 1e-22])
+@pytest.mark.parametrize("nw", [1, 3])
+def test_gradients_of_bands_all_in_branch_2(gpp, small, nw):
+    """Bands whose every frequency is in branch 2 for every pole: asxtemp's cotangent alone, a small
+    one, reaches their rows."""
+    rng = np.random.Generator(np.random.PCG64(63))
+    prob = inputs.make_problem(30, 12, 70, 1, nw, seed=63)
+    w = rng.uniform(1.5, 1.7, (1, 70)) + 1j * rng.uniform(-0.05, 0.05, (1, 70))
+    wx = prob.wx_array.copy()
+    wx[::5] = 1.6
+    ga, gs = random_cotangents(nw, 64)
+    for occ in ("all", "occupied"):
+        check_weak_gradients(gpp, prob.replace(wtilde_array=w, wx_array=wx), ga, small * gs, occ)
